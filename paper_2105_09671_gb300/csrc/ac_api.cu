@@ -397,7 +397,60 @@ bool ac_plan_depths(int64_t n, int k, std::vector<int> &depths) {
   return false;
 }
 
+// Whether a schedule runs on the register-tile kernel (block2d.cuh): the
+// default 2D schedule of FP32 / FP16 storage, unless the caller forced a
+// schedule or a strip width (those run the streaming kernel as asked).  Its
+// results are bit for bit those of the default schedule's passes: FP32 does
+// not depend on the depth, and FP16 storage is rounded where they end.
+static bool takes_block2d(const ac_ctx *c, int variant, int k, int tile) {
+  if (c->d.ndim != 2 || c->d.dtype == AC_F64 || c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO)
+    return false;
+  int dv, dk;
+  default_schedule(c, &dv, &dk);
+  return variant == dv && k == dk && tile == default_tile(c, dk);
+}
+
+// n steps on the register-tile kernel; *done is false if it does not serve
+// the grid (nothing was launched).
+static int issue_block2d(ac_ctx *c, int64_t n, int k, bool *done) {
+  // FP16 storage: the passes whose ends round the field; FP32: single steps
+  std::vector<int> passes;
+  if (c->d.dtype == AC_F16S) ac_plan_depths(n, k, passes);
+  const int64_t np = c->d.dtype == AC_F16S ? (int64_t)passes.size() : n;
+  Block2DPlan plan;
+  *done = block2d_plan(c->d.dtype, c->d.nx, c->d.ny, np, c->d.dtype == AC_F16S ? k : 1, c->num_sms, &plan);
+  if (!*done) return AC_OK;
+  void *src = c->phi, *dst = c->ws;
+  for (int64_t i = 0; i < plan.launches; ++i) {
+    const int64_t p0 = np * i / plan.launches, p1 = np * (i + 1) / plan.launches;
+    int steps = (int)(p1 - p0);
+    uint32_t mask = 0;
+    if (!passes.empty()) {
+      steps = 0;
+      for (int64_t p = p0; p < p1; ++p) {
+        steps += passes[p];
+        if (p + 1 < p1) mask |= 1u << (steps - 1);  // (the store rounds after the last)
+      }
+    }
+    cudaError_t e = launch_block2d(c->d.dtype, plan, c->gp, src, dst, steps, mask, c->stream);
+    if (e != cudaSuccess) return fail(AC_ERR_CUDA, "stencil launch failed: %s", cudaGetErrorString(e));
+    ++c->launches;
+    std::swap(src, dst);
+  }
+  if (plan.launches % 2) {
+    const size_t es = ac_elem_size(c->d.dtype);
+    AC_CUDA(cudaMemcpy2DAsync(c->phi, c->d.pitch_x * es, c->ws, c->d.pitch_x * es, c->d.nx * es,
+                              (size_t)c->d.ny, cudaMemcpyDeviceToDevice, c->stream));
+  }
+  return AC_OK;
+}
+
 static int issue_steps(ac_ctx *c, int64_t n, int variant, int k, int tile) {
+  if (takes_block2d(c, variant, k, tile)) {
+    bool done = false;
+    const int rc = issue_block2d(c, n, k, &done);
+    if (rc || done) return rc;
+  }
   std::vector<int> depths;
   const bool even = variant == AC_VARIANT_DIRECT ? (n % 2 == 0) : ac_plan_depths(n, k, depths);
   if (variant == AC_VARIANT_DIRECT) depths.assign((size_t)n, 1);
@@ -439,7 +492,7 @@ extern "C" int ac_step(ac_ctx *c, int64_t n) {
   if (!c->use_graph || c->stream == nullptr) return issue_steps(c, n, variant, k, tile);
   // graph replay: capture the launch sequence for this (n, schedule) once
   if (c->graph_exec == nullptr || c->graph_n != n || c->graph_variant != variant ||
-      c->graph_k != k || c->graph_tile != tile) {
+      c->graph_k != k || c->graph_tile != tile || c->graph_block != takes_block2d(c, variant, k, tile)) {
     release_graph(c);
     AC_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed));
     const int64_t before = c->launches;
@@ -457,6 +510,7 @@ extern "C" int ac_step(ac_ctx *c, int64_t n) {
     c->graph_variant = variant;
     c->graph_k = k;
     c->graph_tile = tile;
+    c->graph_block = takes_block2d(c, variant, k, tile);
   }
   AC_CUDA(cudaGraphLaunch(c->graph_exec, c->stream));
   c->launches += c->graph_launches;

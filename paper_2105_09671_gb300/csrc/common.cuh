@@ -70,6 +70,34 @@ __device__ __forceinline__ uint4 pack16<__half>(const float *in) {
   return w;
 }
 
+// V storage elements (one 16-byte word, or 8 bytes of FP16 storage) at an
+// address aligned to their size <-> V compute values.
+template <typename T, int V>
+__device__ __forceinline__ void ld_cells(const T *p, typename Traits<T>::C *out) {
+  if constexpr (sizeof(T) * V == 16) {
+    unpack16<T>(*reinterpret_cast<const uint4 *>(p), out);
+  } else {
+    static_assert(sizeof(T) == 2 && V == 4, "8-byte vectors are FP16 storage");
+    const uint2 w = *reinterpret_cast<const uint2 *>(p);
+    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&w.x));
+    const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&w.y));
+    out[0] = a.x; out[1] = a.y; out[2] = b.x; out[3] = b.y;
+  }
+}
+template <typename T, int V>
+__device__ __forceinline__ void st_cells(T *p, const typename Traits<T>::C *in) {
+  if constexpr (sizeof(T) * V == 16) {
+    *reinterpret_cast<uint4 *>(p) = pack16<T>(in);
+  } else {
+    static_assert(sizeof(T) == 2 && V == 4, "8-byte vectors are FP16 storage");
+    const __half2 a = __floats2half2_rn(in[0], in[1]), b = __floats2half2_rn(in[2], in[3]);
+    uint2 w;
+    w.x = *reinterpret_cast<const uint32_t *>(&a);
+    w.y = *reinterpret_cast<const uint32_t *>(&b);
+    *reinterpret_cast<uint2 *>(p) = w;
+  }
+}
+
 // ------------------------------------------------------------ the update --
 // One explicit Euler step of Eq. (pytorchACeq) for one cell:
 //   phi' = phi + beta * (nsum - 2 d phi) + alpha * (phi - phi^3),

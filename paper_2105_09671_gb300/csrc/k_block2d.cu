@@ -1,0 +1,117 @@
+// Register-tile 2D stencil: kernel variants, the rule that picks one for a
+// grid, and the launch.
+#include "block2d.cuh"
+
+namespace ac {
+
+namespace {
+
+// The variants and their measured costs on GB300 (graph-replayed launches,
+// microseconds): a launch of k steps over n tiles takes about
+//   t0 + sum over an SM's rounds of (load + k * max(lat, tiles * warps * busy))
+// with t0 the launch, load one tile's load and store, lat one step's latency
+// and busy the time a warp's step keeps the SM busy.  Fitted to sweeps over
+// 64^2 .. 8192^2, warps and k; on those grids the variant, warps and k that
+// the fit picks run within 2 % of the best measured.  Which wins where:
+// 4 x 4 cells a lane up to 512^2 (400x200: 0.405 us a step against 0.42 .. 0.46
+// for the others), 8 rows near 1024^2 (0.81 against 0.99 / 0.88), 7 rows in 64
+// registers (two CTAs to an SM) from 2048^2 cells (4096^2: 8.6 us against
+// 9.6 / 10.9), and for FP16 storage 8 x 8 cells there (4096^2: 8.3 against 9.1).
+struct B2Variant {
+  int E, R, regs;
+  double t0, load, lat, busy;
+};
+constexpr B2Variant kB2[] = {
+    {4, 4, 56, 1.44, 1.21, 0.074, 0.0260},
+    {4, 7, 64, 1.65, 1.69, 0.057, 0.0402},
+    {4, 8, 96, 1.50, 1.93, 0.086, 0.0473},
+    {8, 8, 128, 2.90, 1.75, 0.246, 0.0928},
+};
+constexpr int kB2Count = sizeof(kB2) / sizeof(kB2[0]);
+
+int halo_x(int dtype, int E, int k) {
+  const int v = std::min(E, dtype == AC_F16S ? 8 : 4);  // whole memory vectors
+  return (k + v - 1) / v * v;
+}
+
+double launch_cost(const B2Variant &b, int dtype, int64_t nx, int64_t ny, int warps, int k, int num_sms) {
+  const int ow = 32 * b.E - 2 * halo_x(dtype, b.E, k), oh = warps * b.R - 2 * k;
+  const double tiles = std::ceil((double)nx / ow) * std::ceil((double)ny / oh);
+  const int occ = std::max(1, std::min(65536 / (b.regs * warps * 32), 64 / warps));
+  const double per_sm = std::ceil(tiles / num_sms);
+  const double full = std::floor(per_sm / occ), rest = per_sm - full * occ;
+  auto step = [&](double c) { return std::max(b.lat, c * warps * b.busy); };
+  return b.t0 + full * (b.load + k * step(occ)) + (rest > 0 ? b.load + k * step(rest) : 0.0);
+}
+
+template <typename T, int E, int R, int MINB>
+cudaError_t launch_t(const GridParams &g, const void *src, void *dst, int warps, int k, uint32_t mask,
+                     cudaStream_t s) {
+  static KernelSetup ks;
+  int occ = 1;
+  cudaError_t e = kernel_setup(ks, (const void *)block2d_k<T, E, R, MINB>, kB2MaxWarps * 32,
+                               b2_smem_bytes(E, kB2MaxWarps), &occ);
+  if (e != cudaSuccess) return e;
+  const int hx = halo_x(sizeof(T) == 2 ? AC_F16S : AC_F32, E, k);
+  const int ow = 32 * E - 2 * hx, oh = warps * R - 2 * k;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((g.nx + ow - 1) / ow), (unsigned)((g.ny + oh - 1) / oh));
+  cfg.blockDim = dim3(warps * 32);
+  cfg.dynamicSmemBytes = b2_smem_bytes(E, warps);
+  cfg.stream = s;
+  // programmatic stream serialization: the launch overlaps the previous
+  // one's tail (0.39 against 0.42 us a step at 64^2, nothing at 4096^2)
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, block2d_k<T, E, R, MINB>, (const T *)src, (T *)dst, g, k, hx, mask);
+}
+
+}  // namespace
+
+bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, int num_sms, Block2DPlan *out) {
+  if (dtype == AC_F64 || passes < 1) return false;
+  double best = 1e300;
+  for (int v = 0; v < kB2Count; ++v) {
+    if (kB2[v].E == 8 && dtype != AC_F16S) continue;
+    for (int warps = 4; warps <= kB2MaxWarps; warps += 4)
+      for (int kmax = 4; kmax <= kB2MaxDepth; kmax += 4) {
+        const int per = kmax / depth;  // passes per launch
+        if (per < 1 || warps * kB2[v].R - 2 * per * depth < 4) continue;
+        int64_t launches = (passes + per - 1) / per;
+        if (launches % 2 && passes > 1) ++launches;  // an even count ends in the source buffer
+        const int k = (int)((passes + launches - 1) / launches) * depth;
+        const int oh = warps * kB2[v].R - 2 * k;
+        if ((ny + oh - 1) / oh > 65535) continue;  // CUDA's grid limit in y
+        const double cost = (double)launches * launch_cost(kB2[v], dtype, nx, ny, warps, k, num_sms);
+        if (cost < best) {
+          best = cost;
+          *out = Block2DPlan{v, warps, launches};
+        }
+      }
+  }
+  return best < 1e300;
+}
+
+cudaError_t launch_block2d(int dtype, const Block2DPlan &p, const GridParams &g, const void *src, void *dst,
+                           int k, uint32_t round_mask, cudaStream_t s) {
+  if (dtype == AC_F32) {
+    switch (p.variant) {
+      case 0: return launch_t<float, 4, 4, 1>(g, src, dst, p.warps, k, 0u, s);
+      case 1: return launch_t<float, 4, 7, 2>(g, src, dst, p.warps, k, 0u, s);
+      case 2: return launch_t<float, 4, 8, 1>(g, src, dst, p.warps, k, 0u, s);
+    }
+  } else if (dtype == AC_F16S) {
+    switch (p.variant) {
+      case 0: return launch_t<__half, 4, 4, 1>(g, src, dst, p.warps, k, round_mask, s);
+      case 1: return launch_t<__half, 4, 7, 2>(g, src, dst, p.warps, k, round_mask, s);
+      case 2: return launch_t<__half, 4, 8, 1>(g, src, dst, p.warps, k, round_mask, s);
+      case 3: return launch_t<__half, 8, 8, 1>(g, src, dst, p.warps, k, round_mask, s);
+    }
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace ac

@@ -67,6 +67,21 @@ cudaError_t launch_stream2d(int dtype, int k, int tile, const GridParams &g, con
 cudaError_t launch_stream3d(int dtype, int k, int tile, const GridParams &g,
                             const CUtensorMap *src_map, void *dst, int num_sms, cudaStream_t s);
 
+// Register-tile 2D stencil (FP32 / FP16 storage): launches of up to
+// kB2MaxDepth steps.  A plan covers `passes` passes of at most `depth` steps
+// each, spread evenly over plan.launches launches (an even count unless there
+// is a single pass); false if no variant serves the grid.
+constexpr int kB2MaxDepth = 16;
+struct Block2DPlan {
+  int variant, warps;
+  int64_t launches;
+};
+bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, int num_sms, Block2DPlan *out);
+// One launch: k steps; bit s of round_mask rounds to the storage type after
+// step s + 1 (a pass end inside the launch).
+cudaError_t launch_block2d(int dtype, const Block2DPlan &p, const GridParams &g, const void *src, void *dst,
+                           int k, uint32_t round_mask, cudaStream_t s);
+
 // FP64 reductions: out[0] = sum F(phi), out[1] = sum over interior faces of
 // (phi_a - phi_b)^2, out[2] = sum (1 + phi)/2, out[3] = non-finite count.
 // partials must hold kReduceBlocks * 4 doubles.
