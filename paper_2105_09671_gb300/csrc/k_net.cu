@@ -16,9 +16,9 @@
 //                     transposed weights, raw FP32 out)
 //   net_dgrad_finish  adds the gradient of ghost cells to the boundary cell
 //                     they copy (adjoint of replicate padding), x gelu'
-//   net_wgrad_tc      dW[t][ci][co] = sum_p a[p+t][ci] g[p][co] on the
-//                     tensor cores, reduced over pixels; an all-ones row
-//                     gives the bias gradient
+//   net_wgrad         dW[t][ci][co] = sum_p a[p+t][ci] g[p][co] on the
+//                     tensor cores, reduced over pixels, and the bias
+//                     gradient (k_net_wgrad.cu)
 //   net_last_fwd/bwd, net_first_wgrad   the 1-channel ends, CUDA cores
 //   net_adam, net_pack                  optimiser and BF16 weight layouts
 #include <cuda_bf16.h>
@@ -27,7 +27,6 @@
 
 #include "kernels.h"
 #include "net.cuh"
-#include "tc.cuh"
 
 namespace ac {
 
@@ -88,129 +87,6 @@ __global__ void __launch_bounds__(256) net_first_fwd_k(const float *__restrict__
   }
 }
 
-
-// -------------------------------------------------- tensor-core wgrad ------
-// dW[t][ci][co] += sum_p a[p + t][ci] * g[p][co] and db[co] += sum_p g[p][co]
-// as a GEMM with M = T*32 (+1 all-ones row for the bias), N = 32, K = pixels,
-// 64 pixels per step, split over CTAs and added to the global gradient.
-template <int NDIM>
-struct WgradGeom {
-  static constexpr int T = net_taps(NDIM);
-  static constexpr int MROWS = T * kNetC + 1;
-  static constexpr int MT = (MROWS + 127) / 128;       // 128-row tiles
-  static constexpr int MPAD = MT * 128;
-  static constexpr int KC = 8;                          // 64 pixels = 8 chunks
-  static constexpr int A_BYTES = MPAD * 64 * 2;
-  static constexpr int B_BYTES = 32 * 64 * 2;
-  static constexpr int TMEM_COLS = MT * 32 <= 32 ? 32 : MT * 32 <= 64 ? 64 : MT * 32 <= 128 ? 128 : 256;
-  static constexpr int SMEM = A_BYTES + B_BYTES + 16;
-};
-
-template <int NDIM>
-__global__ void __launch_bounds__(128) net_wgrad_tc_k(const bf16 *__restrict__ apad,
-                                                      const bf16 *__restrict__ gpad, NetShape sh,
-                                                      float *__restrict__ gw, float *__restrict__ gb,
-                                                      int *status) {
-  using Gm = WgradGeom<NDIM>;
-  constexpr int T = Gm::T;
-  constexpr uint32_t idesc = tc_idesc_bf16_f32(128, 32);
-  extern __shared__ __align__(128) unsigned char sm[];
-  unsigned char *sA = sm;
-  unsigned char *sB = sm + Gm::A_BYTES;
-  uint64_t *bar = reinterpret_cast<uint64_t *>(sB + Gm::B_BYTES);
-  uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  for (int i = tid; i < Gm::A_BYTES / 16; i += 128) reinterpret_cast<uint4 *>(sA)[i] = make_uint4(0, 0, 0, 0);
-  if (tid == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
-  }
-  if (warp == 0) {
-    tmem_alloc(slot, Gm::TMEM_COLS);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *slot;
-  uint32_t phase = 0;
-  const int64_t n = sh.cells();
-  const int64_t chunks = (n + 63) / 64;
-  bool first = true;
-  for (int64_t ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
-    // A: rows (t, ci) = a[p_k + t][ci]; row T*32 = 1 (valid pixel) for the bias
-    for (int i = tid; i < T * 64 * 4; i += 128) {
-      const int c8 = i & 3, k = (i >> 2) & 63, t = i >> 8;
-      const int64_t pi = ch * 64 + k;
-      float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      if (pi < n) {
-        int b, z, y, x, oz, oy, ox;
-        decode_cell<NDIM>(sh, pi, b, z, y, x);
-        net_tap(NDIM, t, oz, oy, ox);
-        unpack8_bf16(*reinterpret_cast<const uint4 *>(apad + sh.ps(b, z, y, x, oz, oy, ox) * kNetC + c8 * 8), v);
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        *reinterpret_cast<bf16 *>(sA + tc_kmajor_off(t * kNetC + c8 * 8 + e, k, Gm::KC)) = __float2bfloat16_rn(v[e]);
-    }
-    for (int k = tid; k < 64; k += 128)
-      *reinterpret_cast<bf16 *>(sA + tc_kmajor_off(T * kNetC, k, Gm::KC)) =
-          __float2bfloat16_rn(ch * 64 + k < n ? 1.0f : 0.0f);
-    // B: rows co = g[p_k][co]
-    for (int i = tid; i < 64 * 4; i += 128) {
-      const int c8 = i & 3, k = i >> 2;
-      const int64_t pi = ch * 64 + k;
-      float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      if (pi < n) {
-        int b, z, y, x;
-        decode_cell<NDIM>(sh, pi, b, z, y, x);
-        unpack8_bf16(*reinterpret_cast<const uint4 *>(gpad + sh.ps(b, z, y, x, 0, 0, 0) * kNetC + c8 * 8), v);
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        *reinterpret_cast<bf16 *>(sB + tc_kmajor_off(c8 * 8 + e, k, Gm::KC)) = __float2bfloat16_rn(v[e]);
-    }
-    fence_proxy_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (tid == 0) {
-      for (int mt = 0; mt < Gm::MT; ++mt)
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t da = tc_smem_desc(sA + mt * (16 * Gm::KC * 128) + kk * 256, 128, Gm::KC * 128);
-          const uint64_t db = tc_smem_desc(sB + kk * 256, 128, Gm::KC * 128);
-          tc_mma_bf16(tmem + mt * 32, da, db, idesc, !first || kk > 0);
-        }
-      tc_commit(bar);
-    }
-    if (!mbar_wait_bounded(bar, phase)) {
-      report_timeout(status);
-      mbar_wait_bounded(bar, phase);
-    }
-    phase ^= 1u;
-    first = false;
-    tc_fence_before();
-    __syncthreads();
-  }
-  if (!first) {
-    tc_fence_after();
-    for (int mt = 0; mt < Gm::MT; ++mt) {
-      float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + mt * 32, v);
-      const int m = mt * 128 + warp * 32 + (tid & 31);
-      if (m < T * kNetC) {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) atomicAdd(gw + (int64_t)m * kNetC + c, v[c]);
-      } else if (m == T * kNetC) {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) atomicAdd(gb + c, v[c]);
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, Gm::TMEM_COLS);
-}
 
 // Cells i with clamp(i + t) == p along one axis of extent n: [lo, hi].
 __device__ __forceinline__ void clamp_preimage(int p, int t, int n, int &lo, int &hi) {
@@ -508,14 +384,12 @@ static int grid_for(int64_t n, int per_block, int num_sms) {
 // default, once per device (thread-safe; the occupancy query is unused).
 template <int NDIM>
 static cudaError_t setup_attrs() {
-  static KernelSetup k_last_t, k_last_f, k_wgrad, k_dfin;
+  static KernelSetup k_last_t, k_last_f, k_dfin;
   int occ = 0;
   cudaError_t e;
   e = kernel_setup(k_last_t, (const void *)net_last_fwd_k<NDIM, true>, 32, last_smem_bytes<NDIM>(), &occ);
   if (e != cudaSuccess) return e;
   e = kernel_setup(k_last_f, (const void *)net_last_fwd_k<NDIM, false>, 32, last_smem_bytes<NDIM>(), &occ);
-  if (e != cudaSuccess) return e;
-  e = kernel_setup(k_wgrad, (const void *)net_wgrad_tc_k<NDIM>, 32, WgradGeom<NDIM>::SMEM, &occ);
   if (e != cudaSuccess) return e;
   return kernel_setup(k_dfin, (const void *)net_dgrad_finish_k<NDIM>, 32,
                       net_taps(NDIM) * kNetC * kNetC * 4, &occ);
@@ -560,12 +434,12 @@ static cudaError_t net_backward_t(const NetBuffers &nb, const NetShape &sh, cons
   const int warps_grid = grid_for(n, 8, num_sms);
   net_last_bwd_k<NDIM><<<warps_grid, 256, 0, s>>>(nb.g6, nb.params, L.w[5], sh, nb.z[4], nb.a[4],
                                                  nb.gz[4], nb.grads, L.w[5], L.b[5]);
-  const int wgrad_grid = (int)std::min<int64_t>((n + 63) / 64, (int64_t)num_sms);
   const int64_t per = (int64_t)kNetC * net_taps(NDIM) * kNetC;
   for (int l = 4; l >= 1; --l) {
-    net_wgrad_tc_k<NDIM><<<wgrad_grid, 128, WgradGeom<NDIM>::SMEM, s>>>(
-        nb.a[l - 1], nb.gz[l], sh, nb.grads + L.w[l], nb.grads + L.b[l], nb.status);
-    cudaError_t e = net_conv_rows(1, nb.gz[l], nb.wd + (l - 1) * per, nullptr, sh, nullptr, nullptr,
+    cudaError_t e = net_wgrad(nb.a[l - 1], nb.gz[l], sh, nb.grads + L.w[l], nb.grads + L.b[l], nb.status,
+                              num_sms, s);
+    if (e != cudaSuccess) return e;
+    e = net_conv_rows(1, nb.gz[l], nb.wd + (l - 1) * per, nullptr, sh, nullptr, nullptr,
                                   nb.raw, nb.status, num_sms, s);
     if (e != cudaSuccess) return e;
     net_dgrad_finish_k<NDIM><<<warps_grid, 256, net_taps(NDIM) * kNetC * kNetC * 4, s>>>(

@@ -103,6 +103,11 @@ cudaError_t net_pack(const NetBuffers &nb, cudaStream_t s);
 cudaError_t net_conv_rows(int mode, const bf16 *in, const bf16 *Wx, const float *bias,
                           const NetShape &sh, bf16 *zout, bf16 *outpad, float *outraw, int *status,
                           int num_sms, cudaStream_t s);
+// Weight and bias gradients of one 32 -> 32 layer, added to gw / gb, from its
+// padded input activations and the padded gradient of its pre-activations
+// (zero ghost ring).
+cudaError_t net_wgrad(const bf16 *apad, const bf16 *gpad, const NetShape &sh, float *gw, float *gb, int *status,
+                      int num_sms, cudaStream_t s);
 cudaError_t net_adam(const NetBuffers &nb, float lr, float b1, float b2, float eps, int step,
                      cudaStream_t s);
 

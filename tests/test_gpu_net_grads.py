@@ -1,0 +1,50 @@
+"""Gradients of the jump network at the edges of the backward kernels' tiles
+(128 pixels x 2 rows of the weight-gradient kernel, 32 x 8 cells of the end
+layers), against the FP64 oracle with the bounds derived in test_gpu_net."""
+import numpy as np
+import pytest
+
+from oracle import net as onet
+from paper_2105_09671_gb300 import _lib as L
+
+from test_gpu_net import C_GRAD, TOL_GRAD, TOL_OUT, _elementwise_ratio, _flat, _params, _rel, _shape_args, _unflat
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(2, (3, 7, 127)), (2, (2, 8, 128)), (2, (1, 9, 129)), (2, (2, 33, 33)), (2, (1, 16, 32)), (2, (5, 1, 1)),
+          (3, (1, 3, 7, 129)), (3, (2, 2, 9, 33)), (3, (1, 1, 8, 32))]
+
+
+@pytest.mark.parametrize("ndim,shape", SHAPES)
+def test_gradients_at_tile_edges(ndim, shape):
+    import torch
+    params = _params(ndim, seed=11)
+    rng = np.random.default_rng(13)
+    phi = rng.uniform(-1, 1, size=shape).astype(np.float32).astype(np.float64)
+    target = (phi + 0.1 * rng.uniform(-1, 1, size=shape)).astype(np.float32).astype(np.float64)
+    scale = 0.1
+    loss_ref, grads_ref = onet.loss_and_grads(params, phi, target, scale, ndim)
+    h = L.ac_net_create(ndim, torch.cuda.current_stream().cuda_stream)
+    try:
+        L.ac_net_set_params(h, _flat(params))
+        d_phi = torch.tensor(phi, dtype=torch.float32, device="cuda")
+        d_tgt = torch.tensor(target, dtype=torch.float32, device="cuda")
+        b, nx, ny, nz = _shape_args(ndim, shape)
+        if nz == 1 and ndim == 3:  # the binding sizes the gradient by nz; ask the library for 3D
+            g = np.empty(L.ac_net_param_count(3), dtype=np.float32)
+            import ctypes
+            loss = ctypes.c_double()
+            L.check(L.lib().ac_net_loss_grads(ctypes.c_void_p(h), ctypes.c_void_p(d_phi.data_ptr()),
+                                              ctypes.c_void_p(d_tgt.data_ptr()), b, nx, ny, nz, scale,
+                                              ctypes.byref(loss), g.ctypes.data_as(ctypes.c_void_p)))
+            loss = loss.value
+        else:
+            loss, g = L.ac_net_loss_grads(h, d_phi.data_ptr(), d_tgt.data_ptr(), b, nx, ny, nz, scale,
+                                          want_grads=True)
+    finally:
+        L.ac_net_destroy(h)
+    assert loss == pytest.approx(loss_ref, rel=TOL_OUT)
+    for li, ((gw, gb), (rw, rb)) in enumerate(zip(_unflat(g.astype(np.float64), params), grads_ref)):
+        for got, ref in ((gw, rw), (gb, rb)):
+            assert _rel(got, ref) <= TOL_GRAD, f"layer {li}"
+            assert _elementwise_ratio(got, ref) <= C_GRAD, f"layer {li}"
