@@ -88,14 +88,6 @@ __global__ void __launch_bounds__(256) net_first_fwd_k(const float *__restrict__
 }
 
 
-// Cells i with clamp(i + t) == p along one axis of extent n: [lo, hi].
-__device__ __forceinline__ void clamp_preimage(int p, int t, int n, int &lo, int &hi) {
-  const int a = (p == 0) ? -1000000 : p;       // lower bound on i + t
-  const int b2 = (p == n - 1) ? 1000000 : p;   // upper bound on i + t
-  lo = max(a - t, 0);
-  hi = min(b2 - t, n - 1);
-}
-
 // ------------------------------------------------------------- last layer --
 // z6 = conv(a5, W6) + b6 (32 -> 1 channel) and phi_hat = phi + s z6; in
 // training also the scaled residual's gradient g6 and the loss sum.  A block
@@ -197,56 +189,6 @@ __global__ void __launch_bounds__(256) net_last_fwd_k(const bf16 *__restrict__ a
   }
 }
 
-// Warp per cell, lane = channel: gradient of the last layer (weights, bias)
-// and the gradient wrt z5 (replicate-padding adjoint, x gelu'(z5)).
-template <int NDIM>
-__global__ void __launch_bounds__(256) net_last_bwd_k(const float *__restrict__ g6,
-                                                      const float *__restrict__ params, int64_t w_off,
-                                                      NetShape sh, const bf16 *__restrict__ z5,
-                                                      const bf16 *__restrict__ a5pad,
-                                                      bf16 *__restrict__ gz5pad,
-                                                      float *__restrict__ grads, int64_t gw_off,
-                                                      int64_t gb_off) {
-  constexpr int T = net_taps(NDIM);
-  __shared__ float w[T * kNetC];
-  for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) w[i] = params[w_off + i];
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  float dw[T];
-#pragma unroll
-  for (int t = 0; t < T; ++t) dw[t] = 0.f;
-  float db = 0.f;
-  const int64_t n = sh.cells();
-  for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-    int b, z, y, x;
-    decode_cell<NDIM>(sh, i, b, z, y, x);
-    const float gp = g6[i];
-    db += gp;
-    float ga = 0.f;
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-      int oz, oy, ox;
-      net_tap(NDIM, t, oz, oy, ox);
-      dw[t] = fmaf(__bfloat162float(a5pad[sh.ps(b, z, y, x, oz, oy, ox) * kNetC + lane]), gp, dw[t]);
-      int xl, xh, yl, yh, zl = 0, zh = 0;
-      clamp_preimage(x, ox, sh.nx, xl, xh);
-      clamp_preimage(y, oy, sh.ny, yl, yh);
-      if (NDIM == 3) clamp_preimage(z, oz, sh.nz, zl, zh);
-      float s = 0.f;
-      for (int zz = zl; zz <= zh; ++zz)
-        for (int yy = yl; yy <= yh; ++yy)
-          for (int xx = xl; xx <= xh; ++xx) s += g6[sh.u(b, zz, yy, xx)];
-      ga = fmaf(w[t * kNetC + lane], s, ga);
-    }
-    const float zv = __bfloat162float(z5[i * kNetC + lane]);
-    gz5pad[sh.ps(b, z, y, x, 0, 0, 0) * kNetC + lane] = __float2bfloat16_rn(ga * net_gelu_grad(zv));
-  }
-#pragma unroll
-  for (int t = 0; t < T; ++t) atomicAdd(grads + gw_off + t * kNetC + lane, dw[t]);
-  if (lane == 0) atomicAdd(grads + gb_off, db);
-}
-
 // Warp per cell: g_{l-1} = (raw + ghost-cell gradients folded in) x gelu'(z_{l-1}).
 // raw[p] = sum_t W[t]^T g[p - t] comes from the tensor-core pass; a boundary
 // cell also receives the gradient of each ghost cell that replicates it.
@@ -304,37 +246,245 @@ __global__ void __launch_bounds__(256) net_dgrad_finish_k(const float *__restric
   }
 }
 
-// Warp per cell, lane = output channel: first-layer weight and bias gradients.
+// ---------------------------------------------- backward of the end layers --
+// A block covers tiles of 32 x 8 cells of one z.  A channel-per-lane pass over
+// staged shared memory forms the weight gradients: a half warp (2 channels a
+// lane) takes 16 cells of a row, and its window of taps is read from shared
+// memory.  kEndRow pads the pixel rows so that a warp's two half warps, on
+// adjacent rows, use different banks.
+constexpr int kEndTX = 32, kEndTY = 8;
+constexpr int kEndRow = kEndTX + 3;   // pixels per staged row of activations (34 used; 64 bytes each)
+constexpr int kEndRow1 = kEndTX + 4;  // floats per staged row of a field (34 used; whole 16-byte groups)
+
 template <int NDIM>
-__global__ void __launch_bounds__(256) net_first_wgrad_k(const float *__restrict__ phi,
-                                                         const bf16 *__restrict__ g1pad, NetShape sh,
+__host__ __device__ constexpr int end_planes() { return NDIM == 3 ? 3 : 1; }
+
+// Adds dw[t] (this lane's two channels) of all half warps of the block in
+// shared memory and then to the global gradient, float by float.
+template <int T>
+__device__ __forceinline__ void end_reduce(float *acc, const float2 *dw, float *gw) {
+  const int cl = (threadIdx.x & 15) * 2;
+  for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) acc[i] = 0.f;
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    atomicAdd(acc + t * kNetC + cl, dw[t].x);
+    atomicAdd(acc + t * kNetC + cl + 1, dw[t].y);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) atomicAdd(gw + i, acc[i]);
+}
+
+__device__ __forceinline__ float2 ld_bf2(const unsigned char *p) {
+  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+}
+
+template <int NDIM>
+__host__ __device__ constexpr int last_bwd_smem() {
+  return end_planes<NDIM>() * (kEndTY + 2) * kEndRow * 64 + end_planes<NDIM>() * (kEndTY + 2) * kEndRow1 * 4 +
+         net_taps(NDIM) * kNetC * 4;
+}
+
+// Gradient of the last layer's weights and bias, and the gradient wrt z5:
+// g5 = (sum_t W6[t] S_t) x gelu'(z5), S_t(p) the sum of g6 over the cells
+// whose tap t reads p (with replicate padding a boundary cell is also read
+// in the place of the ghosts that copy it).
+// First pass, one thread per cell: S_t from the staged g6 (zero outside the
+// grid): the cell at p - t, and per axis, where p is a face cell, the cell
+// at offset 0 once more for the tap that points out of the grid.
+// Second pass: dW6[t][c] += a5[p + t][c] g6[p] from the staged a5.
+// Bound by instruction issue (about 9 + 9 multiply-adds and a gelu' per cell
+// and channel).  One warp per cell with every operand read from global memory
+// took 2818 us for 32 x 256^2 cells.
+template <int NDIM>
+__global__ void __launch_bounds__(256, 2) net_last_bwd_k(const float *__restrict__ g6,
+                                                         const float *__restrict__ params, int64_t w_off,
+                                                         NetShape sh, const bf16 *__restrict__ z5,
+                                                         const bf16 *__restrict__ a5pad,
+                                                         bf16 *__restrict__ gz5pad,
                                                          float *__restrict__ grads, int64_t gw_off,
                                                          int64_t gb_off) {
-  constexpr int T = net_taps(NDIM);
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  float dw[T];
+  constexpr int T = net_taps(NDIM), NZR = end_planes<NDIM>(), RW = kEndTX + 2, RH = kEndTY + 2;
+  extern __shared__ __align__(16) unsigned char lsm[];
+  unsigned char *ta = lsm;                                                   // [NZR][RH][kEndRow] pixels
+  float *tg = reinterpret_cast<float *>(lsm + NZR * RH * kEndRow * 64);       // [NZR][RH][kEndRow1]
+  float *w = tg + NZR * RH * kEndRow1;                                        // [T][32]
+  for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) w[i] = params[w_off + i];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tiles_x = (sh.nx + kEndTX - 1) / kEndTX, tiles_y = (sh.ny + kEndTY - 1) / kEndTY;
+  const int64_t items = (int64_t)sh.batch * sh.nz * tiles_y * tiles_x;
+  float2 dw[T];
 #pragma unroll
-  for (int t = 0; t < T; ++t) dw[t] = 0.f;
+  for (int t = 0; t < T; ++t) dw[t] = make_float2(0.f, 0.f);
   float db = 0.f;
-  const int64_t n = sh.cells();
-  for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-    int b, z, y, x;
-    decode_cell<NDIM>(sh, i, b, z, y, x);
-    const float g = __bfloat162float(g1pad[sh.ps(b, z, y, x, 0, 0, 0) * kNetC + lane]);
-    db += g;
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const int tx = (int)(item % tiles_x);
+    int64_t r = item / tiles_x;
+    const int ty = (int)(r % tiles_y);
+    r /= tiles_y;
+    const int z = (int)(r % sh.nz), b = (int)(r / sh.nz);
+    const int x0 = tx * kEndTX, y0 = ty * kEndTY;
+    __syncthreads();  // the previous item's tiles are released (and w is complete)
+    for (int i = threadIdx.x; i < NZR * RH * RW * 4; i += blockDim.x) {
+      const int c = i & 3, q = i >> 2;
+      const int px = q % RW, row = (q / RW) % RH, dz = q / (RW * RH);
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (x0 + px < sh.px() && y0 + row < sh.py())
+        v = *reinterpret_cast<const uint4 *>(
+            a5pad + (sh.p(b, NDIM == 3 ? z + dz : 0, y0 + row, x0 + px) * kNetC + c * 8));
+      *reinterpret_cast<uint4 *>(ta + ((dz * RH + row) * kEndRow + px) * 64 + c * 16) = v;
+    }
+    for (int i = threadIdx.x; i < NZR * RH * RW; i += blockDim.x) {
+      const int px = i % RW, row = (i / RW) % RH, dz = i / (RW * RH);
+      const int xx = x0 + px - 1, yy = y0 + row - 1, zz = NDIM == 3 ? z + dz - 1 : 0;
+      const bool in = xx >= 0 && xx < sh.nx && yy >= 0 && yy < sh.ny && zz >= 0 && zz < sh.nz;
+      tg[(dz * RH + row) * kEndRow1 + px] = in ? g6[sh.u(b, zz, yy, xx)] : 0.f;
+    }
+    __syncthreads();
+    {
+      const int x = x0 + lane, y = y0 + warp;
+      if (x < sh.nx && y < sh.ny) {
+        // S[t] = g6[p - t], then the faces' second reads axis by axis
+        float S[T];
 #pragma unroll
-    for (int t = 0; t < T; ++t) {
-      int oz, oy, ox;
-      net_tap(NDIM, t, oz, oy, ox);
-      const int xx = min(max(x + ox, 0), sh.nx - 1), yy = min(max(y + oy, 0), sh.ny - 1);
-      const int zz = NDIM == 3 ? min(max(z + oz, 0), sh.nz - 1) : 0;
-      dw[t] = fmaf(phi[sh.u(b, zz, yy, xx)], g, dw[t]);
+        for (int t = 0; t < T; ++t) {
+          const int ox = t % 3 - 1, oy = (t / 3) % 3 - 1, oz = NDIM == 3 ? t / 9 - 1 : 0;
+          S[t] = tg[((NDIM == 3 ? 1 - oz : 0) * RH + warp + 1 - oy) * kEndRow1 + lane + 1 - ox];
+        }
+        db += S[T / 2];
+        if (NDIM == 3) {
+#pragma unroll
+          for (int i = 0; i < 9; ++i) {
+            const float m = S[(9 + i) % T];
+            if (z == 0) S[i] += m;
+            if (z == sh.nz - 1) S[(18 + i) % T] += m;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < T / 3; ++i) {  // (plane, ox)
+          const int o = (i / 3) * 9 + i % 3;
+          const float m = S[o + 3];
+          if (y == 0) S[o] += m;
+          if (y == sh.ny - 1) S[o + 6] += m;
+        }
+#pragma unroll
+        for (int i = 0; i < T / 3; ++i) {  // (plane, oy)
+          const float m = S[3 * i + 1];
+          if (x == 0) S[3 * i] += m;
+          if (x == sh.nx - 1) S[3 * i + 2] += m;
+        }
+        const uint4 *zs = reinterpret_cast<const uint4 *>(z5 + sh.u(b, z, y, x) * kNetC);
+        uint4 *dst = reinterpret_cast<uint4 *>(gz5pad + sh.ps(b, z, y, x, 0, 0, 0) * kNetC);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint4 zw = zs[c];
+          float ga[8] = {};
+#pragma unroll
+          for (int t = 0; t < T; ++t) {
+            const float4 wa = *reinterpret_cast<const float4 *>(w + t * kNetC + c * 8);
+            const float4 wb = *reinterpret_cast<const float4 *>(w + t * kNetC + c * 8 + 4);
+            ga[0] = fmaf(wa.x, S[t], ga[0]); ga[1] = fmaf(wa.y, S[t], ga[1]);
+            ga[2] = fmaf(wa.z, S[t], ga[2]); ga[3] = fmaf(wa.w, S[t], ga[3]);
+            ga[4] = fmaf(wb.x, S[t], ga[4]); ga[5] = fmaf(wb.y, S[t], ga[5]);
+            ga[6] = fmaf(wb.z, S[t], ga[6]); ga[7] = fmaf(wb.w, S[t], ga[7]);
+          }
+          float zv[8];
+          unpack8_bf16(zw, zv);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) ga[e] *= net_gelu_grad(zv[e]);
+          dst[c] = pack8_bf16(ga);
+        }
+      }
+    }
+    // second pass: rows 2 (warp % 4) + half, 16 cells from 16 (warp / 4)
+    const int row = 2 * (warp & 3) + (lane >> 4), xs = 16 * (warp >> 2);
+    const unsigned char *pa = ta + (row * kEndRow + xs) * 64 + (lane & 15) * 4;
+    const float *pg = tg + ((NZR / 2) * RH + row + 1) * kEndRow1 + xs + 1;
+#pragma unroll(NDIM == 3 ? 2 : 16)
+    for (int i = 0; i < 16; ++i) {
+      const float gp = pg[i];  // (zero outside the grid)
+#pragma unroll
+      for (int t = 0; t < T; ++t) {
+        const int ox = t % 3, oy = (t / 3) % 3, dz = t / 9;
+        const float2 a = ld_bf2(pa + ((dz * RH + oy) * kEndRow + i + ox) * 64);
+        dw[t].x = fmaf(a.x, gp, dw[t].x);
+        dw[t].y = fmaf(a.y, gp, dw[t].y);
+      }
     }
   }
+  __syncthreads();
+  end_reduce<T>(w, dw, grads + gw_off);
 #pragma unroll
-  for (int t = 0; t < T; ++t) atomicAdd(grads + gw_off + t * kNetC + lane, dw[t]);
-  atomicAdd(grads + gb_off + lane, db);
+  for (int o = 16; o > 0; o >>= 1) db += __shfl_xor_sync(0xffffffffu, db, o);
+  if (lane == 0) atomicAdd(grads + gb_off, db);
+}
+
+template <int NDIM>
+__host__ __device__ constexpr int first_wgrad_smem() {
+  return kEndTY * kEndRow * 64 + end_planes<NDIM>() * (kEndTY + 2) * kEndRow1 * 4 + net_taps(NDIM) * kNetC * 4;
+}
+
+// First-layer weight and bias gradients, dW1[t][c] += phi[p + t] g1[p][c]: g1
+// and phi (boundary cells replicated) staged per tile, half warps as above.
+template <int NDIM>
+__global__ void __launch_bounds__(256, 2) net_first_wgrad_k(const float *__restrict__ phi,
+                                                            const bf16 *__restrict__ g1pad, NetShape sh,
+                                                            float *__restrict__ grads, int64_t gw_off,
+                                                            int64_t gb_off) {
+  constexpr int T = net_taps(NDIM), NZR = end_planes<NDIM>(), RW = kEndTX + 2, RH = kEndTY + 2;
+  extern __shared__ __align__(16) unsigned char lsm[];
+  unsigned char *tg = lsm;                                                 // [kEndTY][kEndRow] pixels
+  float *tp = reinterpret_cast<float *>(lsm + kEndTY * kEndRow * 64);       // [NZR][RH][kEndRow1]
+  float *acc = tp + NZR * RH * kEndRow1;                                    // [T][32]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tiles_x = (sh.nx + kEndTX - 1) / kEndTX, tiles_y = (sh.ny + kEndTY - 1) / kEndTY;
+  const int64_t items = (int64_t)sh.batch * sh.nz * tiles_y * tiles_x;
+  float2 dw[T], db = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int t = 0; t < T; ++t) dw[t] = make_float2(0.f, 0.f);
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const int tx = (int)(item % tiles_x);
+    int64_t r = item / tiles_x;
+    const int ty = (int)(r % tiles_y);
+    r /= tiles_y;
+    const int z = (int)(r % sh.nz), b = (int)(r / sh.nz);
+    const int x0 = tx * kEndTX, y0 = ty * kEndTY;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kEndTY * kEndTX * 4; i += blockDim.x) {
+      const int c = i & 3, px = (i >> 2) % kEndTX, row = (i >> 2) / kEndTX;
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (x0 + px < sh.nx && y0 + row < sh.ny)
+        v = *reinterpret_cast<const uint4 *>(g1pad + sh.ps(b, z, y0 + row, x0 + px, 0, 0, 0) * kNetC + c * 8);
+      *reinterpret_cast<uint4 *>(tg + (row * kEndRow + px) * 64 + c * 16) = v;
+    }
+    for (int i = threadIdx.x; i < NZR * RH * RW; i += blockDim.x) {
+      const int px = i % RW, row = (i / RW) % RH, dz = i / (RW * RH);
+      const int xx = min(max(x0 + px - 1, 0), sh.nx - 1), yy = min(max(y0 + row - 1, 0), sh.ny - 1);
+      const int zz = NDIM == 3 ? min(max(z + dz - 1, 0), sh.nz - 1) : 0;
+      tp[(dz * RH + row) * kEndRow1 + px] = phi[sh.u(b, zz, yy, xx)];
+    }
+    __syncthreads();
+    const int row = 2 * (warp & 3) + (lane >> 4), xs = 16 * (warp >> 2);
+    const unsigned char *pg = tg + (row * kEndRow + xs) * 64 + (lane & 15) * 4;
+    const float *pp = tp + row * kEndRow1 + xs;
+#pragma unroll(NDIM == 3 ? 2 : 16)
+    for (int i = 0; i < 16; ++i) {
+      const float2 g = ld_bf2(pg + i * 64);  // (zero outside the grid)
+      db.x += g.x;
+      db.y += g.y;
+#pragma unroll
+      for (int t = 0; t < T; ++t) {
+        const int ox = t % 3, oy = (t / 3) % 3, dz = t / 9;
+        const float p = pp[(dz * RH + oy) * kEndRow1 + i + ox];
+        dw[t].x = fmaf(p, g.x, dw[t].x);
+        dw[t].y = fmaf(p, g.y, dw[t].y);
+      }
+    }
+  }
+  __syncthreads();
+  end_reduce<T>(acc, dw, grads + gw_off);
+  __syncthreads();
+  end_reduce<1>(acc, &db, grads + gb_off);
 }
 
 // ---------------------------------------------------------- optimiser -----
@@ -432,11 +582,20 @@ static cudaError_t net_backward_t(const NetBuffers &nb, const NetShape &sh, cons
   const NetLayout &L = nb.layout;
   const int64_t n = sh.cells();
   const int warps_grid = grid_for(n, 8, num_sms);
-  net_last_bwd_k<NDIM><<<warps_grid, 256, 0, s>>>(nb.g6, nb.params, L.w[5], sh, nb.z[4], nb.a[4],
-                                                 nb.gz[4], nb.grads, L.w[5], L.b[5]);
+  static KernelSetup k_last, k_first;
+  int occ_last = 1, occ_first = 1;
+  cudaError_t e = kernel_setup(k_last, (const void *)net_last_bwd_k<NDIM>, 256, last_bwd_smem<NDIM>(), &occ_last);
+  if (e != cudaSuccess) return e;
+  e = kernel_setup(k_first, (const void *)net_first_wgrad_k<NDIM>, 256, first_wgrad_smem<NDIM>(), &occ_first);
+  if (e != cudaSuccess) return e;
+  const int64_t end_items = (int64_t)sh.batch * sh.nz * ((sh.ny + kEndTY - 1) / kEndTY) *
+                            ((sh.nx + kEndTX - 1) / kEndTX);
+  net_last_bwd_k<NDIM><<<(int)std::min<int64_t>(end_items, (int64_t)num_sms * occ_last), 256,
+                         last_bwd_smem<NDIM>(), s>>>(nb.g6, nb.params, L.w[5], sh, nb.z[4], nb.a[4], nb.gz[4],
+                                                     nb.grads, L.w[5], L.b[5]);
   const int64_t per = (int64_t)kNetC * net_taps(NDIM) * kNetC;
   for (int l = 4; l >= 1; --l) {
-    cudaError_t e = net_wgrad(nb.a[l - 1], nb.gz[l], sh, nb.grads + L.w[l], nb.grads + L.b[l], nb.status,
+    e = net_wgrad(nb.a[l - 1], nb.gz[l], sh, nb.grads + L.w[l], nb.grads + L.b[l], nb.status,
                               num_sms, s);
     if (e != cudaSuccess) return e;
     e = net_conv_rows(1, nb.gz[l], nb.wd + (l - 1) * per, nullptr, sh, nullptr, nullptr,
@@ -445,7 +604,8 @@ static cudaError_t net_backward_t(const NetBuffers &nb, const NetShape &sh, cons
     net_dgrad_finish_k<NDIM><<<warps_grid, 256, net_taps(NDIM) * kNetC * kNetC * 4, s>>>(
         nb.raw, nb.gz[l], nb.params, L.w[l], sh, nb.z[l - 1], nb.gz[l - 1]);
   }
-  net_first_wgrad_k<NDIM><<<warps_grid, 256, 0, s>>>(phi, nb.gz[0], sh, nb.grads, L.w[0], L.b[0]);
+  net_first_wgrad_k<NDIM><<<(int)std::min<int64_t>(end_items, (int64_t)num_sms * occ_first), 256,
+                            first_wgrad_smem<NDIM>(), s>>>(phi, nb.gz[0], sh, nb.grads, L.w[0], L.b[0]);
   return cudaGetLastError();
 }
 
