@@ -13,9 +13,10 @@
 //                     tensor cores (k_net_conv.cu: TMA row ring, tcgen05,
 //                     accumulators in TMEM); forward (bias, GELU, ghost
 //                     writes) and the data gradient (flipped taps,
-//                     transposed weights, raw FP32 out)
-//   net_dgrad_finish  adds the gradient of ghost cells to the boundary cell
-//                     they copy (adjoint of replicate padding), x gelu'
+//                     transposed weights, x gelu')
+//   net_dgrad_faces   the data gradient of face cells: adds the gradient of
+//                     the ghost cells that copy them (adjoint of replicate
+//                     padding), x gelu'
 //   net_wgrad         dW[t][ci][co] = sum_p a[p+t][ci] g[p][co] on the
 //                     tensor cores, reduced over pixels, and the bias
 //                     gradient (k_net_wgrad.cu)
@@ -189,58 +190,82 @@ __global__ void __launch_bounds__(256) net_last_fwd_k(const bf16 *__restrict__ a
   }
 }
 
-// Warp per cell: g_{l-1} = (raw + ghost-cell gradients folded in) x gelu'(z_{l-1}).
-// raw[p] = sum_t W[t]^T g[p - t] comes from the tensor-core pass; a boundary
-// cell also receives the gradient of each ghost cell that replicates it.
+// Warp per face cell: g_{l-1} = (raw + ghost-cell gradients folded in) x
+// gelu'(z_{l-1}).  raw[p] = sum_t W[t]^T g[p - t] comes from the tensor-core
+// pass; a face cell also receives the gradient of each ghost cell that
+// replicates it.
 template <int NDIM>
-__global__ void __launch_bounds__(256) net_dgrad_finish_k(const float *__restrict__ raw,
-                                                          const bf16 *__restrict__ gpad,
-                                                          const float *__restrict__ params,
-                                                          int64_t w_off, NetShape sh,
-                                                          const bf16 *__restrict__ zprev,
-                                                          bf16 *__restrict__ gprevpad) {
-  constexpr int T = net_taps(NDIM);
-  extern __shared__ float wsm[];  // W[t][ci][co]
-  for (int i = threadIdx.x; i < T * kNetC * kNetC; i += blockDim.x) wsm[i] = params[w_off + i];
+__host__ __device__ constexpr int faces_smem() { return net_taps(NDIM) * kNetC * (kNetC + 1) * 4; }
+
+template <int NDIM>
+__global__ void __launch_bounds__(256) net_dgrad_faces_k(const float *__restrict__ raw,
+                                                         const bf16 *__restrict__ gpad,
+                                                         const float *__restrict__ params,
+                                                         int64_t w_off, NetShape sh,
+                                                         const bf16 *__restrict__ zprev,
+                                                         bf16 *__restrict__ gprevpad) {
+  constexpr int T = net_taps(NDIM), WS = kNetC + 1;  // (odd stride: lanes on different banks)
+  extern __shared__ float wsm[];                     // W[t][ci][co], WS floats per (t, ci)
+  for (int i = threadIdx.x; i < T * kNetC * kNetC; i += blockDim.x)
+    wsm[(i / kNetC) * WS + i % kNetC] = params[w_off + i];
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  const int64_t n = sh.cells();
-  for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-    int b, z, y, x;
-    decode_cell<NDIM>(sh, i, b, z, y, x);
-    float g = raw[i * kNetC + lane];
-    const bool bx = (x == 0 || x == sh.nx - 1), by = (y == 0 || y == sh.ny - 1);
-    const bool bz = NDIM == 3 && (z == 0 || z == sh.nz - 1);
-    if (bx || by || bz) {
-      // ghost cells q (outside the grid) with clamp(q) == p
-      for (int gz = (NDIM == 3 ? -1 : 0); gz <= (NDIM == 3 ? 1 : 0); ++gz)
-        for (int gy = -1; gy <= 1; ++gy)
-          for (int gx = -1; gx <= 1; ++gx) {
-            const int qx = x + gx, qy = y + gy, qz = z + gz;
-            const bool out = qx < 0 || qx >= sh.nx || qy < 0 || qy >= sh.ny ||
-                             (NDIM == 3 && (qz < 0 || qz >= sh.nz));
-            if (!out) continue;
-            if (min(max(qx, 0), sh.nx - 1) != x || min(max(qy, 0), sh.ny - 1) != y) continue;
-            if (NDIM == 3 && min(max(qz, 0), sh.nz - 1) != z) continue;
-            if (qx < -1 || qx > sh.nx || qy < -1 || qy > sh.ny) continue;
-            if (NDIM == 3 && (qz < -1 || qz > sh.nz)) continue;
-            // gradient of the ghost cell q: sum_t W[t][ci = lane][co] g[q - t][co]
-            float acc = 0.f;
-            for (int t = 0; t < T; ++t) {
-              int oz, oy, ox;
-              net_tap(NDIM, t, oz, oy, ox);
-              const int sx = qx - ox, sy = qy - oy, sz = qz - oz;
-              if (sx < 0 || sx >= sh.nx || sy < 0 || sy >= sh.ny) continue;
-              if (NDIM == 3 && (sz < 0 || sz >= sh.nz)) continue;
-              const float gv = __bfloat162float(gpad[sh.ps(b, NDIM == 3 ? sz : 0, sy, sx, 0, 0, 0) * kNetC + lane]);
-              // lane holds g[.][co = lane]; W[t][ci = lane][co] needs all co
-              for (int co = 0; co < kNetC; ++co)
-                acc = fmaf(wsm[(t * kNetC + lane) * kNetC + co], __shfl_sync(0xffffffffu, gv, co), acc);
-            }
-            g += acc;
-          }
+  // face cells of an image: the rows on y and z faces whole, then the two end
+  // cells of the other rows
+  const int fy = min(sh.ny, 2), fz = NDIM == 3 ? min(sh.nz, 2) : 0, fx = min(sh.nx, 2);
+  const int64_t whole = ((int64_t)fz * sh.ny + (int64_t)(sh.nz - fz) * fy) * sh.nx;
+  const int64_t per = whole + (int64_t)(sh.nz - fz) * (sh.ny - fy) * fx;
+  for (int64_t u = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); u < per * sh.batch; u += warps) {
+    const int b = (int)(u / per);
+    int64_t f = u - b * per;
+    int z, y, x;
+    if (f < whole) {
+      x = (int)(f % sh.nx);
+      f /= sh.nx;
+      if (f < (int64_t)fz * sh.ny) {
+        z = f < sh.ny ? 0 : sh.nz - 1;
+        y = (int)(f % sh.ny);
+      } else {
+        f -= (int64_t)fz * sh.ny;
+        z = (NDIM == 3 ? 1 : 0) + (int)(f / fy);
+        y = f % fy ? sh.ny - 1 : 0;
+      }
+    } else {
+      f -= whole;
+      x = f % fx ? sh.nx - 1 : 0;
+      f /= fx;
+      z = (NDIM == 3 ? 1 : 0) + (int)(f / (sh.ny - fy));
+      y = 1 + (int)(f % (sh.ny - fy));
     }
+    const int64_t i = sh.u(b, z, y, x);
+    float g = raw[i * kNetC + lane];
+    // ghost cells q (one cell outside the grid) with clamp(q) == p
+    for (int gz = (NDIM == 3 ? -1 : 0); gz <= (NDIM == 3 ? 1 : 0); ++gz)
+      for (int gy = -1; gy <= 1; ++gy)
+        for (int gx = -1; gx <= 1; ++gx) {
+          const int qx = x + gx, qy = y + gy, qz = z + gz;
+          const bool out = qx < 0 || qx >= sh.nx || qy < 0 || qy >= sh.ny ||
+                           (NDIM == 3 && (qz < 0 || qz >= sh.nz));
+          if (!out) continue;
+          if (min(max(qx, 0), sh.nx - 1) != x || min(max(qy, 0), sh.ny - 1) != y) continue;
+          if (NDIM == 3 && min(max(qz, 0), sh.nz - 1) != z) continue;
+          // gradient of the ghost cell q: sum_t W[t][ci = lane][co] g[q - t][co]
+          float acc = 0.f;
+          for (int t = 0; t < T; ++t) {
+            int oz, oy, ox;
+            net_tap(NDIM, t, oz, oy, ox);
+            const int sx = qx - ox, sy = qy - oy, sz = qz - oz;
+            if (sx < 0 || sx >= sh.nx || sy < 0 || sy >= sh.ny) continue;
+            if (NDIM == 3 && (sz < 0 || sz >= sh.nz)) continue;
+            const float gv = __bfloat162float(gpad[sh.ps(b, NDIM == 3 ? sz : 0, sy, sx, 0, 0, 0) * kNetC + lane]);
+            // lane holds g[.][co = lane]; W[t][ci = lane][co] needs all co
+#pragma unroll 8
+            for (int co = 0; co < kNetC; ++co)
+              acc = fmaf(wsm[(t * kNetC + lane) * WS + co], __shfl_sync(0xffffffffu, gv, co), acc);
+          }
+          g += acc;
+        }
     const float zv = __bfloat162float(zprev[i * kNetC + lane]);
     gprevpad[sh.ps(b, z, y, x, 0, 0, 0) * kNetC + lane] = __float2bfloat16_rn(g * net_gelu_grad(zv));
   }
@@ -541,8 +566,8 @@ static cudaError_t setup_attrs() {
   if (e != cudaSuccess) return e;
   e = kernel_setup(k_last_f, (const void *)net_last_fwd_k<NDIM, false>, 32, last_smem_bytes<NDIM>(), &occ);
   if (e != cudaSuccess) return e;
-  return kernel_setup(k_dfin, (const void *)net_dgrad_finish_k<NDIM>, 32,
-                      net_taps(NDIM) * kNetC * kNetC * 4, &occ);
+  return kernel_setup(k_dfin, (const void *)net_dgrad_faces_k<NDIM>, 32,
+                      faces_smem<NDIM>(), &occ);
 }
 
 template <int NDIM>
@@ -562,7 +587,7 @@ static cudaError_t net_forward_t(const NetBuffers &nb, const NetShape &sh, const
     bf16 *in = nb.a[(l - 1) % (train ? 5 : 2)];
     bf16 *out = nb.a[l % (train ? 5 : 2)];
     e = net_conv_rows(0, in, nb.wf + (l - 1) * per, nb.params + L.b[l], sh,
-                      train ? nb.z[l] : nullptr, out, nullptr, nb.status, num_sms, s);
+                      train ? nb.z[l] : nullptr, out, nullptr, nullptr, nb.status, num_sms, s);
     if (e != cudaSuccess) return e;
   }
   const bf16 *a5 = nb.a[4 % (train ? 5 : 2)];
@@ -581,7 +606,6 @@ static cudaError_t net_backward_t(const NetBuffers &nb, const NetShape &sh, cons
                                   int num_sms, cudaStream_t s) {
   const NetLayout &L = nb.layout;
   const int64_t n = sh.cells();
-  const int warps_grid = grid_for(n, 8, num_sms);
   static KernelSetup k_last, k_first;
   int occ_last = 1, occ_first = 1;
   cudaError_t e = kernel_setup(k_last, (const void *)net_last_bwd_k<NDIM>, 256, last_bwd_smem<NDIM>(), &occ_last);
@@ -598,10 +622,10 @@ static cudaError_t net_backward_t(const NetBuffers &nb, const NetShape &sh, cons
     e = net_wgrad(nb.a[l - 1], nb.gz[l], sh, nb.grads + L.w[l], nb.grads + L.b[l], nb.status,
                               num_sms, s);
     if (e != cudaSuccess) return e;
-    e = net_conv_rows(1, nb.gz[l], nb.wd + (l - 1) * per, nullptr, sh, nullptr, nullptr,
-                                  nb.raw, nb.status, num_sms, s);
+    e = net_conv_rows(1, nb.gz[l], nb.wd + (l - 1) * per, nullptr, sh, nullptr, nb.gz[l - 1], nb.raw,
+                      nb.z[l - 1], nb.status, num_sms, s);
     if (e != cudaSuccess) return e;
-    net_dgrad_finish_k<NDIM><<<warps_grid, 256, net_taps(NDIM) * kNetC * kNetC * 4, s>>>(
+    net_dgrad_faces_k<NDIM><<<(int)std::min<int64_t>((n + 7) / 8, (int64_t)num_sms * (NDIM == 3 ? 2 : 4)), 256, faces_smem<NDIM>(), s>>>(
         nb.raw, nb.gz[l], nb.params, L.w[l], sh, nb.z[l - 1], nb.gz[l - 1]);
   }
   net_first_wgrad_k<NDIM><<<(int)std::min<int64_t>(end_items, (int64_t)num_sms * occ_first), 256,
