@@ -4,31 +4,36 @@
 //   out[p][n] = sum_{t < T} sum_{c < 32} in[p + t][c] * Wx[n][t*32 + c]
 //
 // Work item: 128 consecutive x positions of a run of output rows (one z, one
-// image).  The input rows reach shared memory once each, by TMA, and stay in
-// a ring while the three output rows that use them are formed:
-//   - layout of one padded input row: 4 planes of 8 channels, each plane the
-//     130 pixels x0-1 .. x0+128 at 16 bytes per pixel (one 2D TMA box of
-//     8 channels x 130 pixels), so that pixel m sits at 16 m bytes; an x
-//     offset of a tap is then +16 bytes on the descriptor's start address
-//     (canonical K-major layout without swizzle: LBO = plane stride between
-//     the K-adjacent 8-channel core matrices, SBO = 128 bytes between 8-pixel
-//     groups);
+// image).  Each input row reaches shared memory once, by TMA, and is used
+// once, for the three output rows that it touches:
+//   - one padded input row is the 130 pixels x0-1 .. x0+128 at 64 bytes (32
+//     channels) each, one 2D TMA box in the 64-byte swizzle (K-major), so an x
+//     offset of a tap is +64 bytes on the descriptor's start address and the
+//     second half of the channels +32;
 //   - warp 0 (one thread) issues the TMA loads into a ring of row sets (the
 //     1 or 3 rows of one y at every needed z), each set on a full / empty
 //     mbarrier pair;
-//   - warps 1 and 6 (one thread each, alternate output rows) issue T x 2
-//     tcgen05.mma (M = 128 pixels, N = 32, K = 16) per output row into one
-//     of their two TMEM accumulators and commit to the accumulator's
-//     barrier and to the empty barriers of the sets this issuer no longer
-//     reads (each set is released once by each issuer);
-//   - warps 2..5 read the accumulator (tcgen05.ld, lanes 32 (w % 4) ..),
-//     release it, and run the epilogue: bias, pre-activation store, GELU
-//     (tanh form, hardware tanh approximation) and the store with its
-//     replicated ghost ring; or, for the data gradient, x gelu'(z) and the
-//     store into the padded gradient for cells inside the grid, the raw FP32
-//     sum for cells on its faces (net_dgrad_faces adds what their ghosts
-//     received).  Writing the raw sums of all cells and finishing them in a
-//     second pass took 140 + 800 us at 32 x 256^2 pixels.
+//   - TMEM holds a ring of 8 output rows of 32 columns.  Input row r adds to
+//     output rows r-1, r, r+1 (through the taps oy = +1, 0, -1), which are
+//     adjacent blocks of columns: with the weights of the three oy side by
+//     side in N, one tcgen05.mma (M = 128 pixels, N = 96, K = 16) per ox, dz
+//     and half of the channels serves all three.  The MMA that touches an
+//     output row first starts it from zero (N = 32), and a triple that wraps
+//     around the ring is split in two.  Warp 1 (one thread) issues them (its
+//     own latency counts: operands that cost ~50 instructions an MMA to form
+//     made a row take 2200 clocks) and
+//     commits to the set's empty barrier and, once its last tap is in, to the
+//     output row's barrier;
+//   - warps 2..9 read finished rows (tcgen05.ld, lanes 32 (w % 4) ..; two
+//     groups of four warps take alternate rows), release them, and run the
+//     epilogue: bias, pre-activation store, GELU (tanh form, hardware tanh
+//     approximation) and the store with its replicated ghost ring; or, for the
+//     data gradient, x gelu'(z) and the store into the padded gradient for
+//     cells inside the grid, the raw FP32 sum for cells on its faces
+//     (net_dgrad_faces adds what their ghosts received).
+// Bound: operand reads from shared memory.  With one MMA per tap (N = 32) the
+// A rows were read 18 times (2D) instead of 6 to 8 times: 720 clocks of
+// 128-byte reads per 128-pixel row.
 // Every wait is bounded; a timeout sets the status word and the roles wind
 // down without leaving copies or MMAs in flight.
 #include "kernels.h"
@@ -40,21 +45,20 @@ namespace ac {
 namespace {
 
 constexpr int kCvPix = 130;                // 128 outputs + 2 halo columns
-constexpr int kCvPlane = 136 * 16;         // bytes of one 8-channel plane (rows padded to 136)
-constexpr int kCvRow = 4 * kCvPlane;       // one padded input row (32 channels)
-constexpr int kCvBox = 8 * kCvPix * 2;     // bytes of one TMA box
-constexpr int kCvThreads = 224;  // TMA warp, 2 MMA warps, 4 epilogue warps
-constexpr int kCvIssuers = 2;    // MMA-issuing warps (alternate output rows)
+constexpr int kCvBox = kCvPix * 64;        // bytes of one input row (one TMA box)
+constexpr int kCvRow = (kCvBox + 511) / 512 * 512;  // its place (the swizzle pattern repeats every 512)
+constexpr int kCvThreads = 320;  // TMA warp, MMA warp, 8 epilogue warps
+constexpr int kCvGroups = 2;     // epilogue groups of four warps (alternate output rows)
 
 template <int NDIM>
 struct CvGeom {
   static constexpr int NZ = NDIM == 3 ? 3 : 1;       // rows per set (z - 1, z, z + 1)
   static constexpr int NS = NDIM == 3 ? 6 : 8;       // sets in the ring
   static constexpr int MINB = NDIM == 3 ? 1 : 2;     // CTAs per SM
-  static constexpr int NACC = 4;                      // TMEM accumulators (2 per issuer)
+  static constexpr int NACC = 8;                      // output rows in TMEM
   static constexpr int T = net_taps(NDIM);
   static constexpr int KB = T * kNetC;                // GEMM K
-  static constexpr int KCB = KB / 8;                  // 8-element K chunks of B
+  static constexpr int NG = T / 3;                    // (dz, ox) groups of B: 96 x 32 each
   static constexpr int SET = NZ * kCvRow;
   static constexpr int OFF_A = (64 * KB + 1023) / 1024 * 1024;
   static constexpr int OFF_BAR = OFF_A + NS * SET;
@@ -96,9 +100,8 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
                     bf16 *__restrict__ outpad, float *__restrict__ outraw, const bf16 *__restrict__ zin,
                     int *status) {
   using Gm = CvGeom<NDIM>;
-  constexpr int NS = Gm::NS, NZ = Gm::NZ, T = Gm::T, KCB = Gm::KCB, KB = Gm::KB;
+  constexpr int NS = Gm::NS, NZ = Gm::NZ, NG = Gm::NG, KB = Gm::KB;
   constexpr int NACC = Gm::NACC;
-  constexpr uint32_t idesc = tc_idesc_bf16_f32(128, 32);
   extern __shared__ __align__(1024) unsigned char sm[];
   unsigned char *sB = sm;
   unsigned char *sA = sm + Gm::OFF_A;
@@ -113,23 +116,26 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid < 32) sbias[tid] = MODE == 0 ? bias[tid] : 0.0f;
 
-  // B operand (32 x KB, canonical K-major) for the CTA's lifetime
-  for (int i = tid; i < 32 * KCB; i += kCvThreads) {
-    const int n = i / KCB, c = i - n * KCB;
-    *reinterpret_cast<uint4 *>(sB + tc_kmajor_off(n, c * 8, KCB)) =
-        *reinterpret_cast<const uint4 *>(Wx + (int64_t)n * KB + c * 8);
+  // B operand for the CTA's lifetime: per group (dz, ox) 96 rows n = (2 - dy)
+  // * 32 + output channel, dy the tap's row (0..2), by 32 input channels,
+  // canonical K-major
+  for (int i = tid; i < NG * 96 * 4; i += kCvThreads) {
+    const int k8 = i & 3, n = (i >> 2) % 96, gq = (i >> 2) / 96;
+    const int t = (gq / 3) * 9 + (2 - n / 32) * 3 + gq % 3;
+    *reinterpret_cast<uint4 *>(sB + gq * 96 * 64 + tc_kmajor_off(n, k8 * 8, 4)) =
+        *reinterpret_cast<const uint4 *>(Wx + (int64_t)(n % 32) * KB + t * 32 + k8 * 8);
   }
   if (tid == 0) {
     tma_prefetch_desc(&in_map);
     for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], kCvIssuers);  // each issuer releases every set once
+      mbar_init(&empty[s], 1);
     }
     for (int a = 0; a < NACC; ++a) {
       mbar_init(&accf[a], 1);
       mbar_init(&acce[a], 4);
     }
-    mbar_init(fin, kCvIssuers);
+    mbar_init(fin, 1);
     fence_mbar_init();
     abort_flag = 0;
   }
@@ -164,13 +170,11 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&full[s], NZ * 4 * kCvBox);
+          mbar_arrive_expect_tx(&full[s], NZ * kCvBox);
           for (int dz = 0; dz < NZ; ++dz) {
             // padded row (z + dz, ya + r) from padded column x0 (= cell x0 - 1)
             const int64_t p0 = sh.p(it.b, NDIM == 3 ? it.z + dz : 0, it.ya + r, it.x0);
-            for (int kc = 0; kc < 4; ++kc)
-              tma_load_2d(sA + s * Gm::SET + dz * kCvRow + kc * kCvPlane, &in_map, &full[s],
-                          kc * 8, (int)p0);
+            tma_load_2d(sA + s * Gm::SET + dz * kCvRow, &in_map, &full[s], 0, (int)p0);
           }
         }
       }
@@ -182,80 +186,70 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
       for (uint32_t v = i > (uint32_t)NS ? i - NS : 0; v < i; ++v)
         mbar_wait_bounded(&full[v % NS], (v / NS) & 1u);
     }
-  } else if (warp == 1 || warp == 6) {
+  } else if (warp == 1) {
     // ------------------------------------------------------------- MMAs --
-    // Issuer p takes the item's output rows j = p, p + 2, ...; its k-th row
-    // goes to accumulator p + 2 (k % 2).  It releases set j and j + 1 after
-    // row j (their last use by this issuer); the item's other sets are
-    // released before its first row (those it never reads) or after its
-    // last row (the rest).
-    const int p = warp == 6 ? 1 : 0;
     if (lane == 0) {
-      const uint64_t a_desc0 = tc_smem_desc(sA, kCvPlane, 128);       // A rows: LBO plane, SBO 8 px
-      const uint64_t b_desc0 = tc_smem_desc(sB, 128, KCB * 128);      // B: canonical K-major
-      uint32_t i = 0, kq = 0;  // row sets consumed (CTA), rows formed by this issuer
+      const uint64_t a_desc0 = tc_smem_desc_sw64(sA, 16, 512);  // A rows: SBO 8 px
+      const uint64_t b_desc0 = tc_smem_desc(sB, 128, 512);      // B: canonical K-major, 32 channels
+      // (dz, ox) and channel half gk: offsets of A's and B's start addresses
+      auto a_off = [](int gk) {
+        return (uint32_t)(((gk / 6) * kCvRow + (gk / 2 % 3) * 64 + (gk & 1) * 32) >> 4);
+      };
+      auto b_off = [](int gk) { return (uint32_t)(((gk >> 1) * 96 * 64 + (gk & 1) * 256) >> 4); };
+      constexpr uint32_t idesc0 = tc_idesc_bf16_f32(128, 0);  // + (N / 32) << 19
+      uint32_t i = 0, q0 = 0;  // row sets used; output rows of the items before this one
       bool ok = true;
       for (int64_t item = blockIdx.x; item < items && ok; item += gridDim.x) {
         const CvItem it = cv_item(item, sh, tiles_x, nchunk, chunk);
-        const uint32_t base = i;
-        const bool had = it.nrows > p;
-        // sets this issuer never reads are released before its first row:
-        // those below it (all of them if it has no row in this item), so
-        // the producer can refill their slots while the other issuer works.
-        // Each release waits for the set to be loaded first: only then has
-        // the slot's previous phase completed, so the arrival counts for
-        // this set and not for the slot's previous occupant.
-        for (int r = 0; r <= it.nrows + 1 && ok; ++r)
-          if (!had || r < p) {
-            const uint32_t k = base + r;
-            if (!mbar_wait_bounded(&full[k % NS], (k / NS) & 1u)) ok = false;
-            else mbar_arrive(&empty[k % NS]);
+        for (int r = 0; r < it.nrows + 2; ++r, ++i) {
+          const int s = (int)(i % NS);
+          // the block that this row starts must have been read
+          if (r < it.nrows) {
+            const uint32_t q = q0 + r;
+            if (q >= (uint32_t)NACC && !mbar_wait_bounded(&acce[q % NACC], (q / NACC - 1) & 1u)) ok = false;
           }
-        for (int j = p; j < it.nrows && ok; j += kCvIssuers, ++kq) {
-          for (uint32_t k = base + j; k <= base + j + 2; ++k)
-            if (!mbar_wait_bounded(&full[k % NS], (k / NS) & 1u)) ok = false;
-          const uint32_t buf = p + kCvIssuers * (kq % 2);
-          if (kq >= 2 && !mbar_wait_bounded(&acce[buf], ((kq / 2) - 1) & 1u)) ok = false;
+          if (ok && !mbar_wait_bounded(&full[s], (i / NS) & 1u)) ok = false;
           if (!ok || abort_flag) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t d = tmem + buf * 32;
-          // descriptors: the start-address field is addr >> 4 in the low 14
-          // bits, so a byte offset off (16-byte multiple, inside shared
-          // memory) is + off >> 4 on the base descriptor
-          uint32_t srow[3];
+          const uint64_t da = a_desc0 + (uint32_t)(s * (Gm::SET >> 4));
+          // output rows j0 .. j1 of the item, row j through tap dy = r - j
+          // (block 2 - dy of B's rows); segment 1 is what wraps around the ring
+          const int j0 = max(r - 2, 0), j1 = min(r, it.nrows - 1);
+          const uint32_t blk = (q0 + j0) % NACC;
+          const int c0 = min(j1 - j0 + 1, NACC - (int)blk), c1 = j1 - j0 + 1 - c0;
+          const uint32_t d0 = tmem + blk * 32;
+          const uint64_t db0 = b_desc0 + (uint32_t)(((2 - (r - j0)) * 4 * 512) >> 4);
+          const uint64_t db1 = db0 + (uint32_t)((c0 * 4 * 512) >> 4);
+          const uint32_t id0 = idesc0 + ((uint32_t)c0 << 19), id1 = idesc0 + ((uint32_t)c1 << 19);
+          // first the MMA that starts row r from zero, and its older rows
+          const int fresh = r < it.nrows ? 1 : 0;
+          if (c1 == 0) {
+            if (fresh)
+              tc_mma_bf16(d0 + (c0 - 1) * 32, da, db0 + (uint32_t)(((c0 - 1) * 4 * 512) >> 4),
+                          idesc0 + (1u << 19), false);
+            if (c0 > fresh) tc_mma_bf16(d0, da, db0, idesc0 + ((uint32_t)(c0 - fresh) << 19), true);
 #pragma unroll
-          for (int dy = 0; dy < 3; ++dy) srow[dy] = ((base + j + dy) % NS) * (Gm::SET >> 4);
+            for (int gk = 1; gk < 2 * NG; ++gk)
+              tc_mma_bf16(d0, da + a_off(gk), db0 + b_off(gk), id0, true);
+          } else {
+            tc_mma_bf16(d0, da, db0, id0, true);
+            if (fresh)
+              tc_mma_bf16(tmem + (c1 - 1) * 32, da, db1 + (uint32_t)(((c1 - 1) * 4 * 512) >> 4),
+                          idesc0 + (1u << 19), false);
+            if (c1 > fresh) tc_mma_bf16(tmem, da, db1, idesc0 + ((uint32_t)(c1 - fresh) << 19), true);
 #pragma unroll
-          for (int t = 0; t < T; ++t) {
-            const int ox = t % 3 - 1, oy = (t / 3) % 3 - 1, dz = NDIM == 3 ? t / 9 : 0;
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk) {
-              const uint64_t da = a_desc0 + srow[oy + 1] +
-                                  (uint32_t)((dz * kCvRow + (ox + 1) * 16 + 2 * kk * kCvPlane) >> 4);
-              const uint64_t db = b_desc0 + (uint32_t)(((t * 4 + kk * 2) * 128) >> 4);
-              tc_mma_bf16(d, da, db, idesc, (t | kk) != 0);
+            for (int gk = 1; gk < 2 * NG; ++gk) {
+              tc_mma_bf16(d0, da + a_off(gk), db0 + b_off(gk), id0, true);
+              tc_mma_bf16(tmem, da + a_off(gk), db1 + b_off(gk), id1, true);
             }
           }
-          tc_commit(&accf[buf]);
-          tc_commit(&empty[(base + j) % NS]);      // this issuer's last use of set j
-          tc_commit(&empty[(base + j + 1) % NS]);  // and of set j + 1
+          tc_commit(&empty[s]);
+          if (r >= 2) tc_commit(&accf[(q0 + r - 2) % NACC]);
         }
-        if (!ok) break;
-        // the sets above its last row + 1, once that row's MMAs completed
-        // (and, as above, once the set is loaded)
-        if (had) {
-          const int last = it.nrows - 1 - ((it.nrows - 1 - p) % kCvIssuers + kCvIssuers) % kCvIssuers;
-          for (int r = last + 2; r <= it.nrows + 1 && ok; ++r) {
-            const uint32_t k = base + r;
-            if (!mbar_wait_bounded(&full[k % NS], (k / NS) & 1u)) ok = false;
-            else tc_commit(&empty[k % NS]);
-          }
-        }
-        if (!ok) break;
-        i = base + it.nrows + 2;
+        q0 += it.nrows;
       }
       if (!ok && !abort_flag) {
         report_timeout(status);
@@ -268,15 +262,14 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
   } else {
     // -------------------------------------------------------- epilogue --
     const int q = warp & 3;  // TMEM lane quarter of this warp
-    uint32_t kq[kCvIssuers] = {};  // rows formed so far by each issuer
+    const uint32_t grp = (uint32_t)(warp - 2) >> 2;
+    uint32_t q0 = 0;  // output rows of the items before this one
     bool ok = true;
     for (int64_t item = blockIdx.x; item < items && ok; item += gridDim.x) {
       const CvItem it = cv_item(item, sh, tiles_x, nchunk, chunk);
-      for (int j = 0; j < it.nrows; ++j) {
-        const int ip = j % kCvIssuers;  // the issuer of this row and its accumulator
-        const uint32_t buf = ip + kCvIssuers * (kq[ip] % 2);
-        const uint32_t par = (kq[ip] / 2) & 1u;
-        ++kq[ip];
+      for (int j = (int)((grp + q0) & 1u); j < it.nrows; j += kCvGroups) {
+        const uint32_t buf = (q0 + j) % NACC;
+        const uint32_t par = ((q0 + j) / NACC) & 1u;
         const int x = it.x0 + q * 32 + lane;
         const int y = it.ya + j;
         bool inner = false;
@@ -332,6 +325,7 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
           }
         }
       }
+      q0 += it.nrows;
     }
     if (!ok && lane == 0 && !abort_flag) {
       report_timeout(status);
@@ -366,9 +360,9 @@ static cudaError_t conv_rows_t(const bf16 *in, const bf16 *Wx, const float *bias
   CUtensorMap map;
   const cuuint64_t dims[2] = {(cuuint64_t)kNetC, (cuuint64_t)P};
   const cuuint64_t strides[1] = {(cuuint64_t)kNetC * 2};
-  const cuuint32_t box[2] = {8, (cuuint32_t)kCvPix}, es[2] = {1, 1};
+  const cuuint32_t box[2] = {(cuuint32_t)kNetC, (cuuint32_t)kCvPix}, es[2] = {1, 1};
   if (fn(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(in), dims, strides, box, es,
-         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   // rows per item: about two items per resident CTA, at least 4 rows (each

@@ -30,6 +30,16 @@ __device__ __forceinline__ uint64_t tc_smem_desc(const void *start, uint32_t lbo
   return d;
 }
 
+// The same for operands in the 64-byte swizzle (layout code 4 in bits 61-63):
+// rows of 64 bytes whose 16-byte chunk index is XORed with bits 7-8 of the
+// shared-memory address, as TMA's SWIZZLE_64B writes them.  The pattern is
+// tied to the address, so a start that is any whole number of rows in (a
+// pixel shift) or 32 bytes in (the second half of K) needs base offset 0.
+__device__ __forceinline__ uint64_t tc_smem_desc_sw64(const void *start, uint32_t lbo_bytes,
+                                                       uint32_t sbo_bytes) {
+  return tc_smem_desc(start, lbo_bytes, sbo_bytes) | ((uint64_t)4 << 61);
+}
+
 // Instruction descriptor of kind::f16 for BF16 x BF16 -> FP32, both operands
 // K-major: D format (bits 4-5) = 1 (F32), A format (7-9) = 1 (BF16), B format
 // (10-12) = 1 (BF16), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
