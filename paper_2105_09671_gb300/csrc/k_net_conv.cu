@@ -278,9 +278,9 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
           inner = x > 0 && x < sh.nx - 1 && y > 0 && y < sh.ny - 1 &&
                   (NDIM == 2 || (it.z > 0 && it.z < sh.nz - 1));
           if (inner) {
-            const uint4 *zs = reinterpret_cast<const uint4 *>(zin + sh.u(it.b, it.z, y, x) * kNetC);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) zw[c] = zs[c];
+            const bf16 *zs = zin + sh.u(it.b, it.z, y, x) * kNetC;
+            ld_global32(zs, zw[0], zw[1]);
+            ld_global32(zs + 16, zw[2], zw[3]);
           }
         }
         const bool got = mbar_wait_bounded(&accf[buf], par);
@@ -297,26 +297,32 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
         if (x < sh.nx) {
           const int64_t pu = sh.u(it.b, it.z, y, x);
           if (MODE == 0) {
+            uint64_t xv[16];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) v[c] += sbias[c];
+            for (int c = 0; c < 16; ++c)
+              xv[c] = add2(pack2(v[2 * c], v[2 * c + 1]), reinterpret_cast<const uint64_t *>(sbias)[c]);
             if (zout) {
-              uint4 *dz = reinterpret_cast<uint4 *>(zout + pu * kNetC);
 #pragma unroll
-              for (int c = 0; c < 4; ++c) dz[c] = pack8_bf16(v + 8 * c);
+              for (int c = 0; c < 16; ++c) unpack2(xv[c], v[2 * c], v[2 * c + 1]);
+              bf16 *dz = zout + pu * kNetC;
+              st_global32(dz, pack8_bf16(v), pack8_bf16(v + 8));
+              st_global32(dz + 16, pack8_bf16(v + 16), pack8_bf16(v + 24));
             }
 #pragma unroll
-            for (int c = 0; c < 32; ++c) v[c] = net_gelu_fast(v[c]);
+            for (int c = 0; c < 16; ++c) unpack2(net_gelu_fast2(xv[c]), v[2 * c], v[2 * c + 1]);
             store_replicated<NDIM>(outpad, sh, it.b, it.z, y, x, v);
           } else if (inner) {
-            uint4 *d = reinterpret_cast<uint4 *>(outpad + sh.ps(it.b, it.z, y, x, 0, 0, 0) * kNetC);
+            bf16 *d = outpad + sh.ps(it.b, it.z, y, x, 0, 0, 0) * kNetC;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               float zv[8];
               unpack8_bf16(zw[c], zv);
 #pragma unroll
               for (int e = 0; e < 8; ++e) zv[e] = v[8 * c + e] * net_gelu_grad(zv[e]);
-              d[c] = pack8_bf16(zv);
+              zw[c] = pack8_bf16(zv);
             }
+            st_global32(d, zw[0], zw[1]);
+            st_global32(d + 16, zw[2], zw[3]);
           } else {
             float4 *d = reinterpret_cast<float4 *>(outraw + pu * kNetC);
 #pragma unroll

@@ -130,6 +130,20 @@ __device__ __forceinline__ void unpack8_bf16(const uint4 &u, float *v) {
   }
 }
 
+// 32 bytes of one lane in one access: a cell's 64 bytes of activations then
+// take two accesses of whole sectors instead of four of half sectors.
+__device__ __forceinline__ void st_global32(void *p, const uint4 &a, const uint4 &b) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y),
+               "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+               : "memory");
+}
+__device__ __forceinline__ void ld_global32(const void *p, uint4 &a, uint4 &b) {
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+               : "l"(p)
+               : "memory");
+}
+
 // Store one cell's 32 activations at its padded position and at the ghost
 // copies it stands for (replicate padding: a boundary cell is also its
 // outside neighbour).
@@ -157,9 +171,9 @@ __device__ __forceinline__ void store_replicated(bf16 *outpad, const NetShape &s
   for (int iz = 0; iz < nzs; ++iz)
     for (int iy = 0; iy < nys; ++iy)
       for (int ix = 0; ix < nxs; ++ix) {
-        uint4 *dst = reinterpret_cast<uint4 *>(outpad + sh.p(b, zs[iz], ys[iy], xs[ix]) * kNetC);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) dst[c] = w[c];
+        bf16 *dst = outpad + sh.p(b, zs[iz], ys[iy], xs[ix]) * kNetC;
+        st_global32(dst, w[0], w[1]);
+        st_global32(dst + 16, w[2], w[3]);
       }
 }
 
@@ -173,6 +187,42 @@ __device__ __forceinline__ float net_gelu_fast(float x) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
   return 0.5f * x * (1.0f + t);
 }
+// The same on two values with packed FP32 arithmetic (fma/mul.rn.f32x2: half
+// the issue slots).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t net_gelu_fast2(uint64_t x) {
+  const float k = 0.7978845608028654f;
+  const uint64_t u = mul2(x, fma2(pack2(k * 0.044715f, k * 0.044715f), mul2(x, x), pack2(k, k)));
+  float a, b;
+  unpack2(u, a, b);
+  asm("tanh.approx.f32 %0, %0;" : "+f"(a));
+  asm("tanh.approx.f32 %0, %0;" : "+f"(b));
+  const uint64_t h = mul2(x, pack2(0.5f, 0.5f));
+  return fma2(h, pack2(a, b), h);
+}
+
 // Its derivative for the backward passes, to FP32 accuracy.  With e = exp(-2u)
 // and s = 1 / (1 + e), tanh u = 2 s - 1 and 1 - tanh^2 u = 4 s (e s), so
 //   gelu'(x) = (1 + t) / 2 + x/2 (1 - t^2) u' = s + 2 x s (e s) u',
