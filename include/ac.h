@@ -48,7 +48,8 @@ enum {
 
 /* ------------------------------------------------------ storage types ---- */
 typedef enum {
-  AC_F64 = 0,  /* FP64 storage, FP64 arithmetic                        */
+  AC_F64 = 0,  /* FP64 storage, FP64 arithmetic (or 64-bit integer
+                  arithmetic of smaller error, see fixed64.cuh)          */
   AC_F32 = 1,  /* FP32 storage, FP32 arithmetic                        */
   AC_F16S = 2  /* FP16 storage (IEEE binary16), FP32 arithmetic; values
                   are rounded to nearest-even only when written to memory */
@@ -175,10 +176,10 @@ int ac_init_shape(ac_ctx *ctx, int32_t kind, double lower_x, double lower_y, dou
 /* Kernel variants selectable with ac_set_schedule. */
 enum {
   AC_VARIANT_AUTO = 0,    /* autotuned choice if ac_autotune ran, else default.
-                             2D FP32 / FP16 storage: while the choice is the
-                             default schedule and no tile is forced, its passes
-                             run on a register-tile kernel, several passes to a
-                             launch, with the same results bit for bit        */
+                             2D: while the choice is the default schedule and
+                             no tile is forced, its passes may run on a
+                             register-tile kernel, several passes to a launch,
+                             with the same results bit for bit                */
   AC_VARIANT_DIRECT = 1,  /* one step per launch, neighbours read from global
                              memory with clamped indices (k must be 1)         */
   AC_VARIANT_STREAM = 2   /* TMA-staged streaming kernel with temporal blocking:

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "ctx.h"
+#include "fixed64.cuh"
 
 using namespace ac;
 
@@ -397,23 +398,23 @@ bool ac_plan_depths(int64_t n, int k, std::vector<int> &depths) {
   return false;
 }
 
-// Whether a schedule runs on the register-tile kernel (block2d.cuh): the
-// default 2D schedule of FP32 / FP16 storage, unless the caller forced a
-// schedule or a strip width (those run the streaming kernel as asked).  Its
-// results are bit for bit those of the default schedule's passes: FP32 does
-// not depend on the depth, and FP16 storage is rounded where they end.
+// Whether a schedule may run on the register-tile kernels (block2d.cuh,
+// block2d_fx.cuh): the default 2D schedule, unless the caller forced a
+// schedule or a strip width (those run as asked).  The results are bit for bit
+// those of the default schedule's passes: FP32 and FP64 do not depend on the
+// depth, and FP16 storage is rounded where they end.
 static bool takes_block2d(const ac_ctx *c, int variant, int k, int tile) {
-  if (c->d.ndim != 2 || c->d.dtype == AC_F64 || c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO)
-    return false;
+  if (c->d.ndim != 2 || c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO) return false;
+  if (c->d.dtype == AC_F64 && !fx_coefficients(c->gp.alpha, c->gp.beta)) return false;
   int dv, dk;
   default_schedule(c, &dv, &dk);
   return variant == dv && k == dk && tile == default_tile(c, dk);
 }
 
-// n steps on the register-tile kernel; *done is false if it does not serve
-// the grid (nothing was launched).
+// n steps on the register-tile kernels; *done is false if none serves the
+// grid (nothing was launched).
 static int issue_block2d(ac_ctx *c, int64_t n, int k, bool *done) {
-  // FP16 storage: the passes whose ends round the field; FP32: single steps
+  // FP16 storage: the passes whose ends round the field; else single steps
   std::vector<int> passes;
   if (c->d.dtype == AC_F16S) ac_plan_depths(n, k, passes);
   const int64_t np = c->d.dtype == AC_F16S ? (int64_t)passes.size() : n;

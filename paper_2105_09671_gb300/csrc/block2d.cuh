@@ -9,7 +9,7 @@
 // Per step and row a warp issues two shuffles (the x neighbours across
 // lanes) and the update's 8 FP32 operations per cell; the rows above and
 // below a warp's own come through shared memory, one CTA barrier per step.
-// Boundary cells cost nothing: see reflect().  Beside the 8 operations that
+// Boundary cells cost nothing: see reflect() in common.cuh.  Beside the 8 operations that
 // is about 0.8 instructions per cell and step, against 3.9 (8-cell strips) to
 // 7.1 in the streaming kernel, and a step's latency is one tile step (0.17 us)
 // where a pass of the streaming kernel walks a chunk of rows one by one.
@@ -20,20 +20,6 @@
 #include "kernels.h"
 
 namespace ac {
-
-// Reflection of index i into [0, n): the zero-Neumann ghost of Section 2 is
-// the boundary cell itself, and a field extended by reflection about its
-// faces keeps that property at every step (cell -1-i stays equal to cell i:
-// both see the same neighbours in the other order, and the paired neighbour
-// sums commute bit for bit).  So a tile whose halo is loaded by reflection
-// needs no boundary handling while it steps.
-__device__ __forceinline__ int reflect(int i, int n) {
-  if (i >= 0 && i < n) return i;
-  const int p = 2 * n;
-  int m = i % p;
-  if (m < 0) m += p;
-  return m < n ? m : p - 1 - m;
-}
 
 constexpr int kB2MaxWarps = 16;
 constexpr int b2_smem_bytes(int E, int warps) { return 4 * warps * 32 * E * (int)sizeof(float); }

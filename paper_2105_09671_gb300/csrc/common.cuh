@@ -98,6 +98,20 @@ __device__ __forceinline__ void st_cells(T *p, const typename Traits<T>::C *in) 
   }
 }
 
+// Reflection of index i into [0, n): the zero-Neumann ghost of Section 2 is
+// the boundary cell itself, and a field extended by reflection about its
+// faces keeps that property at every step (cell -1-i stays equal to cell i:
+// both see the same neighbours in the other order, and the paired neighbour
+// sums commute bit for bit).  So a tile whose halo is loaded by reflection
+// needs no boundary handling while it steps.
+__device__ __forceinline__ int reflect(int i, int n) {
+  if (i >= 0 && i < n) return i;
+  const int p = 2 * n;
+  int m = i % p;
+  if (m < 0) m += p;
+  return m < n ? m : p - 1 - m;
+}
+
 // ------------------------------------------------------------ the update --
 // One explicit Euler step of Eq. (pytorchACeq) for one cell:
 //   phi' = phi + beta * (nsum - 2 d phi) + alpha * (phi - phi^3),

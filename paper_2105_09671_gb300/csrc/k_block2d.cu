@@ -1,6 +1,7 @@
 // Register-tile 2D stencil: kernel variants, the rule that picks one for a
 // grid, and the launch.
 #include "block2d.cuh"
+#include "block2d_fx.cuh"
 
 namespace ac {
 
@@ -26,11 +27,23 @@ constexpr B2Variant kB2[] = {
     {4, 7, 64, 1.65, 1.69, 0.057, 0.0402},
     {4, 8, 96, 1.50, 1.93, 0.086, 0.0473},
     {8, 8, 128, 2.90, 1.75, 0.246, 0.0928},
+    // FP64 (block2d_fx.cuh): two rows a lane for the smallest grids (200^2 1.42
+    // us a step against 1.66 with four), four from 512^2 on (3.56 against 4.14)
+    {1, 2, 32, 1.30, 1.37, 0.0, 0.0632},
+    {1, 4, 56, 2.09, 0.97, 0.629, 0.1161},
 };
 constexpr int kB2Count = sizeof(kB2) / sizeof(kB2[0]);
 
+// A step of the marching FP64 kernel (k_direct.cu) on GB300: 11.7, 32 and 116
+// us at 1024^2, 2048^2 and 4096^2.
+double march_cost(int64_t nx, int64_t ny) { return 3.5 + 6.7e-6 * (double)nx * (double)ny; }
+
+bool offered(const B2Variant &b, int dtype) {
+  return dtype == AC_F64 ? b.E == 1 : b.E == 4 || (b.E == 8 && dtype == AC_F16S);
+}
+
 int halo_x(int dtype, int E, int k) {
-  const int v = std::min(E, dtype == AC_F16S ? 8 : 4);  // whole memory vectors
+  const int v = std::min(E, dtype == AC_F16S ? 8 : 4);  // whole memory vectors (FP64: single cells)
   return (k + v - 1) / v * v;
 }
 
@@ -69,15 +82,39 @@ cudaError_t launch_t(const GridParams &g, const void *src, void *dst, int warps,
   return cudaLaunchKernelEx(&cfg, block2d_k<T, E, R, MINB>, (const T *)src, (T *)dst, g, k, hx, mask);
 }
 
+template <int R>
+cudaError_t launch_fx_t(const GridParams &g, const void *src, void *dst, int warps, int k, cudaStream_t s) {
+  static KernelSetup ks;
+  int occ = 1;
+  cudaError_t e = kernel_setup(ks, (const void *)block2d_fx_k<R>, kB2FxMaxWarps * 32,
+                               b2fx_smem_bytes(kB2FxMaxWarps), &occ);
+  if (e != cudaSuccess) return e;
+  const int ow = 32 - 2 * k, oh = warps * R - 2 * k;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((g.nx + ow - 1) / ow), (unsigned)((g.ny + oh - 1) / oh));
+  cfg.blockDim = dim3(warps * 32);
+  cfg.dynamicSmemBytes = b2fx_smem_bytes(warps);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, block2d_fx_k<R>, (const double *)src, (double *)dst, g, k);
+}
+
 }  // namespace
 
 bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, int num_sms, Block2DPlan *out) {
-  if (dtype == AC_F64 || passes < 1) return false;
-  double best = 1e300;
+  if (passes < 1) return false;
+  // FP64: against one step a launch
+  double best = dtype == AC_F64 ? (double)passes * march_cost(nx, ny) : 1e300;
+  bool found = false;
   for (int v = 0; v < kB2Count; ++v) {
-    if (kB2[v].E == 8 && dtype != AC_F16S) continue;
+    if (!offered(kB2[v], dtype)) continue;
     for (int warps = 4; warps <= kB2MaxWarps; warps += 4)
-      for (int kmax = 4; kmax <= kB2MaxDepth; kmax += 4) {
+      for (int kmax = dtype == AC_F64 ? 2 : 4; kmax <= (dtype == AC_F64 ? 8 : kB2MaxDepth);
+           kmax += dtype == AC_F64 ? 1 : 4) {
         const int per = kmax / depth;  // passes per launch
         if (per < 1 || warps * kB2[v].R - 2 * per * depth < 4) continue;
         int64_t launches = (passes + per - 1) / per;
@@ -88,11 +125,12 @@ bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, 
         const double cost = (double)launches * launch_cost(kB2[v], dtype, nx, ny, warps, k, num_sms);
         if (cost < best) {
           best = cost;
+          found = true;
           *out = Block2DPlan{v, warps, launches};
         }
       }
   }
-  return best < 1e300;
+  return found;
 }
 
 cudaError_t launch_block2d(int dtype, const Block2DPlan &p, const GridParams &g, const void *src, void *dst,
@@ -102,6 +140,11 @@ cudaError_t launch_block2d(int dtype, const Block2DPlan &p, const GridParams &g,
       case 0: return launch_t<float, 4, 4, 1>(g, src, dst, p.warps, k, 0u, s);
       case 1: return launch_t<float, 4, 7, 2>(g, src, dst, p.warps, k, 0u, s);
       case 2: return launch_t<float, 4, 8, 1>(g, src, dst, p.warps, k, 0u, s);
+    }
+  } else if (dtype == AC_F64) {
+    switch (p.variant) {
+      case 4: return launch_fx_t<2>(g, src, dst, p.warps, k, s);
+      case 5: return launch_fx_t<4>(g, src, dst, p.warps, k, s);
     }
   } else if (dtype == AC_F16S) {
     switch (p.variant) {

@@ -3,6 +3,11 @@
 // the domain, which realises the zero-Neumann ghost copy of Section 2
 // (the ghost equals its adjacent interior cell).  This is the plain variant
 // the streaming kernels are checked and timed against.
+//
+// Larger FP64 grids march: a value is taken apart for the integer form of the
+// update (fixed64.cuh) once per lane and shared by warp shuffles (x) and
+// registers (y, z) while a warp walks a chunk of rows or planes.
+#include "fixed64.cuh"
 #include "kernels.h"
 
 namespace ac {
@@ -17,8 +22,7 @@ __device__ __forceinline__ void step2d_cell(const T *__restrict__ src, T *__rest
   C p = to_c(row[i]);
   C w = to_c(row[im]), e = to_c(row[ip]);
   C s = to_c(src[jm * g.pitch + i]), n = to_c(src[jp * g.pitch + i]);
-  C nsum = (w + e) + (s + n);
-  dst[j * g.pitch + i] = from_c<T>(ac_update<C>(p, nsum, C(-4), C(g.alpha), C(g.beta)));
+  dst[j * g.pitch + i] = from_c<T>(cell_update2<C>(p, w, e, s, n, Coef<C>(g.alpha, g.beta)));
 }
 
 template <typename T>
@@ -34,8 +38,7 @@ __device__ __forceinline__ void step3d_cell(const T *__restrict__ src, T *__rest
   C w = to_c(row[im]), e = to_c(row[ip]);
   C s = to_c(src[k * plane + jm * g.pitch + i]), n = to_c(src[k * plane + jp * g.pitch + i]);
   C b = to_c(src[km * plane + j * g.pitch + i]), f = to_c(src[kp * plane + j * g.pitch + i]);
-  C nsum = ((w + e) + (s + n)) + (b + f);
-  dst[k * plane + j * g.pitch + i] = from_c<T>(ac_update<C>(p, nsum, C(-6), C(g.alpha), C(g.beta)));
+  dst[k * plane + j * g.pitch + i] = from_c<T>(cell_update3<C>(p, w, e, s, n, b, f, Coef<C>(g.alpha, g.beta)));
 }
 
 // one thread per x; y and z as for_cell_yz (see cell_grid)
@@ -53,6 +56,205 @@ __global__ void __launch_bounds__(256) step3d_direct(const T *__restrict__ src,
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= g.nx) return;
   for_cell_yz<TALL>(g, [&](int64_t j, int64_t k) { step3d_cell(src, dst, g, i, j, k); });
+}
+
+// -------------------------------------------------- FP64, integer form --
+constexpr int64_t kFxMarchCells = 512 * 512;
+constexpr int kFxWarps = 4;                      // per CTA, independent of one another
+constexpr int kFx2E = 4, kFx2W = 32 * kFx2E;      // 2D: cells a lane, columns a warp
+constexpr int kFx3E = 2, kFx3W = 32 * kFx3E;      // 3D
+constexpr int kFx3R = 2;                         // 3D: rows a warp writes per plane
+constexpr int kFxHalo = 2;                       // halo columns per side (one 16-byte vector)
+
+// One row's cells of a lane: E cells from column xl, or from the reflected
+// columns xi where the strip leaves the grid.
+template <int E>
+__device__ __forceinline__ void fx_load(const double *row, int xl, const int *xi, bool inside, double *v) {
+  if (inside) {
+#pragma unroll
+    for (int q = 0; q < E; q += 2) {
+      const double2 d = *reinterpret_cast<const double2 *>(row + xl + q);
+      v[q] = d.x;
+      v[q + 1] = d.y;
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = row[xi[e]];
+  }
+}
+// Store of the cells that are outputs of the strip (columns kFxHalo .. W - kFxHalo) and in the grid.
+template <int E>
+__device__ __forceinline__ void fx_store(double *row, int xl, int lane, int nx, const double *v) {
+#pragma unroll
+  for (int q = 0; q < E; q += 2) {
+    const int c = lane * E + q, x = xl + q;
+    if (c < kFxHalo || c >= 32 * E - kFxHalo || x >= nx) continue;
+    if (x + 1 < nx) *reinterpret_cast<double2 *>(row + x) = make_double2(v[q], v[q + 1]);
+    else row[x] = v[q];
+  }
+}
+
+// A warp owns kFx2W columns and marches over `chunk` rows.  Bound by integer
+// issue (some 140 instructions a cell, 14 of them wide multiply-adds): 4096^2
+// 253 -> 116 us a step, 2048^2 64 -> 32 against the FP64 operations.
+__global__ void __launch_bounds__(kFxWarps * 32) step2d_fx(const double *__restrict__ src,
+                                                           double *__restrict__ dst, GridParams g, int strips,
+                                                           int chunk) {
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = (int64_t)blockIdx.x * kFxWarps + (threadIdx.x >> 5);
+  const int nx = (int)g.nx, ny = (int)g.ny;
+  const int x0 = (int)(gw % strips) * (kFx2W - 2 * kFxHalo) - kFxHalo, xl = x0 + lane * kFx2E;
+  const int64_t ys = gw / strips * chunk;
+  if (ys >= ny) return;
+  const int ya = (int)ys, ye = min(ny, ya + chunk);
+  const bool inside = x0 >= 0 && x0 + kFx2W <= nx;
+  int xi[kFx2E];
+#pragma unroll
+  for (int e = 0; e < kFx2E; ++e) xi[e] = reflect(xl + e, nx);
+  const Coef<double> coef(g.alpha, g.beta);
+  double v[kFx2E];
+  FxV below[kFx2E], x[kFx2E];  // the row below, the row
+  fx_load<kFx2E>(src + (int64_t)reflect(ya - 1, ny) * g.pitch, xl, xi, inside, v);
+#pragma unroll
+  for (int e = 0; e < kFx2E; ++e) below[e] = fx_in(v[e]);
+  fx_load<kFx2E>(src + (int64_t)ya * g.pitch, xl, xi, inside, v);
+#pragma unroll
+  for (int e = 0; e < kFx2E; ++e) x[e] = fx_in(v[e]);
+  fx_load<kFx2E>(src + (int64_t)reflect(ya + 1, ny) * g.pitch, xl, xi, inside, v);
+  for (int y = ya; y < ye; ++y) {
+    FxV up[kFx2E];
+#pragma unroll
+    for (int e = 0; e < kFx2E; ++e) up[e] = fx_in(v[e]);
+    if (y + 1 < ye)  // the row after next, ahead of its use
+      fx_load<kFx2E>(src + (int64_t)reflect(y + 2, ny) * g.pitch, xl, xi, inside, v);
+    const FxV left = fx_shfl<-1>(x[kFx2E - 1]), right = fx_shfl<1>(x[0]);
+    double out[kFx2E];
+#pragma unroll
+    for (int e = 0; e < kFx2E; ++e) {
+      const FxV &w = e == 0 ? left : x[e - 1], &ea = e == kFx2E - 1 ? right : x[e + 1];
+      const int m = max(max(max(w.e, ea.e), max(below[e].e, up[e].e)), x[e].e);
+      if (fx_in_range(m)) {
+        const int64_t ns =
+            (fx_align(w, m) + fx_align(ea, m)) + (fx_align(below[e], m) + fx_align(up[e], m));
+        out[e] = fx_update<2>(x[e], ns, m, coef);
+      } else {
+        // the FP64 operations, from memory
+        const int im = xi[e] > 0 ? xi[e] - 1 : 0, ip = min(xi[e] + 1, nx - 1);
+        const double *row = src + (int64_t)y * g.pitch;
+        out[e] = ac_update<double>(row[xi[e]],
+                                   (row[im] + row[ip]) + (src[(int64_t)max(y - 1, 0) * g.pitch + xi[e]] +
+                                                          src[(int64_t)min(y + 1, ny - 1) * g.pitch + xi[e]]),
+                                   -4.0, coef.alpha, coef.beta);
+      }
+    }
+    fx_store<kFx2E>(dst + (int64_t)y * g.pitch, xl, lane, nx, out);
+#pragma unroll
+    for (int e = 0; e < kFx2E; ++e) {
+      below[e] = x[e];
+      x[e] = up[e];
+    }
+  }
+}
+
+// A warp owns kFx3W columns of kFx3R rows and marches over `chunk` planes; it
+// takes apart kFx3R + 2 rows of each plane (against a barrier a plane to share
+// them; two rows in 124 registers rather than three or four in 160).  256^3
+// 317 -> 228 us a step, 200 x 100 x 100 45 -> 26.
+__global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restrict__ src,
+                                                           double *__restrict__ dst, GridParams g, int strips,
+                                                           int bands, int chunk) {
+  constexpr int R = kFx3R, E = kFx3E;
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = (int64_t)blockIdx.x * kFxWarps + (threadIdx.x >> 5);
+  const int nx = (int)g.nx, ny = (int)g.ny, nz = (int)g.nz;
+  const int x0 = (int)(gw % strips) * (kFx3W - 2 * kFxHalo) - kFxHalo, xl = x0 + lane * E;
+  const int y0 = (int)(gw / strips % bands) * R;
+  const int64_t zs = gw / strips / bands * chunk;
+  if (zs >= nz) return;
+  const int za = (int)zs, ze = min(nz, za + chunk);
+  const int64_t plane = g.pitch * g.ny;
+  const bool inside = x0 >= 0 && x0 + kFx3W <= nx;
+  int xi[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) xi[e] = reflect(xl + e, nx);
+  int64_t ro[R + 2];
+#pragma unroll
+  for (int r = 0; r < R + 2; ++r) ro[r] = (int64_t)reflect(y0 - 1 + r, ny) * g.pitch;
+  const Coef<double> coef(g.alpha, g.beta);
+  FxV below[R][E], x[R + 2][E];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    double v[E];
+    fx_load<E>(src + (int64_t)reflect(za - 1, nz) * plane + ro[r + 1], xl, xi, inside, v);
+#pragma unroll
+    for (int e = 0; e < E; ++e) below[r][e] = fx_in(v[e]);
+  }
+#pragma unroll
+  for (int r = 0; r < R + 2; ++r) {
+    double v[E];
+    fx_load<E>(src + (int64_t)za * plane + ro[r], xl, xi, inside, v);
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[r][e] = fx_in(v[e]);
+  }
+  for (int z = za; z < ze; ++z) {
+    FxV up[R + 2][E];
+    const double *zp = src + (int64_t)reflect(z + 1, nz) * plane;
+#pragma unroll
+    for (int r = 0; r < R + 2; ++r) {
+      double v[E];
+      fx_load<E>(zp + ro[r], xl, xi, inside, v);
+#pragma unroll
+      for (int e = 0; e < E; ++e) up[r][e] = fx_in(v[e]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const FxV left = fx_shfl<-1>(x[r + 1][E - 1]), right = fx_shfl<1>(x[r + 1][0]);
+      double out[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const FxV &p = x[r + 1][e], &w = e == 0 ? left : x[r + 1][e - 1],
+                  &ea = e == E - 1 ? right : x[r + 1][e + 1];
+        const FxV &s = x[r][e], &n = x[r + 2][e], &lo = below[r][e], &hi = up[r + 1][e];
+        const int m = max(max(max(max(w.e, ea.e), max(s.e, n.e)), max(lo.e, hi.e)), p.e);
+        if (fx_in_range(m)) {
+          const int64_t ns = ((fx_align(w, m) + fx_align(ea, m)) + (fx_align(s, m) + fx_align(n, m))) +
+                             (fx_align(lo, m) + fx_align(hi, m));
+          out[e] = fx_update<3>(p, ns, m, coef);
+        } else {
+          const int im = xi[e] > 0 ? xi[e] - 1 : 0, ip = min(xi[e] + 1, nx - 1);
+          const double *pl = src + (int64_t)z * plane, *row = pl + ro[r + 1];
+          out[e] = ac_update<double>(
+              row[xi[e]],
+              ((row[im] + row[ip]) + (pl[ro[r] + xi[e]] + pl[ro[r + 2] + xi[e]])) +
+                  (src[(int64_t)max(z - 1, 0) * plane + ro[r + 1] + xi[e]] + zp[ro[r + 1] + xi[e]]),
+              -6.0, coef.alpha, coef.beta);
+        }
+        below[r][e] = p;
+      }
+      if (y0 + r < ny) fx_store<E>(dst + (int64_t)z * plane + (int64_t)(y0 + r) * g.pitch, xl, lane, nx, out);
+    }
+#pragma unroll
+    for (int r = 0; r < R + 2; ++r)
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[r][e] = up[r][e];
+  }
+}
+
+static cudaError_t direct_fx(int ndim, const GridParams &g, const double *src, double *dst, cudaStream_t s) {
+  // chunks of rows (planes) that give every SM about 16 warps (each chunk
+  // converts two more rows than it writes, so no shorter ones)
+  const int64_t kFxTarget = 152 * (ndim == 2 ? 24 : 16), kMin = 1;
+  const int w = ndim == 2 ? kFx2W : kFx3W;
+  const int64_t strips = (g.nx + w - 2 * kFxHalo - 1) / (w - 2 * kFxHalo);
+  const int64_t bands = ndim == 2 ? 1 : (g.ny + kFx3R - 1) / kFx3R;
+  const int64_t len = ndim == 2 ? g.ny : g.nz;
+  const int64_t chunks = std::max<int64_t>(1, std::min(kFxTarget / std::max<int64_t>(1, strips * bands), len / kMin));
+  const int64_t chunk = (len + chunks - 1) / chunks;
+  const int64_t warps = strips * bands * ((len + chunk - 1) / chunk);
+  const unsigned blocks = (unsigned)((warps + kFxWarps - 1) / kFxWarps);
+  if (ndim == 2) step2d_fx<<<blocks, kFxWarps * 32, 0, s>>>(src, dst, g, (int)strips, (int)chunk);
+  else step3d_fx<<<blocks, kFxWarps * 32, 0, s>>>(src, dst, g, (int)strips, (int)bands, (int)chunk);
+  return cudaGetLastError();
 }
 
 template <typename T>
@@ -73,7 +275,12 @@ static cudaError_t direct_t(int ndim, const GridParams &g, const void *src, void
 cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *src, void *dst,
                           cudaStream_t s) {
   switch (dtype) {
-    case AC_F64: return direct_t<double>(ndim, g, src, dst, s);
+    case AC_F64:
+      // below that many cells a march's few warps wait for one row after
+      // another: one thread a cell (64^2 1.9 us a step against 3.5)
+      if (fx_coefficients(g.alpha, g.beta) && g.nx * g.ny * g.nz >= kFxMarchCells)
+        return direct_fx(ndim, g, (const double *)src, (double *)dst, s);
+      return direct_t<double>(ndim, g, src, dst, s);
     case AC_F32: return direct_t<float>(ndim, g, src, dst, s);
     case AC_F16S: return direct_t<__half>(ndim, g, src, dst, s);
   }

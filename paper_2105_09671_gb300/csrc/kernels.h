@@ -67,10 +67,11 @@ cudaError_t launch_stream2d(int dtype, int k, int tile, const GridParams &g, con
 cudaError_t launch_stream3d(int dtype, int k, int tile, const GridParams &g,
                             const CUtensorMap *src_map, void *dst, int num_sms, cudaStream_t s);
 
-// Register-tile 2D stencil (FP32 / FP16 storage): launches of up to
+// Register-tile 2D stencils: launches of up to
 // kB2MaxDepth steps.  A plan covers `passes` passes of at most `depth` steps
 // each, spread evenly over plan.launches launches (an even count unless there
-// is a single pass); false if no variant serves the grid.
+// is a single pass); false if no variant serves the grid (FP64: if one step a
+// launch is faster).
 constexpr int kB2MaxDepth = 16;
 struct Block2DPlan {
   int variant, warps;

@@ -26,6 +26,7 @@
 
 #include <algorithm>
 
+#include "fixed64.cuh"
 #include "kernels.h"
 
 namespace ac {
@@ -73,8 +74,8 @@ struct S2Item {
 template <typename T, int K, bool FASTX, int VPL_ = S2Cfg<T>::VPL>
 __device__ __forceinline__ bool s2_item(T *ring_smem, uint64_t *bars, uint32_t &u,
                                         const CUtensorMap *src_map, T *__restrict__ dst,
-                                        const S2Item &it, typename Traits<T>::C alpha,
-                                        typename Traits<T>::C beta, int *status) {
+                                        const S2Item &it, const Coef<typename Traits<T>::C> &coef,
+                                        int *status) {
   using Gm = S2Geom<T, K, VPL_>;
   using C = typename Traits<T>::C;
   constexpr int E = Gm::E, V = Gm::V, VPL = Gm::VPL, D = kS2Stages;
@@ -181,7 +182,7 @@ __device__ __forceinline__ bool s2_item(T *ring_smem, uint64_t *bars, uint32_t &
             if (e == eR) ea = p;
           }
         }
-        out[e] = ac_update<C>(p, (w + ea) + (ring[l][SA][e] + ring[l][SN][e]), C(-4), alpha, beta);
+        out[e] = cell_update2<C>(p, w, ea, ring[l][SA][e], ring[l][SN][e], coef);
       }
       if (l + 1 < K) {
 #pragma unroll
@@ -288,7 +289,8 @@ __global__ void __launch_bounds__(kS2Warps * 32, 1)
   }
   __syncwarp();
   uint32_t u = 0;
-  s2_item<T, K, FASTX, VPL_>(ring.smem, ring.bars, u, &src_map, dst, it, (C)g.alpha, (C)g.beta, g.status);
+  s2_item<T, K, FASTX, VPL_>(ring.smem, ring.bars, u, &src_map, dst, it, Coef<C>(g.alpha, g.beta),
+                             g.status);
 }
 
 // ------------------------------------------------------------------ host ---

@@ -43,6 +43,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "fixed64.cuh"
 #include "kernels.h"
 
 namespace ac {
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(S3Geom<T, K, TILE>::NT, S3Geom<T, K, TILE>::MI
   const int r0 = R * qg;
   const int nx = (int)g.nx, ny = (int)g.ny, nz = (int)g.nz;
   const int64_t plane_stride = g.pitch * g.ny;
-  const C alpha = (C)g.alpha, beta = (C)g.beta;
+  const Coef<C> coef(g.alpha, g.beta);
   const bool esm = lsm || rsm;
 
   // Level l keeps its last three planes in a ring of register slots: at
@@ -450,8 +451,7 @@ __global__ void __launch_bounds__(S3Geom<T, K, TILE>::NT, S3Geom<T, K, TILE>::MI
               sv = sself ? p : sv;
               nv = nself ? p : nv;
             }
-            const C nsum = ((w + ea) + (sv + nv)) + (ring[l][SA][i][e] + ring[l][SN][i][e]);
-            out[e] = ac_update<C>(p, nsum, C(-6), alpha, beta);
+            out[e] = cell_update3<C>(p, w, ea, sv, nv, ring[l][SA][i][e], ring[l][SN][i][e], coef);
           }
           if (l + 1 < K) {
 #pragma unroll
