@@ -8,13 +8,12 @@
 // channels contiguous, pixels strided), so staging is TMA copies only.
 //
 // Work item: two rows of g by 128 pixels (one z, one image) and the four
-// padded rows of a that the taps of one dz reach from them.  A stage holds,
-// per block of 8 channels, 4 rows x 130 pixels of a and 2 rows x 128 pixels
-// of g at 16 bytes a pixel.  With the MN groups (8 channels of one row) a
-// constant distance apart,
-//   A = a: M = 128 = (channel block, a row 0..3, channel), K = 16 pixels,
-//   B = g: N = 64 = (channel block, g row 0..1, channel),
-// and the x offset of a tap is +16 bytes on A's start address, so a stage is
+// padded rows of a that the taps of one dz reach from them.  A stage holds 4
+// rows x 130 pixels of a and 2 rows x 128 pixels of g, 64 bytes (32 channels)
+// a pixel in the 64-byte swizzle, one TMA box each:
+//   A = a: M = 128 = (a row 0..3, channel), K = 16 pixels,
+//   B = g: N = 64 = (g row 0..1, channel),
+// and the x offset of a tap is +64 bytes on A's start address, so a stage is
 // 3 (ox) x 8 (k) MMAs into 3 TMEM accumulators that live for the whole CTA.
 // Of the 4 x 2 (a row, g row) pairs 6 are taps (oy = a row - g row - 1), the
 // other two are dropped.  In 3D blockIdx.y is the tap's dz.
@@ -38,16 +37,15 @@ namespace ac {
 namespace {
 
 constexpr int kWgPix = 128;                         // pixels of g per row of an item
-constexpr int kWgRowA = (kWgPix + 2) * 16;          // bytes: one row of one 8-channel block of a
-constexpr int kWgRowG = kWgPix * 16;                // the same of g
-constexpr int kWgBoxA = 4 * kWgRowA, kWgBoxG = 2 * kWgRowG;
-constexpr int kWgStageG = 4 * kWgBoxA;              // offset of g in a stage
-constexpr int kWgStage = 4 * kWgBoxA + 4 * kWgBoxG;
+constexpr int kWgRowA = (kWgPix + 2) * 64;          // bytes: one row of a
+constexpr int kWgRowG = kWgPix * 64;                // one row of g
+constexpr int kWgStageG = 4 * kWgRowA;              // offset of g in a stage
+constexpr int kWgStage = 4 * kWgRowA + 2 * kWgRowG;
 constexpr int kWgStages = 4;
 constexpr int kWgThreads = 128;
 constexpr int kWgTmem = 256;                        // 3 accumulators of 64 columns
 constexpr int kWgSmem = kWgStages * kWgStage + (2 * kWgStages + 1) * 8 + 8;
-static_assert(kWgBoxA % 128 == 0 && kWgBoxG % 128 == 0, "TMA destination alignment");
+static_assert(kWgStageG % 512 == 0 && kWgStage % 512 == 0, "the swizzle pattern repeats every 512 bytes");
 static_assert(kWgSmem <= 227 * 1024, "shared memory");
 
 // kind::f16, BF16 x BF16 -> FP32, M = 128, N = 64, both operands MN-major
@@ -74,7 +72,7 @@ template <int NDIM>
 __global__ void __launch_bounds__(kWgThreads, 1)
     net_wgrad_rows_k(const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap g_map,
                      NetShape sh, float *__restrict__ gw, float *__restrict__ gb, int *status) {
-  extern __shared__ __align__(128) unsigned char sm[];
+  extern __shared__ __align__(1024) unsigned char sm[];
   uint64_t *full = reinterpret_cast<uint64_t *>(sm + kWgStages * kWgStage);
   uint64_t *empty = full + kWgStages;
   uint64_t *fin = empty + kWgStages;
@@ -123,10 +121,8 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         const int64_t row0 = ((int64_t)it.b * sh.pz()) * sh.py() + it.y;
         const int ra = (int)(row0 + (NDIM == 3 ? (int64_t)(it.z + dz) * sh.py() : 0));
         const int rg = (int)(row0 + 1 + (NDIM == 3 ? (int64_t)(it.z + 1) * sh.py() : 0));
-        for (int c = 0; c < 4; ++c) {
-          tma_load_3d(st + c * kWgBoxA, &a_map, &full[s], c * 8, it.x0, ra);
-          tma_load_3d(st + kWgStageG + c * kWgBoxG, &g_map, &full[s], c * 8, it.x0 + 1, rg);
-        }
+        tma_load_3d(st, &a_map, &full[s], 0, it.x0, ra);
+        tma_load_3d(st + kWgStageG, &g_map, &full[s], 0, it.x0 + 1, rg);
       }
       if (!ok && !abort_flag) {
         report_timeout(status);
@@ -146,16 +142,16 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         if (!ok || abort_flag) { ok = false; break; }
         tc_fence_after();
         unsigned char *st = sm + s * kWgStage;
-        // MN-major without swizzle: 8 x 8 blocks of (8 pixels, 8 channels at
-        // 16 bytes a pixel); LBO between blocks along the pixels (128 bytes),
-        // SBO between MN groups
-        const uint64_t da = tc_smem_desc(st, 128, kWgRowA), db = tc_smem_desc(st + kWgStageG, 128, kWgRowG);
+        // MN-major in the 64-byte swizzle: LBO between blocks of 32 channels
+        // (rows), SBO between groups of 8 pixels
+        const uint64_t da = tc_smem_desc_sw64(st, kWgRowA, 512);
+        const uint64_t db = tc_smem_desc_sw64(st + kWgStageG, kWgRowG, 512);
 #pragma unroll
         for (int kk = 0; kk < kWgPix / 16; ++kk)
 #pragma unroll
           for (int ox = 0; ox < 3; ++ox)
-            tc_mma_bf16(tmem + ox * 64, da + (uint32_t)((kk * 256 + ox * 16) >> 4),
-                        db + (uint32_t)((kk * 256) >> 4), kWgIdesc, i > 0 || kk > 0);
+            tc_mma_bf16(tmem + ox * 64, da + (uint32_t)((kk * 1024 + ox * 64) >> 4),
+                        db + (uint32_t)((kk * 1024) >> 4), kWgIdesc, i > 0 || kk > 0);
         tc_commit(&empty[s]);
       }
       if (!ok && !abort_flag) {
@@ -181,13 +177,14 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         break;
       }
       if (sums) {
-        const unsigned char *gr = sm + s * kWgStage + kWgStageG + (warp - 2) * kWgRowG + lane * 16;
+        const unsigned char *gr = sm + s * kWgStage + kWgStageG + (warp - 2) * kWgRowG + lane * 64;
+        const int sw = (lane >> 1) & 3;  // the swizzle of this lane's pixels
 #pragma unroll
         for (int c = 0; c < 4; ++c)
 #pragma unroll
           for (int m = 0; m < kWgPix / 32; ++m) {
             float v[8];
-            unpack8_bf16(*reinterpret_cast<const uint4 *>(gr + c * kWgBoxG + m * 512), v);
+            unpack8_bf16(*reinterpret_cast<const uint4 *>(gr + m * 2048 + ((c ^ sw) << 4)), v);
 #pragma unroll
             for (int e = 0; e < 8; ++e) bias[c * 8 + e] += v[e];
           }
@@ -214,24 +211,19 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   __syncwarp();
   tc_fence_after();
   if (any && done) {
-    // accumulator lane (channel block warp, a row, channel) and column
-    // (channel block, g row, channel) -> tap and channels
-    const int ar = lane >> 3, ci = warp * 8 + (lane & 7);
+    // accumulator lane: a row = warp, channel = lane; column: g row, channel
 #pragma unroll
     for (int ox = 0; ox < 3; ++ox)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
+        const int oy = warp - h;
+        if (oy < 0 || oy > 2) continue;
         float v[32];
         tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + ox * 64 + h * 32, v);
+        float4 *d = reinterpret_cast<float4 *>(gw + ((int64_t)(dz * 9 + oy * 3 + ox) * kNetC + lane) * kNetC);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {  // 8 output channels of one g row
-          const int oy = ar - (q & 1), co = (h * 2 + (q >> 1)) * 8;
-          if (oy < 0 || oy > 2) continue;
-          const int t = dz * 9 + oy * 3 + ox;
-          float4 *d = reinterpret_cast<float4 *>(gw + ((int64_t)t * kNetC + ci) * kNetC + co);
-          atomicAdd(d, make_float4(v[q * 8], v[q * 8 + 1], v[q * 8 + 2], v[q * 8 + 3]));
-          atomicAdd(d + 1, make_float4(v[q * 8 + 4], v[q * 8 + 5], v[q * 8 + 6], v[q * 8 + 7]));
-        }
+        for (int q = 0; q < 8; ++q)
+          atomicAdd(d + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
       }
   }
   tc_fence_before();
@@ -258,9 +250,9 @@ static cudaError_t wgrad_t(const bf16 *apad, const bf16 *gpad, const NetShape &s
   const cuuint32_t es[3] = {1, 1, 1};
   CUtensorMap maps[2];
   for (int w = 0; w < 2; ++w) {
-    const cuuint32_t box[3] = {8, (cuuint32_t)(w ? kWgPix : kWgPix + 2), (cuuint32_t)(w ? 2 : 4)};
+    const cuuint32_t box[3] = {(cuuint32_t)kNetC, (cuuint32_t)(w ? kWgPix : kWgPix + 2), (cuuint32_t)(w ? 2 : 4)};
     if (fn(&maps[w], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16 *>(w ? gpad : apad), dims, strides,
-           box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+           box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
   }
