@@ -222,7 +222,7 @@ extern "C" int ac_create(const ac_grid_desc *desc, void *phi_dev, void *workspac
   c->gp.alpha = desc->dt / (desc->eps * desc->eps);
   c->gp.beta = desc->dt / (desc->h * desc->h);
   cudaError_t e = cudaMalloc(&c->d_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_partials, sizeof(double) * 4 * kReduceBlocks);
+  if (e == cudaSuccess) e = observe_alloc(&c->d_partials, c->stream);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_out, sizeof(double) * 4);
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_out, sizeof(double) * 4);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
@@ -520,10 +520,10 @@ extern "C" int ac_step(ac_ctx *c, int64_t n) {
 
 // ----------------------------------------------------------- reductions ---
 static int observe(ac_ctx *c, double out[4]) {
-  cudaError_t e = launch_observe(c->d.dtype, c->gp, c->phi, c->d_partials, c->d_out, c->stream);
+  // (the kernel writes the pinned host words itself: no copy to wait for)
+  cudaError_t e = launch_observe(c->d.dtype, c->gp, c->phi, c->d_partials, c->h_out, c->stream);
   if (e != cudaSuccess) return fail(AC_ERR_CUDA, "reduction launch failed: %s", cudaGetErrorString(e));
-  c->launches += 2;
-  AC_CUDA(cudaMemcpyAsync(c->h_out, c->d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  ++c->launches;
   AC_CUDA(cudaStreamSynchronize(c->stream));
   memcpy(out, c->h_out, 4 * sizeof(double));
   return AC_OK;

@@ -60,7 +60,7 @@ struct ac_batch {
   int *d_progress = nullptr;
   unsigned long long *d_ticket = nullptr;
   int *d_status = nullptr;
-  double *d_partials = nullptr, *d_out = nullptr, *h_out = nullptr;
+  double *d_partials = nullptr, *h_out = nullptr;
   long long total_tickets = 0;
   uint32_t wait_limit = kDefaultWaitPolls;
   int64_t launches = 0;
@@ -222,8 +222,7 @@ extern "C" int ac_batch_create(const ac_grid_desc *descs, void *const *phi_devs,
     if (e == cudaSuccess) e = cudaMalloc(&b->d_ticket, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(b->d_status, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_partials, sizeof(double) * 4 * kReduceBlocks);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_out, sizeof(double) * 4);
+    if (e == cudaSuccess) e = observe_alloc(&b->d_partials, b->stream);
     if (e == cudaSuccess) e = cudaMallocHost(&b->h_out, sizeof(double) * 4);
     if (e != cudaSuccess) rc = bfail(AC_ERR_NOMEM, "internal allocation failed: %s", cudaGetErrorString(e));
   }
@@ -231,7 +230,7 @@ extern "C" int ac_batch_create(const ac_grid_desc *descs, void *const *phi_devs,
   if (rc != AC_OK) {
     cudaGetLastError();
     cudaFree(b->d_maps); cudaFree(b->d_maps_wide); cudaFree(b->d_inst); cudaFree(b->d_ticket); cudaFree(b->d_status);
-    cudaFree(b->d_partials); cudaFree(b->d_out); cudaFreeHost(b->h_out);
+    cudaFree(b->d_partials); cudaFreeHost(b->h_out);
     delete b;
     return rc;
   }
@@ -245,7 +244,7 @@ extern "C" int ac_batch_destroy(ac_batch *b) {
   release_graph(b);
   release_items(b);
   cudaFree(b->d_maps); cudaFree(b->d_maps_wide); cudaFree(b->d_inst); cudaFree(b->d_ticket); cudaFree(b->d_status);
-  cudaFree(b->d_partials); cudaFree(b->d_out); cudaFreeHost(b->h_out);
+  cudaFree(b->d_partials); cudaFreeHost(b->h_out);
   delete b;
   return AC_OK;
 }
@@ -384,10 +383,9 @@ extern "C" int ac_batch_observe(ac_batch *b, int32_t i, double out[3]) {
   GridParams g;
   g.nx = d.nx; g.ny = d.ny; g.nz = d.nz; g.pitch = d.pitch_x;
   g.alpha = b->h_inst[i].alpha; g.beta = b->h_inst[i].beta; g.status = nullptr;
-  cudaError_t e = launch_observe(b->dtype, g, b->phi[i], b->d_partials, b->d_out, b->stream);
+  cudaError_t e = launch_observe(b->dtype, g, b->phi[i], b->d_partials, b->h_out, b->stream);
   if (e != cudaSuccess) return bfail(AC_ERR_CUDA, "reduction launch failed: %s", cudaGetErrorString(e));
-  b->launches += 2;
-  BC_CUDA(cudaMemcpyAsync(b->h_out, b->d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+  ++b->launches;
   BC_CUDA(cudaStreamSynchronize(b->stream));
   const double hd = d.h * d.h;
   out[0] = hd * (b->h_out[0] / (d.eps * d.eps) + 0.5 * b->h_out[1] / (d.h * d.h));

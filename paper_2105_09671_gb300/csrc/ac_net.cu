@@ -453,7 +453,7 @@ extern "C" int ac_learned_advance(ac_ctx *c, ac_net *net, int64_t jumps, const a
     if (use_spot)
       NC_CUDA(cudaMemcpyAsync(hr + 6, net->spot_out, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     NC_CUDA(cudaStreamSynchronize(c->stream));
-    c->launches += 3 + (use_spot ? 2 : 0);
+    c->launches += 2 + (use_spot ? 2 : 0);
     unsigned int gw[2];
     memcpy(gw, hr, sizeof gw);
     float mabs, mres;

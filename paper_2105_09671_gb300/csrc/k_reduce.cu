@@ -15,9 +15,9 @@
 // keep ~46 bits, and each lane adds its terms in float-float over groups of
 // kFFGroup cells before the group's sum is added in FP64 (relative error of
 // the sums ~1e-15, against the FP64 oracle's ~1e-16).  The result is
-// deterministic: a fixed grid of blocks each reduces a fixed set of rows in
-// a fixed order, and a single block adds the per-block partials in index
-// order.
+// deterministic: a grid of blocks fixed by the field's shape each reduces a
+// fixed set of row segments in a fixed order, and the block that finishes last
+// adds the per-block partials in index order.
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -26,10 +26,18 @@
 
 namespace ac {
 
-__device__ __forceinline__ double warp_sum(double v) {
+// Sums of v0 .. v3 over the warp: lane 8 q gets that of v_q.  The lanes halve
+// the number of values they carry in the first two exchanges: 6 FP64 additions
+// a lane instead of 20 (the FP64 pipe bounds a reduction over small fields).
+__device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, double v3) {
+  const int lane = threadIdx.x & 31;
+  const bool b4 = lane & 16, b3 = lane & 8;
+  double a = (b4 ? v2 : v0) + __shfl_xor_sync(0xffffffffu, b4 ? v0 : v2, 16);
+  const double c = (b4 ? v3 : v1) + __shfl_xor_sync(0xffffffffu, b4 ? v1 : v3, 16);
+  a = (b3 ? c : a) + __shfl_xor_sync(0xffffffffu, b3 ? a : c, 8);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
 }
 
 // Error-free transformations in FP32 (every operation rounded as written).
@@ -59,105 +67,129 @@ __device__ __forceinline__ void add_ff(FF &acc, FF t) {
 }
 constexpr int kFFGroup = 16;
 
+// Sums of one block over its segments (a segment: up to 32 * kFFGroup cells of
+// a row, one warp); the sum of quantity q is valid in thread q < 4.
 template <typename T>
-__global__ void __launch_bounds__(256) observe_partial(const T *__restrict__ phi, GridParams g,
-                                                       double *__restrict__ partials) {
-  constexpr int kWarps = 8;
+__device__ __forceinline__ double observe_block(const T *__restrict__ phi, const GridParams &g) {
+  constexpr int kWarps = 8, group = kFFGroup;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double bulk = 0.0, grad = 0.0, vol = 0.0, bad = 0.0;
-  const int64_t rows = g.ny * g.nz;
+  double bulk = 0.0, grad = 0.0, vol = 0.0;
+  int bad = 0, cnt = 0;
   const int64_t plane = g.pitch * g.ny;
-  // each warp takes whole rows, rows strided over all warps of the grid
-  for (int64_t r = (int64_t)blockIdx.x * kWarps + warp; r < rows;
-       r += (int64_t)gridDim.x * kWarps) {
+  const int64_t segs = (g.nx + 32 * group - 1) / (32 * group);
+  const int64_t units = g.ny * g.nz * segs;
+  // each warp takes segments strided over all warps of the grid
+  for (int64_t u = (int64_t)blockIdx.x * kWarps + warp; u < units; u += (int64_t)gridDim.x * kWarps) {
+    const int64_t r = u / segs, first = (u - r * segs) * 32 * group;
     const int64_t j = r % g.ny, k = r / g.ny;
     const T *row = phi + k * plane + j * g.pitch;
     const bool has_up = j + 1 < g.ny, has_front = k + 1 < g.nz;
     if constexpr (std::is_same_v<T, double>) {
-      for (int64_t i = lane; i < g.nx; i += 32) {
+      const int64_t end = min(g.nx, first + 32 * group);
+      for (int64_t i = first + lane; i < end; i += 32) {
         const double p = row[i];
-        if (!isfinite(p)) bad += 1.0;
+        if (!isfinite(p)) ++bad;
         const double q = p * p - 1.0;
-        bulk += 0.25 * q * q;
-        vol += 0.5 * (1.0 + p);
+        bulk += q * q;
+        vol += p;
+        ++cnt;
         if (i + 1 < g.nx) { double d = row[i + 1] - p; grad += d * d; }
         if (has_up) { double d = row[i + g.pitch] - p; grad += d * d; }
         if (has_front) { double d = row[i + plane] - p; grad += d * d; }
       }
     } else {
-      for (int64_t i0 = lane; i0 < g.nx; i0 += 32 * kFFGroup) {
-        FF b{0.f, 0.f}, gr{0.f, 0.f}, sp{0.f, 0.f};
-        int cnt = 0;
+      FF b{0.f, 0.f}, gr{0.f, 0.f}, sp{0.f, 0.f};
 #pragma unroll 4
-        for (int u = 0; u < kFFGroup; ++u) {
-          const int64_t i = i0 + 32 * u;
-          if (i >= g.nx) break;
-          const float p = to_c(row[i]);
-          if (!isfinite(p)) bad += 1.0;
-          ++cnt;
-          // (p^2 - 1)^2: p^2 = p2.h + p2.l exactly, q = p^2 - 1 to ~48 bits
-          const FF p2 = two_prod(p, p);
-          FF q = two_sum(p2.h, -1.0f);
-          q.l = __fadd_rn(q.l, p2.l);
-          add_ff(b, square_ff(q.h, q.l));
-          add_ff(sp, FF{p, 0.f});
-          // (phi_a - p)^2 over the faces to the +x, +y, +z neighbours
-          if (i + 1 < g.nx) {
-            const FF d = two_sum(to_c(row[i + 1]), -p);
-            add_ff(gr, square_ff(d.h, d.l));
-          }
-          if (has_up) {
-            const FF d = two_sum(to_c(row[i + g.pitch]), -p);
-            add_ff(gr, square_ff(d.h, d.l));
-          }
-          if (has_front) {
-            const FF d = two_sum(to_c(row[i + plane]), -p);
-            add_ff(gr, square_ff(d.h, d.l));
-          }
+      for (int q = 0; q < group; ++q) {
+        const int64_t i = first + lane + 32 * q;
+        if (i >= g.nx) break;
+        const float p = to_c(row[i]);
+        if (!isfinite(p)) ++bad;
+        ++cnt;
+        // (p^2 - 1)^2: p^2 = p2.h + p2.l exactly, q = p^2 - 1 to ~48 bits
+        const FF p2 = two_prod(p, p);
+        FF qq = two_sum(p2.h, -1.0f);
+        qq.l = __fadd_rn(qq.l, p2.l);
+        add_ff(b, square_ff(qq.h, qq.l));
+        add_ff(sp, FF{p, 0.f});
+        // (phi_a - p)^2 over the faces to the +x, +y, +z neighbours
+        if (i + 1 < g.nx) {
+          const FF d = two_sum(to_c(row[i + 1]), -p);
+          add_ff(gr, square_ff(d.h, d.l));
         }
-        bulk += 0.25 * ((double)b.h + (double)b.l);
-        grad += (double)gr.h + (double)gr.l;
-        vol += 0.5 * (double)cnt + 0.5 * ((double)sp.h + (double)sp.l);
+        if (has_up) {
+          const FF d = two_sum(to_c(row[i + g.pitch]), -p);
+          add_ff(gr, square_ff(d.h, d.l));
+        }
+        if (has_front) {
+          const FF d = two_sum(to_c(row[i + plane]), -p);
+          add_ff(gr, square_ff(d.h, d.l));
+        }
       }
+      bulk += (double)b.h + (double)b.l;
+      grad += (double)gr.h + (double)gr.l;
+      vol += (double)sp.h + (double)sp.l;
     }
   }
   __shared__ double red[4][kWarps];
-  bulk = warp_sum(bulk); grad = warp_sum(grad); vol = warp_sum(vol); bad = warp_sum(bad);
-  if (lane == 0) { red[0][warp] = bulk; red[1][warp] = grad; red[2][warp] = vol; red[3][warp] = bad; }
+  const double w4 = warp_sum4(0.25 * bulk, grad, 0.5 * ((double)cnt + vol), (double)bad);
+  if ((lane & 7) == 0) red[lane >> 3][warp] = w4;
   __syncthreads();
-  if (threadIdx.x < 4) {
-    double s = 0.0;
+  double s = 0.0;
+  if (threadIdx.x < 4)
     for (int w = 0; w < kWarps; ++w) s += red[threadIdx.x][w];
-    partials[(int64_t)blockIdx.x * 4 + threadIdx.x] = s;
-  }
+  return s;
 }
 
-// One block of 128 threads: thread t adds partials t, t+128, ... in order,
-// then a fixed tree over the 128 thread sums.
-__global__ void __launch_bounds__(128) observe_final(const double *__restrict__ partials, int nb,
-                                                     double *__restrict__ out) {
-  __shared__ double s[4][128];
+// The partials of nb blocks added by one block of 256 threads (thread t adds
+// partials t, t + 256, ... in order, then a fixed tree); the total q is valid
+// in thread q < 4.
+__device__ __forceinline__ double observe_total(const double *partials, int nb) {
+  __shared__ double s[4][256];
   double a[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int b = threadIdx.x; b < nb; b += 128)
+  for (int b = threadIdx.x; b < nb; b += 256)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) a[q] += partials[(int64_t)b * 4 + q];
+    for (int q = 0; q < 4; ++q) a[q] += __ldcg(partials + (int64_t)b * 4 + q);
 #pragma unroll
   for (int q = 0; q < 4; ++q) s[q][threadIdx.x] = a[q];
   __syncthreads();
-  for (int w = 64; w > 0; w >>= 1) {
+  for (int w = 128; w > 0; w >>= 1) {
     if (threadIdx.x < w)
 #pragma unroll
       for (int q = 0; q < 4; ++q) s[q][threadIdx.x] += s[q][threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x < 4) out[threadIdx.x] = s[threadIdx.x][0];
+  return threadIdx.x < 4 ? s[threadIdx.x][0] : 0.0;
 }
 
+// `done` counts finished blocks and returns to zero with the last one, which
+// adds the partials; out may be device or (mapped) host memory.
+template <typename T>
+__global__ void __launch_bounds__(256) observe_k(const T *__restrict__ phi, GridParams g, double *partials,
+                                                 unsigned int *done, double *out) {
+  const double s = observe_block<T>(phi, g);
+  if (threadIdx.x < 4) partials[(int64_t)blockIdx.x * 4 + threadIdx.x] = s;
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const double t = observe_total(partials, gridDim.x);
+  if (threadIdx.x < 4) out[threadIdx.x] = t;
+}
+
+// One warp to a segment of 512 cells (16 a lane, a float-float group).  With one
+// warp to a row, two kernels and 20 FP64 additions a lane to reduce a warp,
+// 1024^2 FP32 took 27 + 8 us.
 template <typename T>
 static cudaError_t observe_t(const GridParams &g, const void *phi, double *partials, double *out,
                              cudaStream_t s) {
-  observe_partial<T><<<kReduceBlocks, 256, 0, s>>>((const T *)phi, g, partials);
-  observe_final<<<1, 128, 0, s>>>(partials, kReduceBlocks, out);
+  const int64_t units = g.ny * g.nz * ((g.nx + 32 * kFFGroup - 1) / (32 * kFFGroup));
+  const int blocks = (int)std::min<int64_t>((units + 7) / 8, kReduceBlocks);
+  observe_k<T><<<blocks, 256, 0, s>>>((const T *)phi, g, partials,
+                                      reinterpret_cast<unsigned int *>(partials + 4 * kReduceBlocks), out);
   return cudaGetLastError();
 }
 
@@ -171,9 +203,15 @@ cudaError_t launch_observe(int dtype, const GridParams &g, const void *phi, doub
   return cudaErrorInvalidValue;
 }
 
+cudaError_t observe_alloc(double **partials, cudaStream_t s) {
+  cudaError_t e = cudaMalloc(partials, sizeof(double) * (4 * kReduceBlocks + 1));
+  if (e == cudaSuccess) e = cudaMemsetAsync(*partials + 4 * kReduceBlocks, 0, sizeof(double), s);
+  return e;
+}
+
 // ------------------------------------------------- allocation-free variant --
-// ac_observe_noalloc (see include/ac.h) runs the same per-block partial-sum
-// kernel, but over a grid of one block per kNoAllocRowsPerBlock rows, with
+// ac_observe_noalloc (see include/ac.h) forms the same per-block partial sums,
+// but over a grid of one block per kNoAllocRowsPerBlock rows, with
 // its partial sums in the fixed array below instead of a buffer from
 // ac_create.  The array is a module global: every GPU that loads the library
 // holds its 512 KiB until the process exits, and all calls on a device share
@@ -185,7 +223,14 @@ constexpr int kNoAllocMaxBlocks = 16384;
 constexpr int kNoAllocRowsPerBlock = 64;
 static __device__ __align__(256) double g_noalloc_partials[kNoAllocMaxBlocks * 4];
 
-// Sums the partials in a fixed order (as observe_final) and forms the
+template <typename T>
+__global__ void __launch_bounds__(256) observe_partial(const T *__restrict__ phi, GridParams g,
+                                                       double *__restrict__ partials) {
+  const double s = observe_block<T>(phi, g);
+  if (threadIdx.x < 4) partials[(int64_t)blockIdx.x * 4 + threadIdx.x] = s;
+}
+
+// Sums the partials in a fixed order (as observe_total) and forms the
 // observables on the device: out[0] = E_h, out[1] = V, out[2] = non-finite count.
 __global__ void __launch_bounds__(128) observe_final_noalloc(const double *__restrict__ partials,
                                                              int nb, double hd, double inv_eps2,

@@ -85,8 +85,11 @@ cudaError_t launch_block2d(int dtype, const Block2DPlan &p, const GridParams &g,
 
 // FP64 reductions: out[0] = sum F(phi), out[1] = sum over interior faces of
 // (phi_a - phi_b)^2, out[2] = sum (1 + phi)/2, out[3] = non-finite count.
-// partials must hold kReduceBlocks * 4 doubles.
+// One kernel; partials comes from observe_alloc (the blocks' sums and a count of
+// finished blocks, which each call leaves at zero); out may be device memory
+// or pinned host memory.
 constexpr int kReduceBlocks = 1216;
+cudaError_t observe_alloc(double **partials, cudaStream_t s);
 cudaError_t launch_observe(int dtype, const GridParams &g, const void *phi, double *partials,
                            double *out, cudaStream_t s);
 
