@@ -176,10 +176,11 @@ int ac_init_shape(ac_ctx *ctx, int32_t kind, double lower_x, double lower_y, dou
 /* Kernel variants selectable with ac_set_schedule. */
 enum {
   AC_VARIANT_AUTO = 0,    /* autotuned choice if ac_autotune ran, else default.
-                             2D: while the choice is the default schedule and
-                             no tile is forced, its passes may run on a
-                             register-tile kernel, several passes to a launch,
-                             with the same results bit for bit                */
+                             While the choice is the default schedule and no
+                             tile is forced, its passes may run on other
+                             kernels (2D: register tiles, several passes to a
+                             launch; small 3D FP32 grids: one step to a
+                             launch) with the same results bit for bit        */
   AC_VARIANT_DIRECT = 1,  /* one step per launch, neighbours read from global
                              memory with clamped indices (k must be 1)         */
   AC_VARIANT_STREAM = 2   /* TMA-staged streaming kernel with temporal blocking:

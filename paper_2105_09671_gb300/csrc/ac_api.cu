@@ -398,13 +398,15 @@ bool ac_plan_depths(int64_t n, int k, std::vector<int> &depths) {
   return false;
 }
 
-// Whether a schedule may run on the register-tile kernels (block2d.cuh,
-// block2d_fx.cuh): the default 2D schedule, unless the caller forced a
-// schedule or a strip width (those run as asked).  The results are bit for bit
-// those of the default schedule's passes: FP32 and FP64 do not depend on the
-// depth, and FP16 storage is rounded where they end.
-static bool takes_block2d(const ac_ctx *c, int variant, int k, int tile) {
-  if (c->d.ndim != 2 || c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO) return false;
+// Whether a schedule may run on the kernels that stand in for the default
+// one's (in 2D the register-tile kernels of block2d.cuh and block2d_fx.cuh, on
+// small 3D FP32 grids step3d_vec): the default schedule, unless the caller
+// forced a schedule or a tile (those run as asked).  The results are bit for
+// bit those of the default schedule's passes: FP32 and FP64 do not depend on
+// the depth, and FP16 storage is rounded where they end.
+static bool takes_stand_in(const ac_ctx *c, int variant, int k, int tile) {
+  if (c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO) return false;
+  if (c->d.ndim == 3 && !step3d_vec_serves(c->d.dtype, c->gp)) return false;
   if (c->d.dtype == AC_F64 && !fx_coefficients(c->gp.alpha, c->gp.beta)) return false;
   int dv, dk;
   default_schedule(c, &dv, &dk);
@@ -447,14 +449,22 @@ static int issue_block2d(ac_ctx *c, int64_t n, int k, bool *done) {
 }
 
 static int issue_steps(ac_ctx *c, int64_t n, int variant, int k, int tile) {
-  if (takes_block2d(c, variant, k, tile)) {
+  const bool stand_in = takes_stand_in(c, variant, k, tile);
+  if (stand_in && c->d.ndim == 2) {
     bool done = false;
     const int rc = issue_block2d(c, n, k, &done);
     if (rc || done) return rc;
   }
+  const bool vec3d = stand_in && c->d.ndim == 3;
   std::vector<int> depths;
   const bool even = variant == AC_VARIANT_DIRECT ? (n % 2 == 0) : ac_plan_depths(n, k, depths);
   if (variant == AC_VARIANT_DIRECT) depths.assign((size_t)n, 1);
+  if (vec3d) {
+    // single steps; an odd count starts with a pass of two, so that an even
+    // number of launches leaves the result in phi
+    depths.assign((size_t)(n % 2 && n > 1 ? n - 1 : n), 1);
+    if (n % 2 && n > 1) depths[0] = 2;
+  }
   bool src_is_phi = true;
   for (int dep : depths) {
     void *src = src_is_phi ? c->phi : c->ws;
@@ -462,6 +472,8 @@ static int issue_steps(ac_ctx *c, int64_t n, int variant, int k, int tile) {
     cudaError_t e;
     if (variant == AC_VARIANT_DIRECT) {
       e = launch_direct(c->d.ndim, c->d.dtype, c->gp, src, dst, c->stream);
+    } else if (vec3d && dep == 1) {
+      e = launch_step3d_vec(c->gp, src, dst, c->stream);
     } else {
       // a remainder depth the tile does not offer runs on tile 0
       const int tl = schedule_ok(c, variant, dep, tile) ? tile : 0;
@@ -493,7 +505,7 @@ extern "C" int ac_step(ac_ctx *c, int64_t n) {
   if (!c->use_graph || c->stream == nullptr) return issue_steps(c, n, variant, k, tile);
   // graph replay: capture the launch sequence for this (n, schedule) once
   if (c->graph_exec == nullptr || c->graph_n != n || c->graph_variant != variant ||
-      c->graph_k != k || c->graph_tile != tile || c->graph_block != takes_block2d(c, variant, k, tile)) {
+      c->graph_k != k || c->graph_tile != tile || c->graph_stand_in != takes_stand_in(c, variant, k, tile)) {
     release_graph(c);
     AC_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed));
     const int64_t before = c->launches;
@@ -511,7 +523,7 @@ extern "C" int ac_step(ac_ctx *c, int64_t n) {
     c->graph_variant = variant;
     c->graph_k = k;
     c->graph_tile = tile;
-    c->graph_block = takes_block2d(c, variant, k, tile);
+    c->graph_stand_in = takes_stand_in(c, variant, k, tile);
   }
   AC_CUDA(cudaGraphLaunch(c->graph_exec, c->stream));
   c->launches += c->graph_launches;

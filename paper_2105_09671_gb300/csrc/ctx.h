@@ -26,7 +26,7 @@ struct ac_ctx {
   bool use_graph = false;
   int64_t graph_n = -1;
   int graph_variant = -1, graph_k = -1, graph_tile = -1;
-  bool graph_block = false;
+  bool graph_stand_in = false;
   cudaGraphExec_t graph_exec = nullptr;
   int64_t graph_launches = 0;  // kernels in the captured graph
   // kernels this context has put on its stream (graph replays count their nodes)

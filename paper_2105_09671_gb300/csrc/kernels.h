@@ -60,6 +60,9 @@ inline dim3 cell_grid(const GridParams &g) {
 
 cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *src, void *dst,
                           cudaStream_t s);
+// One step of a small 3D FP32 grid (see k_direct.cu).
+bool step3d_vec_serves(int dtype, const GridParams &g);
+cudaError_t launch_step3d_vec(const GridParams &g, const void *src, void *dst, cudaStream_t s);
 // k steps per launch.  src_map describes the source field with the box of
 // stream{2,3}d_geom(dtype, k).
 cudaError_t launch_stream2d(int dtype, int k, int tile, const GridParams &g, const CUtensorMap *src_map,

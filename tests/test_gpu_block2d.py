@@ -1,6 +1,6 @@
-"""The default 2D schedule's register-tile kernel against the streaming kernel
-at the schedule it stands for: the same bits, for every tile variant that the
-rule can pick, with ragged tiles, grids smaller than a tile (the halo reflected
+"""The kernels that stand in for the default schedule (2D register tiles, small
+3D grids) against the streaming kernel at the schedule they stand for: the
+same bits, for every variant that the rules can pick, with ragged tiles, grids smaller than a tile (the halo reflected
 several times), and step counts that split unevenly over the launches."""
 import numpy as np
 import pytest
@@ -40,6 +40,34 @@ def test_default_equals_the_streaming_schedule_bitwise(shape, dtype):
         assert bool(a.padded[:, :, nx:].isnan().all()), "padding written"
         if np.prod(shape) < 1 << 19:
             assert_parity(out.astype(np.float64), oracle_run(phi0, h, eps, dt, 100, dtype), dtype)
+    finally:
+        a.close()
+        b.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 5), (7, 1, 64), (33, 35, 31), (40, 60, 70), (81, 90, 101)])
+def test_small_3d_default_equals_the_streaming_schedule_bitwise(shape):
+    # one step to a launch, in each of its plane counts a thread; odd step
+    # counts start with a pass of two
+    h = 1.0 / max(shape)
+    eps, dt = 2.5 * h, 0.1 * h * h
+    phi0 = wl.random_field(shape, seed=sum(shape))
+    nx = shape[-1]
+    a = ac.Simulation(shape, h, eps, dt, dtype="f32", pitch_x=-(-nx // 4) * 4 + 4)
+    b = ac.Simulation(shape, h, eps, dt, dtype="f32")
+    try:
+        b.set_schedule(*b.schedule())
+        for n in (1, 2, 3, 8, 17):
+            a.padded.fill_(float("nan"))
+            a._ws.fill_(float("nan"))
+            a.load(phi0)
+            b.load(phi0)
+            a.step(n)
+            b.step(n)
+            out = a.to_numpy()
+            assert np.array_equal(out, b.to_numpy()), f"{shape} n={n}"
+        assert bool(a.padded[:, :, nx:].isnan().all()), "padding written"
+        assert_parity(out.astype(np.float64), oracle_run(phi0, h, eps, dt, 17, "f32"), "f32")
     finally:
         a.close()
         b.close()
