@@ -13,20 +13,21 @@ namespace {
 // with t0 the launch, load one tile's load and store, lat one step's latency
 // and busy the time a warp's step keeps the SM busy.  Fitted to sweeps over
 // 64^2 .. 8192^2, warps and k; on those grids the variant, warps and k that
-// the fit picks run within 2 % of the best measured.  Which wins where:
-// 4 x 4 cells a lane up to 512^2 (400x200: 0.405 us a step against 0.42 .. 0.46
-// for the others), 8 rows near 1024^2 (0.81 against 0.99 / 0.88), 7 rows in 64
-// registers (two CTAs to an SM) from 2048^2 cells (4096^2: 8.6 us against
-// 9.6 / 10.9), and for FP16 storage 8 x 8 cells there (4096^2: 8.3 against 9.1).
+// the fit picks run within 2 % of the best measured (FP16 storage at 8192^2:
+// 7 %).  Which wins where: 4 x 4 cells a lane up to 512^2 (400x200: 0.371 us a
+// step against 0.405 and 0.486), 8 rows near 1024^2 (0.78 against 0.87 and
+// 0.98), 7 rows in 64 registers (two CTAs to an SM) from 2048^2 (4096^2: 8.0 us
+// against 9.4 and 10.9), and for FP16 storage 9 rows there (4096^2: 7.3; 7.7
+// with 8 x 8 cells).
 struct B2Variant {
-  int E, R, regs;
+  int E, R, regs;  // E: cells a lane and row (FP64: 1)
   double t0, load, lat, busy;
 };
 constexpr B2Variant kB2[] = {
-    {4, 4, 56, 1.44, 1.21, 0.074, 0.0260},
-    {4, 7, 64, 1.65, 1.69, 0.057, 0.0402},
-    {4, 8, 96, 1.50, 1.93, 0.086, 0.0473},
-    {8, 8, 128, 2.90, 1.75, 0.246, 0.0928},
+    {4, 4, 72, 1.06, 1.55, 0.069, 0.0202},
+    {4, 7, 64, 1.49, 1.81, 0.131, 0.0363},
+    {4, 8, 112, 1.13, 2.15, 0.005, 0.0404},
+    {4, 9, 64, 2.18, 1.41, 0.207, 0.0476},  // FP16 storage
     // FP64 (block2d_fx.cuh): two rows a lane for the smallest grids (200^2 1.42
     // us a step against 1.66 with four), four from 512^2 on (3.56 against 4.14)
     {1, 2, 32, 1.30, 1.37, 0.0, 0.0632},
@@ -39,16 +40,14 @@ constexpr int kB2Count = sizeof(kB2) / sizeof(kB2[0]);
 double march_cost(int64_t nx, int64_t ny) { return 3.5 + 6.7e-6 * (double)nx * (double)ny; }
 
 bool offered(const B2Variant &b, int dtype) {
-  return dtype == AC_F64 ? b.E == 1 : b.E == 4 || (b.E == 8 && dtype == AC_F16S);
+  return dtype == AC_F64 ? b.E == 1 : b.E == 4 && (b.R != 9 || dtype == AC_F16S);
 }
 
-int halo_x(int dtype, int E, int k) {
-  const int v = std::min(E, dtype == AC_F16S ? 8 : 4);  // whole memory vectors (FP64: single cells)
-  return (k + v - 1) / v * v;
-}
+// Halo columns: whole memory vectors of 4 cells (FP64: single cells).
+int halo_x(int E, int k) { return (k + E - 1) / E * E; }
 
-double launch_cost(const B2Variant &b, int dtype, int64_t nx, int64_t ny, int warps, int k, int num_sms) {
-  const int ow = 32 * b.E - 2 * halo_x(dtype, b.E, k), oh = warps * b.R - 2 * k;
+double launch_cost(const B2Variant &b, int64_t nx, int64_t ny, int warps, int k, int num_sms) {
+  const int ow = 32 * b.E - 2 * halo_x(b.E, k), oh = warps * b.R - 2 * k;
   const double tiles = std::ceil((double)nx / ow) * std::ceil((double)ny / oh);
   const int occ = std::max(1, std::min(65536 / (b.regs * warps * 32), 64 / warps));
   const double per_sm = std::ceil(tiles / num_sms);
@@ -65,7 +64,7 @@ cudaError_t launch_t(const GridParams &g, const void *src, void *dst, int warps,
   cudaError_t e = kernel_setup(ks, (const void *)block2d_k<T, E, R, MINB>, kB2MaxWarps * 32,
                                b2_smem_bytes(E, kB2MaxWarps), &occ);
   if (e != cudaSuccess) return e;
-  const int hx = halo_x(sizeof(T) == 2 ? AC_F16S : AC_F32, E, k);
+  const int hx = halo_x(E, k);
   const int ow = 32 * E - 2 * hx, oh = warps * R - 2 * k;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((g.nx + ow - 1) / ow), (unsigned)((g.ny + oh - 1) / oh));
@@ -122,7 +121,7 @@ bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, 
         const int k = (int)((passes + launches - 1) / launches) * depth;
         const int oh = warps * kB2[v].R - 2 * k;
         if ((ny + oh - 1) / oh > 65535) continue;  // CUDA's grid limit in y
-        const double cost = (double)launches * launch_cost(kB2[v], dtype, nx, ny, warps, k, num_sms);
+        const double cost = (double)launches * launch_cost(kB2[v], nx, ny, warps, k, num_sms);
         if (cost < best) {
           best = cost;
           found = true;
@@ -151,7 +150,7 @@ cudaError_t launch_block2d(int dtype, const Block2DPlan &p, const GridParams &g,
       case 0: return launch_t<__half, 4, 4, 1>(g, src, dst, p.warps, k, round_mask, s);
       case 1: return launch_t<__half, 4, 7, 2>(g, src, dst, p.warps, k, round_mask, s);
       case 2: return launch_t<__half, 4, 8, 1>(g, src, dst, p.warps, k, round_mask, s);
-      case 3: return launch_t<__half, 8, 8, 1>(g, src, dst, p.warps, k, round_mask, s);
+      case 3: return launch_t<__half, 4, 9, 2>(g, src, dst, p.warps, k, round_mask, s);
     }
   }
   return cudaErrorInvalidValue;
