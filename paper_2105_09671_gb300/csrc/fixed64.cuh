@@ -30,15 +30,23 @@ struct Fx {  // x = hi 2^32 + lo with lo signed
 __device__ __forceinline__ Fx fx_split(int64_t x) {
   Fx r;
   r.lo = (int)(uint32_t)x;
-  r.hi = (int)(x >> 32) + (r.lo < 0);
+  r.hi = (int)(x >> 32) + (int)((uint32_t)x >> 31);
   return r;
 }
 // a * b / 2^64, rounded; the product of the low halves (a quarter of a unit
-// at most) is left out.
+// at most) is left out.  Three wide multiply-adds and a sign extension, in
+// PTX: from C the same arithmetic took 13 instructions.
 __device__ __forceinline__ int64_t fx_mulhi(const Fx &a, const Fx &b) {
-  int64_t t = (int64_t)a.hi * b.lo + 0x80000000ll;
-  t += (int64_t)a.lo * b.hi;
-  return (int64_t)a.hi * b.hi + (t >> 32);
+  int64_t r;
+  asm("{\n\t.reg .s64 t, u;\n\t.reg .s32 l, h;\n\t"
+      "mad.wide.s32 t, %1, %4, %5;\n\t"
+      "mad.wide.s32 t, %2, %3, t;\n\t"
+      "mov.b64 {l, h}, t;\n\t"
+      "cvt.s64.s32 u, h;\n\t"
+      "mad.wide.s32 %0, %1, %3, u;\n\t}"
+      : "=l"(r)
+      : "r"(a.hi), "r"(a.lo), "r"(b.hi), "r"(b.lo), "l"(0x80000000ll));
+  return r;
 }
 
 // A value as m 2^(e - 1084), 2^61 <= |m| < 2^62 (0 and subnormal values: any m,
@@ -52,17 +60,22 @@ constexpr int kFxOut = 2047;
 // are slower than the FP64 operations they would replace.)
 __device__ __forceinline__ FxV fx_in(double v) {
   const int hi = __double2hiint(v);
+  const uint32_t twice = 2u * (uint32_t)hi;  // without the sign
   const int64_t a =
       (int64_t)(((uint64_t)(uint32_t)((hi & 0xfffff) | 0x100000) << 32 | (uint32_t)__double2loint(v)) << 9);
-  const int64_t sgn = hi >> 31;
   FxV r;
-  r.m = (a ^ sgn) - sgn;
-  r.e = (hi & 0x7fffffff) < 0x3ff40000 ? (hi >> 20) & 0x7ff : kFxOut;
+  r.m = hi < 0 ? -a : a;
+  r.e = twice < 2u * 0x3ff40000u ? (int)(twice >> 21) : kFxOut;
   return r;
 }
 // Whether a stencil with largest exponent e takes the integer form.
 __device__ __forceinline__ bool fx_in_range(int e) { return (unsigned)(e - 64) < 1024u - 64u; }
-__device__ __forceinline__ int64_t fx_shift(int64_t m, int d) { return m >> min(d, 63); }
+// m / 2^d, d >= 0, rounded down (the instruction clamps d).
+__device__ __forceinline__ int64_t fx_shift(int64_t m, int d) {
+  int64_t r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(d));
+  return r;
+}
 // v in units of 2^(e - 1081), e at least its exponent.
 __device__ __forceinline__ int64_t fx_align(const FxV &v, int e) { return fx_shift(v.m, e - v.e + 3); }
 // x 2^(e - 1082), rounded once: its halves become the mantissas of doubles
@@ -113,10 +126,10 @@ __device__ __forceinline__ double fx_update(const FxV &p, int64_t nsum, int e, c
   const int64_t x = fx_align(p, e);
   const int64_t lap = NDIM == 2 ? nsum - (x << 2) : nsum - ((x << 2) + (x << 1));
   const Fx P = fx_split(p.m);
-  // phi^2 in units of 2^-58, phi (1 - phi^2) and alpha times it in units of p.m
-  const int64_t w = ((1ll << 58) - fx_shift(fx_mulhi(P, P), 2 * (1023 - p.e))) << 4;
+  // 1 - phi^2 in units of 2^-58, phi times it in 2^(p.e - 1078)
+  const int64_t w = (1ll << 58) - fx_shift(fx_mulhi(P, P), 2046 - 2 * p.e);
   const int64_t q = fx_mulhi(P, fx_split(w));
-  const int64_t a = fx_mulhi(fx_split(q << 2), c.A);  // units 2^(p.e - 1083)
+  const int64_t a = fx_mulhi(fx_split(q << 6), c.A);  // units 2^(p.e - 1083)
   const int64_t b = fx_mulhi(fx_split(lap), c.B);     // units 2^(e - 1082)
   return fx_out((x << 1) + b + fx_shift(a, e - p.e + 1), e);
 }

@@ -97,7 +97,7 @@ __device__ __forceinline__ void fx_store(double *row, int xl, int lane, int nx, 
 // A warp owns kFx2W columns and marches over `chunk` rows.  Bound by integer
 // issue (some 140 instructions a cell, 14 of them wide multiply-adds): 4096^2
 // 253 -> 116 us a step, 2048^2 64 -> 32 against the FP64 operations.
-__global__ void __launch_bounds__(kFxWarps * 32) step2d_fx(const double *__restrict__ src,
+__global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__restrict__ src,
                                                            double *__restrict__ dst, GridParams g, int strips,
                                                            int chunk) {
   const int lane = threadIdx.x & 31;
