@@ -209,6 +209,21 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, u
       : "memory");
 }
 
+// Asynchronous copies of 16 or 4 bytes from global to shared memory (zeros
+// where !valid; g must be a readable address all the same); cp_async_wait
+// waits for all of this thread's.
+__device__ __forceinline__ void cp_async16(void *smem, const void *g, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem)), "l"(g),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *smem, const void *g, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(smem)), "l"(g),
+               "r"(valid ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ void report_timeout(int *status) {
   if (status) atomicExch(status, AC_ERR_TIMEOUT);
 }

@@ -31,18 +31,9 @@
 
 namespace ac {
 
-template <int NDIM>
-__device__ __forceinline__ void decode_cell(const NetShape &sh, int64_t i, int &b, int &z, int &y,
-                                            int &x) {
-  x = (int)(i % sh.nx);
-  i /= sh.nx;
-  y = (int)(i % sh.ny);
-  i /= sh.ny;
-  z = (int)(i % sh.nz);
-  b = (int)(i / sh.nz);
-}
-
 // ------------------------------------------------------------ first layer --
+// A thread per cell of a 32 x 8 block of one z (no index division), packed FP32
+// pairs of channels.
 template <int NDIM, bool TRAIN>
 __global__ void __launch_bounds__(256) net_first_fwd_k(const float *__restrict__ phi,
                                                        const float *__restrict__ params,
@@ -50,58 +41,66 @@ __global__ void __launch_bounds__(256) net_first_fwd_k(const float *__restrict__
                                                        bf16 *__restrict__ z1, bf16 *__restrict__ a1pad) {
   constexpr int T = net_taps(NDIM);
   __shared__ __align__(16) float w[T * kNetC];
-  __shared__ float bb[kNetC];
+  __shared__ __align__(16) float bb[kNetC];
   for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) w[i] = params[w_off + i];
   if (threadIdx.x < kNetC) bb[threadIdx.x] = params[b_off + threadIdx.x];
   __syncthreads();
-  const int64_t n = sh.cells();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int b, z, y, x;
-    decode_cell<NDIM>(sh, i, b, z, y, x);
-    float acc[kNetC];
+  const int x = (int)blockIdx.x * 32 + (threadIdx.x & 31);
+  const int64_t planes = (int64_t)sh.batch * sh.nz;
+  if (x >= sh.nx) return;
+  for (int64_t bz = blockIdx.z; bz < planes; bz += gridDim.z)
+  for (int y = (int)blockIdx.y * 8 + (threadIdx.x >> 5); y < sh.ny; y += (int)gridDim.y * 8) {
+    const int b = (int)(bz / sh.nz), z = (int)(bz - (int64_t)b * sh.nz);
+    uint64_t acc[kNetC / 2];
 #pragma unroll
-    for (int c = 0; c < kNetC; ++c) acc[c] = bb[c];
+    for (int c = 0; c < kNetC / 2; ++c) acc[c] = reinterpret_cast<const uint64_t *>(bb)[c];
+#pragma unroll
     for (int t = 0; t < T; ++t) {
-      int oz, oy, ox;
-      net_tap(NDIM, t, oz, oy, ox);
+      const int ox = t % 3 - 1, oy = (t / 3) % 3 - 1, oz = NDIM == 3 ? t / 9 - 1 : 0;
       const int xx = min(max(x + ox, 0), sh.nx - 1), yy = min(max(y + oy, 0), sh.ny - 1);
       const int zz = NDIM == 3 ? min(max(z + oz, 0), sh.nz - 1) : 0;
       const float v = phi[sh.u(b, zz, yy, xx)];
+      const uint64_t vv = pack2(v, v);
 #pragma unroll
-      for (int c = 0; c < kNetC; c += 4) {  // 16-byte weight reads (broadcast)
-        const float4 wv = *reinterpret_cast<const float4 *>(w + t * kNetC + c);
-        acc[c] = fmaf(v, wv.x, acc[c]);
-        acc[c + 1] = fmaf(v, wv.y, acc[c + 1]);
-        acc[c + 2] = fmaf(v, wv.z, acc[c + 2]);
-        acc[c + 3] = fmaf(v, wv.w, acc[c + 3]);
+      for (int c = 0; c < kNetC / 2; c += 2) {  // 16-byte weight reads (broadcast)
+        const ulonglong2 wv = *reinterpret_cast<const ulonglong2 *>(w + t * kNetC + 2 * c);
+        acc[c] = fma2(vv, wv.x, acc[c]);
+        acc[c + 1] = fma2(vv, wv.y, acc[c + 1]);
       }
     }
+    float a[kNetC];
     if (TRAIN) {
-      uint4 *dz = reinterpret_cast<uint4 *>(z1 + i * kNetC);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) dz[c] = pack8_bf16(acc + 8 * c);
+      for (int c = 0; c < kNetC / 2; ++c) unpack2(acc[c], a[2 * c], a[2 * c + 1]);
+      bf16 *dz = z1 + sh.u(b, z, y, x) * kNetC;
+      st_global32(dz, pack8_bf16(a), pack8_bf16(a + 8));
+      st_global32(dz + 16, pack8_bf16(a + 16), pack8_bf16(a + 24));
     }
 #pragma unroll
-    for (int c = 0; c < kNetC; ++c) acc[c] = net_gelu_fast(acc[c]);
-    store_replicated<NDIM>(a1pad, sh, b, z, y, x, acc);
+    for (int c = 0; c < kNetC / 2; ++c) unpack2(net_gelu_fast2(acc[c]), a[2 * c], a[2 * c + 1]);
+    store_replicated<NDIM>(a1pad, sh, b, z, y, x, a);
   }
 }
-
 
 // ------------------------------------------------------------- last layer --
 // z6 = conv(a5, W6) + b6 (32 -> 1 channel) and phi_hat = phi + s z6; in
 // training also the scaled residual's gradient g6 and the loss sum.  A block
-// covers 32 x 8 cells of one z: the 10 x 34 padded pixels (x 3 planes in 3D)
-// it reads are staged once in shared memory with coalesced 16-byte loads
-// (pixel stride 80 bytes: conflict-free 16-byte reads by consecutive lanes),
-// then each thread forms one cell.
-constexpr int kLastTX = 32, kLastTY = 8, kLastPix = 5;  // uint4 per staged pixel (4 + pad)
+// covers 32 x 32 cells of one z, a thread 4 cells above one another: the
+// padded pixels of one plane at a time are staged in shared memory with
+// asynchronous 16-byte copies, all in flight at once (pixel stride 80 bytes:
+// conflict-free 16-byte reads by consecutive lanes), and a pixel read serves the up to 3 cells of the
+// thread that it is a tap of, a weight read all 4 (one cell a thread read each
+// pixel 9 times and all weights: 64 us at 1024^2).
+constexpr int kLastTX = 32, kLastRows = 4, kLastTY = 8 * kLastRows, kLastPix = 5;  // uint4 per staged pixel (4 + pad)
 
 template <int NDIM>
 __host__ __device__ constexpr int last_smem_bytes() {
-  return (NDIM == 3 ? 3 : 1) * (kLastTY + 2) * (kLastTX + 2) * kLastPix * 16 +
-         net_taps(NDIM) * kNetC * 4;
+  return (kLastTY + 2) * (kLastTX + 2) * kLastPix * 16 + net_taps(NDIM) * kNetC * 4;
+}
+
+// Two BF16 values as a packed FP32 pair.
+__device__ __forceinline__ uint64_t bf16_pair(uint32_t w) {
+  return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
 
 template <int NDIM, bool TRAIN>
@@ -116,8 +115,8 @@ __global__ void __launch_bounds__(256) net_last_fwd_k(const bf16 *__restrict__ a
   constexpr int NZR = NDIM == 3 ? 3 : 1;
   constexpr int RW = kLastTX + 2, RH = kLastTY + 2;
   extern __shared__ __align__(16) unsigned char lsm[];
-  uint4 *tile = reinterpret_cast<uint4 *>(lsm);                         // [NZR][RH][RW][kLastPix]
-  float *w = reinterpret_cast<float *>(lsm + NZR * RH * RW * kLastPix * 16);  // [T][32]
+  uint4 *tile = reinterpret_cast<uint4 *>(lsm);                          // [RH][RW][kLastPix]
+  float *w = reinterpret_cast<float *>(lsm + RH * RW * kLastPix * 16);   // [T][32]
   __shared__ double red[8];
   for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) w[i] = params[w_off + i];
   const float b6 = params[b_off];
@@ -133,42 +132,57 @@ __global__ void __launch_bounds__(256) net_last_fwd_k(const bf16 *__restrict__ a
     r /= tiles_y;
     const int z = (int)(r % sh.nz), b = (int)(r / sh.nz);
     const int x0 = tx * kLastTX, y0 = ty * kLastTY;
-    __syncthreads();  // the previous item's tile (and w) is complete / released
-    // padded pixels (xp, yp) = (x0 + i, y0 + j), i < RW, j < RH, of planes z .. z+2
-    for (int i = threadIdx.x; i < NZR * RH * RW * 4; i += blockDim.x) {
-      const int c = i & 3;
-      const int q = i >> 2;
-      const int px = q % RW, row = (q / RW) % RH, dz = q / (RW * RH);
-      const int xp = x0 + px, yp = y0 + row;
-      if (xp < sh.px() && yp < sh.py())
-        tile[q * kLastPix + c] = *reinterpret_cast<const uint4 *>(
-            a5pad + (sh.p(b, NDIM == 3 ? z + dz : 0, yp, xp) * kNetC + c * 8));
-    }
-    __syncthreads();
-    const int x = x0 + lane, y = y0 + wy;
-    if (x < sh.nx && y < sh.ny) {
-      float acc = b6;
-      for (int t = 0; t < T; ++t) {
-        int oz, oy, ox;
-        net_tap(NDIM, t, oz, oy, ox);
-        const int dz = NDIM == 3 ? oz + 1 : 0;
-        const uint4 *src = tile + ((dz * RH + wy + oy + 1) * RW + lane + ox + 1) * kLastPix;
+    uint64_t acc[kLastRows];
 #pragma unroll
+    for (int q = 0; q < kLastRows; ++q) acc[q] = 0;
+    for (int dz = 0; dz < NZR; ++dz) {
+      __syncthreads();  // the previous plane (and w) is complete / released
+      // padded pixels (xp, yp) = (x0 + i, y0 + j), i < RW, j < RH, of plane z + dz
+      for (int i = threadIdx.x; i < RH * RW * 4; i += blockDim.x) {
+        const int c = i & 3, q = i >> 2;
+        const int px = q % RW, row = q / RW;
+        const int xp = x0 + px, yp = y0 + row;
+        const bool in = xp < sh.px() && yp < sh.py();
+        cp_async16(tile + q * kLastPix + c,
+                   a5pad + (in ? sh.p(b, NDIM == 3 ? z + dz : 0, yp, xp) * kNetC + c * 8 : 0), in);
+      }
+      cp_async_wait();
+      __syncthreads();
+#pragma unroll
+      for (int ox = 0; ox < 3; ++ox)
+#pragma unroll 1
         for (int c = 0; c < 4; ++c) {
-          float v[8];
-          unpack8_bf16(src[c], v);
+          uint64_t wv[3][4];  // 8 channels of the three oy
 #pragma unroll
-          for (int e = 0; e < 8; e += 4) {  // 16-byte weight reads (broadcast)
-            const float4 wv = *reinterpret_cast<const float4 *>(w + t * kNetC + c * 8 + e);
-            acc = fmaf(v[e], wv.x, acc);
-            acc = fmaf(v[e + 1], wv.y, acc);
-            acc = fmaf(v[e + 2], wv.z, acc);
-            acc = fmaf(v[e + 3], wv.w, acc);
+          for (int oy = 0; oy < 3; ++oy) {
+            const float *wp = w + (dz * 9 + oy * 3 + ox) * kNetC + c * 8;
+            const ulonglong2 lo = *reinterpret_cast<const ulonglong2 *>(wp);
+            const ulonglong2 hi = *reinterpret_cast<const ulonglong2 *>(wp + 4);
+            wv[oy][0] = lo.x; wv[oy][1] = lo.y; wv[oy][2] = hi.x; wv[oy][3] = hi.y;
+          }
+#pragma unroll
+          for (int j = 0; j < kLastRows + 2; ++j) {
+            const uint4 u = tile[((wy * kLastRows + j) * RW + lane + ox) * kLastPix + c];
+            const uint64_t a[4] = {bf16_pair(u.x), bf16_pair(u.y), bf16_pair(u.z), bf16_pair(u.w)};
+#pragma unroll
+            for (int oy = 0; oy < 3; ++oy) {
+              const int q = j - oy;  // the cell whose tap oy this row is
+              if (q < 0 || q >= kLastRows) continue;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) acc[q] = fma2(a[e], wv[oy][e], acc[q]);
+            }
           }
         }
-      }
+    }
+    const int x = x0 + lane;
+#pragma unroll
+    for (int q = 0; q < kLastRows; ++q) {
+      const int y = y0 + wy * kLastRows + q;
+      if (x >= sh.nx || y >= sh.ny) continue;
+      float even, odd;
+      unpack2(acc[q], even, odd);
       const int64_t i = sh.u(b, z, y, x);
-      const float ph = phi[i] + scale * acc;
+      const float ph = phi[i] + scale * (b6 + (even + odd));
       phihat[i] = ph;
       if (TRAIN) {
         const float rr = (ph - target[i]) / scale;
@@ -353,18 +367,17 @@ __global__ void __launch_bounds__(256, 2) net_last_bwd_k(const float *__restrict
     for (int i = threadIdx.x; i < NZR * RH * RW * 4; i += blockDim.x) {
       const int c = i & 3, q = i >> 2;
       const int px = q % RW, row = (q / RW) % RH, dz = q / (RW * RH);
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (x0 + px < sh.px() && y0 + row < sh.py())
-        v = *reinterpret_cast<const uint4 *>(
-            a5pad + (sh.p(b, NDIM == 3 ? z + dz : 0, y0 + row, x0 + px) * kNetC + c * 8));
-      *reinterpret_cast<uint4 *>(ta + ((dz * RH + row) * kEndRow + px) * 64 + c * 16) = v;
+      const bool in = x0 + px < sh.px() && y0 + row < sh.py();
+      cp_async16(ta + ((dz * RH + row) * kEndRow + px) * 64 + c * 16,
+                 a5pad + (in ? sh.p(b, NDIM == 3 ? z + dz : 0, y0 + row, x0 + px) * kNetC + c * 8 : 0), in);
     }
     for (int i = threadIdx.x; i < NZR * RH * RW; i += blockDim.x) {
       const int px = i % RW, row = (i / RW) % RH, dz = i / (RW * RH);
       const int xx = x0 + px - 1, yy = y0 + row - 1, zz = NDIM == 3 ? z + dz - 1 : 0;
       const bool in = xx >= 0 && xx < sh.nx && yy >= 0 && yy < sh.ny && zz >= 0 && zz < sh.nz;
-      tg[(dz * RH + row) * kEndRow1 + px] = in ? g6[sh.u(b, zz, yy, xx)] : 0.f;
+      cp_async4(tg + (dz * RH + row) * kEndRow1 + px, g6 + (in ? sh.u(b, zz, yy, xx) : 0), in);
     }
+    cp_async_wait();
     __syncthreads();
     {
       const int x = x0 + lane, y = y0 + warp;
@@ -477,17 +490,17 @@ __global__ void __launch_bounds__(256, 2) net_first_wgrad_k(const float *__restr
     __syncthreads();
     for (int i = threadIdx.x; i < kEndTY * kEndTX * 4; i += blockDim.x) {
       const int c = i & 3, px = (i >> 2) % kEndTX, row = (i >> 2) / kEndTX;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (x0 + px < sh.nx && y0 + row < sh.ny)
-        v = *reinterpret_cast<const uint4 *>(g1pad + sh.ps(b, z, y0 + row, x0 + px, 0, 0, 0) * kNetC + c * 8);
-      *reinterpret_cast<uint4 *>(tg + (row * kEndRow + px) * 64 + c * 16) = v;
+      const bool in = x0 + px < sh.nx && y0 + row < sh.ny;
+      cp_async16(tg + (row * kEndRow + px) * 64 + c * 16,
+                 g1pad + (in ? sh.ps(b, z, y0 + row, x0 + px, 0, 0, 0) * kNetC + c * 8 : 0), in);
     }
     for (int i = threadIdx.x; i < NZR * RH * RW; i += blockDim.x) {
       const int px = i % RW, row = (i / RW) % RH, dz = i / (RW * RH);
       const int xx = min(max(x0 + px - 1, 0), sh.nx - 1), yy = min(max(y0 + row - 1, 0), sh.ny - 1);
       const int zz = NDIM == 3 ? min(max(z + dz - 1, 0), sh.nz - 1) : 0;
-      tp[(dz * RH + row) * kEndRow1 + px] = phi[sh.u(b, zz, yy, xx)];
+      cp_async4(tp + (dz * RH + row) * kEndRow1 + px, phi + sh.u(b, zz, yy, xx), true);
     }
+    cp_async_wait();
     __syncthreads();
     const int row = 2 * (warp & 3) + (lane >> 4), xs = 16 * (warp >> 2);
     const unsigned char *pg = tg + (row * kEndRow + xs) * 64 + (lane & 15) * 4;
@@ -551,10 +564,6 @@ __global__ void net_pack_k(const float *__restrict__ params, int T, int64_t w0, 
 }
 
 // ------------------------------------------------------------ launchers ----
-static int grid_for(int64_t n, int per_block, int num_sms) {
-  return (int)std::min<int64_t>((n + per_block - 1) / per_block, (int64_t)num_sms * 16);
-}
-
 // Dynamic shared-memory limits of the kernels that need more than the
 // default, once per device (thread-safe; the occupancy query is unused).
 template <int NDIM>
@@ -577,11 +586,18 @@ static cudaError_t net_forward_t(const NetBuffers &nb, const NetShape &sh, const
   cudaError_t e = setup_attrs<NDIM>();
   if (e != cudaSuccess) return e;
   const NetLayout &L = nb.layout;
-  const int64_t n = sh.cells();
+  // first layer: about six blocks to an SM, each over several row tiles, as
+  // every block stages the weights first
+  const int fx = (sh.nx + 31) / 32, fy = (sh.ny + 7) / 8;
+  const int64_t planes = (int64_t)sh.batch * sh.nz;
+  const int64_t fz = std::min<int64_t>(planes, 65535);
+  const dim3 first_grid((unsigned)fx,
+                        (unsigned)std::min<int64_t>(fy, std::max<int64_t>(1, (int64_t)num_sms * 6 / (fx * fz) + 1)),
+                        (unsigned)fz);
   if (train)
-    net_first_fwd_k<NDIM, true><<<grid_for(n, 256, num_sms), 256, 0, s>>>(phi, nb.params, L.w[0], L.b[0], sh, nb.z[0], nb.a[0]);
+    net_first_fwd_k<NDIM, true><<<first_grid, 256, 0, s>>>(phi, nb.params, L.w[0], L.b[0], sh, nb.z[0], nb.a[0]);
   else
-    net_first_fwd_k<NDIM, false><<<grid_for(n, 256, num_sms), 256, 0, s>>>(phi, nb.params, L.w[0], L.b[0], sh, nullptr, nb.a[0]);
+    net_first_fwd_k<NDIM, false><<<first_grid, 256, 0, s>>>(phi, nb.params, L.w[0], L.b[0], sh, nullptr, nb.a[0]);
   const int64_t per = (int64_t)kNetC * net_taps(NDIM) * kNetC;
   for (int l = 1; l <= 4; ++l) {
     bf16 *in = nb.a[(l - 1) % (train ? 5 : 2)];
@@ -593,7 +609,7 @@ static cudaError_t net_forward_t(const NetBuffers &nb, const NetShape &sh, const
   const bf16 *a5 = nb.a[4 % (train ? 5 : 2)];
   const int64_t last_items = (int64_t)sh.batch * sh.nz * ((sh.ny + kLastTY - 1) / kLastTY) *
                              ((sh.nx + kLastTX - 1) / kLastTX);
-  const int last_grid = (int)std::min<int64_t>(last_items, (int64_t)num_sms * 8);
+  const int last_grid = (int)std::min<int64_t>(last_items, (int64_t)num_sms * 2);
   if (train)
     net_last_fwd_k<NDIM, true><<<last_grid, 256, last_smem_bytes<NDIM>(), s>>>(a5, nb.params, L.w[5], L.b[5], sh, phi, scale, phihat, target, nb.g6, nb.loss);
   else
