@@ -301,14 +301,16 @@ __host__ __device__ constexpr int end_planes() { return NDIM == 3 ? 3 : 1; }
 // Adds dw[t] (this lane's two channels) of all half warps of the block in
 // shared memory and then to the global gradient, float by float.
 template <int T>
-__device__ __forceinline__ void end_reduce(float *acc, const float2 *dw, float *gw) {
+__device__ __forceinline__ void end_reduce(float *acc, const uint64_t *dw, float *gw) {
   const int cl = (threadIdx.x & 15) * 2;
   for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) acc[i] = 0.f;
   __syncthreads();
 #pragma unroll
   for (int t = 0; t < T; ++t) {
-    atomicAdd(acc + t * kNetC + cl, dw[t].x);
-    atomicAdd(acc + t * kNetC + cl + 1, dw[t].y);
+    float a, b;
+    unpack2(dw[t], a, b);
+    atomicAdd(acc + t * kNetC + cl, a);
+    atomicAdd(acc + t * kNetC + cl + 1, b);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) atomicAdd(gw + i, acc[i]);
@@ -352,9 +354,9 @@ __global__ void __launch_bounds__(256, 2) net_last_bwd_k(const float *__restrict
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tiles_x = (sh.nx + kEndTX - 1) / kEndTX, tiles_y = (sh.ny + kEndTY - 1) / kEndTY;
   const int64_t items = (int64_t)sh.batch * sh.nz * tiles_y * tiles_x;
-  float2 dw[T];
+  uint64_t dw[T];  // two channels, packed
 #pragma unroll
-  for (int t = 0; t < T; ++t) dw[t] = make_float2(0.f, 0.f);
+  for (int t = 0; t < T; ++t) dw[t] = 0;
   float db = 0.f;
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
     const int tx = (int)(item % tiles_x);
@@ -416,20 +418,22 @@ __global__ void __launch_bounds__(256, 2) net_last_bwd_k(const float *__restrict
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const uint4 zw = zs[c];
-          float ga[8] = {};
+          uint64_t g2[4] = {};
 #pragma unroll
           for (int t = 0; t < T; ++t) {
-            const float4 wa = *reinterpret_cast<const float4 *>(w + t * kNetC + c * 8);
-            const float4 wb = *reinterpret_cast<const float4 *>(w + t * kNetC + c * 8 + 4);
-            ga[0] = fmaf(wa.x, S[t], ga[0]); ga[1] = fmaf(wa.y, S[t], ga[1]);
-            ga[2] = fmaf(wa.z, S[t], ga[2]); ga[3] = fmaf(wa.w, S[t], ga[3]);
-            ga[4] = fmaf(wb.x, S[t], ga[4]); ga[5] = fmaf(wb.y, S[t], ga[5]);
-            ga[6] = fmaf(wb.z, S[t], ga[6]); ga[7] = fmaf(wb.w, S[t], ga[7]);
+            const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(w + t * kNetC + c * 8);
+            const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(w + t * kNetC + c * 8 + 4);
+            const uint64_t st = pack2(S[t], S[t]);
+            g2[0] = fma2(wa.x, st, g2[0]);
+            g2[1] = fma2(wa.y, st, g2[1]);
+            g2[2] = fma2(wb.x, st, g2[2]);
+            g2[3] = fma2(wb.y, st, g2[3]);
           }
-          float zv[8];
+          float zv[8], ga[8];
           unpack8_bf16(zw, zv);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) ga[e] *= net_gelu_grad(zv[e]);
+          for (int e = 0; e < 4; ++e)
+            unpack2(mul2(g2[e], net_gelu_grad2(pack2(zv[2 * e], zv[2 * e + 1]))), ga[2 * e], ga[2 * e + 1]);
           dst[c] = pack8_bf16(ga);
         }
       }
@@ -440,13 +444,12 @@ __global__ void __launch_bounds__(256, 2) net_last_bwd_k(const float *__restrict
     const float *pg = tg + ((NZR / 2) * RH + row + 1) * kEndRow1 + xs + 1;
 #pragma unroll(NDIM == 3 ? 2 : 16)
     for (int i = 0; i < 16; ++i) {
-      const float gp = pg[i];  // (zero outside the grid)
+      const uint64_t gp = pack2(pg[i], pg[i]);  // (zero outside the grid)
 #pragma unroll
       for (int t = 0; t < T; ++t) {
         const int ox = t % 3, oy = (t / 3) % 3, dz = t / 9;
         const float2 a = ld_bf2(pa + ((dz * RH + oy) * kEndRow + i + ox) * 64);
-        dw[t].x = fmaf(a.x, gp, dw[t].x);
-        dw[t].y = fmaf(a.y, gp, dw[t].y);
+        dw[t] = fma2(pack2(a.x, a.y), gp, dw[t]);
       }
     }
   }
@@ -477,9 +480,9 @@ __global__ void __launch_bounds__(256, 2) net_first_wgrad_k(const float *__restr
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tiles_x = (sh.nx + kEndTX - 1) / kEndTX, tiles_y = (sh.ny + kEndTY - 1) / kEndTY;
   const int64_t items = (int64_t)sh.batch * sh.nz * tiles_y * tiles_x;
-  float2 dw[T], db = make_float2(0.f, 0.f);
+  uint64_t dw[T], db = 0;  // two channels, packed
 #pragma unroll
-  for (int t = 0; t < T; ++t) dw[t] = make_float2(0.f, 0.f);
+  for (int t = 0; t < T; ++t) dw[t] = 0;
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
     const int tx = (int)(item % tiles_x);
     int64_t r = item / tiles_x;
@@ -507,15 +510,14 @@ __global__ void __launch_bounds__(256, 2) net_first_wgrad_k(const float *__restr
     const float *pp = tp + row * kEndRow1 + xs;
 #pragma unroll(NDIM == 3 ? 2 : 16)
     for (int i = 0; i < 16; ++i) {
-      const float2 g = ld_bf2(pg + i * 64);  // (zero outside the grid)
-      db.x += g.x;
-      db.y += g.y;
+      const float2 gf = ld_bf2(pg + i * 64);  // (zero outside the grid)
+      const uint64_t g = pack2(gf.x, gf.y);
+      db = add2(db, g);
 #pragma unroll
       for (int t = 0; t < T; ++t) {
         const int ox = t % 3, oy = (t / 3) % 3, dz = t / 9;
         const float p = pp[(dz * RH + oy) * kEndRow1 + i + ox];
-        dw[t].x = fmaf(p, g.x, dw[t].x);
-        dw[t].y = fmaf(p, g.y, dw[t].y);
+        dw[t] = fma2(pack2(p, p), g, dw[t]);
       }
     }
   }

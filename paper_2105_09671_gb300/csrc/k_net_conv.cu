@@ -318,7 +318,9 @@ __global__ void __launch_bounds__(kCvThreads, CvGeom<NDIM>::MINB)
               float zv[8];
               unpack8_bf16(zw[c], zv);
 #pragma unroll
-              for (int e = 0; e < 8; ++e) zv[e] = v[8 * c + e] * net_gelu_grad(zv[e]);
+              for (int e = 0; e < 8; e += 2)
+                unpack2(mul2(pack2(v[8 * c + e], v[8 * c + e + 1]), net_gelu_grad2(pack2(zv[e], zv[e + 1]))),
+                        zv[e], zv[e + 1]);
               zw[c] = pack8_bf16(zv);
             }
             st_global32(d, zw[0], zw[1]);
