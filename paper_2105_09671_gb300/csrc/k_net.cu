@@ -207,78 +207,110 @@ __global__ void __launch_bounds__(256) net_last_fwd_k(const bf16 *__restrict__ a
 // Warp per face cell: g_{l-1} = (raw + ghost-cell gradients folded in) x
 // gelu'(z_{l-1}).  raw[p] = sum_t W[t]^T g[p - t] comes from the tensor-core
 // pass; a face cell also receives the gradient of each ghost cell that
-// replicates it.
+// replicates it: lane ci sums W[t][ci][co] g[p - t][co] over the taps that
+// read a cell of the grid.  Bound by latency: a warp meets 7 cells one after
+// the other at 32 x 256^2 pixels (30 us).  So the gradients of a plane's nine
+// taps are loaded together and shared through shared memory (one load at a
+// time, and a shuffle per value: 50 us), and the cells are enumerated in 32
+// bits (64-bit divisions: 41 us).
+constexpr int kFacesThreads = 512;
 template <int NDIM>
-__host__ __device__ constexpr int faces_smem() { return net_taps(NDIM) * kNetC * (kNetC + 1) * 4; }
+__host__ __device__ constexpr int faces_smem() {
+  return net_taps(NDIM) * kNetC * kNetC * 4 + kFacesThreads / 32 * 9 * kNetC * 4;
+}
 
 template <int NDIM>
-__global__ void __launch_bounds__(256) net_dgrad_faces_k(const float *__restrict__ raw,
-                                                         const bf16 *__restrict__ gpad,
-                                                         const float *__restrict__ params,
-                                                         int64_t w_off, NetShape sh,
-                                                         const bf16 *__restrict__ zprev,
-                                                         bf16 *__restrict__ gprevpad) {
-  constexpr int T = net_taps(NDIM), WS = kNetC + 1;  // (odd stride: lanes on different banks)
-  extern __shared__ float wsm[];                     // W[t][ci][co], WS floats per (t, ci)
-  for (int i = threadIdx.x; i < T * kNetC * kNetC; i += blockDim.x)
-    wsm[(i / kNetC) * WS + i % kNetC] = params[w_off + i];
+__global__ void __launch_bounds__(kFacesThreads) net_dgrad_faces_k(const float *__restrict__ raw,
+                                                                   const bf16 *__restrict__ gpad,
+                                                                   const float *__restrict__ params,
+                                                                   int64_t w_off, NetShape sh,
+                                                                   const bf16 *__restrict__ zprev,
+                                                                   bf16 *__restrict__ gprevpad) {
+  constexpr int T = net_taps(NDIM);
+  // W[t][ci][co], the four-float groups of a row at (group ^ ci % 8) so that
+  // eight lanes read eight different ones; then 9 x 32 gradients per warp
+  extern __shared__ __align__(16) float wsm[];
+  for (int i = threadIdx.x; i < T * kNetC * kNetC / 4; i += blockDim.x) {
+    const int ci = i / 8 % kNetC;
+    reinterpret_cast<float4 *>(wsm)[(i & ~7) + ((i ^ ci) & 7)] = reinterpret_cast<const float4 *>(params + w_off)[i];
+  }
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  float *gs = wsm + T * kNetC * kNetC + (threadIdx.x >> 5) * 9 * kNetC;
+  const int warps = (int)(gridDim.x * (blockDim.x >> 5));
   // face cells of an image: the rows on y and z faces whole, then the two end
-  // cells of the other rows
+  // cells of the other rows (in 32 bits: the layers' padded cells are fewer
+  // than 2^31)
   const int fy = min(sh.ny, 2), fz = NDIM == 3 ? min(sh.nz, 2) : 0, fx = min(sh.nx, 2);
-  const int64_t whole = ((int64_t)fz * sh.ny + (int64_t)(sh.nz - fz) * fy) * sh.nx;
-  const int64_t per = whole + (int64_t)(sh.nz - fz) * (sh.ny - fy) * fx;
-  for (int64_t u = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); u < per * sh.batch; u += warps) {
-    const int b = (int)(u / per);
-    int64_t f = u - b * per;
+  const int whole = (fz * sh.ny + (sh.nz - fz) * fy) * sh.nx;
+  const int per = whole + (sh.nz - fz) * (sh.ny - fy) * fx;
+  for (int64_t u = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < (int64_t)per * sh.batch; u += warps) {
+    const int b = (int)((uint32_t)u / (uint32_t)per);
+    int f = (int)((uint32_t)u % (uint32_t)per);
     int z, y, x;
     if (f < whole) {
-      x = (int)(f % sh.nx);
+      x = f % sh.nx;
       f /= sh.nx;
-      if (f < (int64_t)fz * sh.ny) {
+      if (f < fz * sh.ny) {
         z = f < sh.ny ? 0 : sh.nz - 1;
-        y = (int)(f % sh.ny);
+        y = f % sh.ny;
       } else {
-        f -= (int64_t)fz * sh.ny;
-        z = (NDIM == 3 ? 1 : 0) + (int)(f / fy);
+        f -= fz * sh.ny;
+        z = (NDIM == 3 ? 1 : 0) + f / fy;
         y = f % fy ? sh.ny - 1 : 0;
       }
     } else {
       f -= whole;
       x = f % fx ? sh.nx - 1 : 0;
       f /= fx;
-      z = (NDIM == 3 ? 1 : 0) + (int)(f / (sh.ny - fy));
-      y = 1 + (int)(f % (sh.ny - fy));
+      z = (NDIM == 3 ? 1 : 0) + f / (sh.ny - fy);
+      y = 1 + f % (sh.ny - fy);
     }
     const int64_t i = sh.u(b, z, y, x);
     float g = raw[i * kNetC + lane];
-    // ghost cells q (one cell outside the grid) with clamp(q) == p
-    for (int gz = (NDIM == 3 ? -1 : 0); gz <= (NDIM == 3 ? 1 : 0); ++gz)
-      for (int gy = -1; gy <= 1; ++gy)
-        for (int gx = -1; gx <= 1; ++gx) {
+    // ghost cells q (outside the grid by one) with clamp(q) == p
+    const int gx0 = x == 0 ? -1 : 0, gx1 = x == sh.nx - 1 ? 1 : 0;
+    const int gy0 = y == 0 ? -1 : 0, gy1 = y == sh.ny - 1 ? 1 : 0;
+    const int gz0 = NDIM == 3 && z == 0 ? -1 : 0, gz1 = NDIM == 3 && z == sh.nz - 1 ? 1 : 0;
+    for (int gz = gz0; gz <= gz1; ++gz)
+      for (int gy = gy0; gy <= gy1; ++gy)
+        for (int gx = gx0; gx <= gx1; ++gx) {
+          if (gx == 0 && gy == 0 && gz == 0) continue;
           const int qx = x + gx, qy = y + gy, qz = z + gz;
-          const bool out = qx < 0 || qx >= sh.nx || qy < 0 || qy >= sh.ny ||
-                           (NDIM == 3 && (qz < 0 || qz >= sh.nz));
-          if (!out) continue;
-          if (min(max(qx, 0), sh.nx - 1) != x || min(max(qy, 0), sh.ny - 1) != y) continue;
-          if (NDIM == 3 && min(max(qz, 0), sh.nz - 1) != z) continue;
           // gradient of the ghost cell q: sum_t W[t][ci = lane][co] g[q - t][co]
-          float acc = 0.f;
-          for (int t = 0; t < T; ++t) {
-            int oz, oy, ox;
-            net_tap(NDIM, t, oz, oy, ox);
-            const int sx = qx - ox, sy = qy - oy, sz = qz - oz;
-            if (sx < 0 || sx >= sh.nx || sy < 0 || sy >= sh.ny) continue;
+          uint64_t acc = 0;
+          for (int tz = 0; tz < T; tz += 9) {
+            const int sz = NDIM == 3 ? qz + 1 - tz / 9 : 0;
             if (NDIM == 3 && (sz < 0 || sz >= sh.nz)) continue;
-            const float gv = __bfloat162float(gpad[sh.ps(b, NDIM == 3 ? sz : 0, sy, sx, 0, 0, 0) * kNetC + lane]);
-            // lane holds g[.][co = lane]; W[t][ci = lane][co] needs all co
-#pragma unroll 8
-            for (int co = 0; co < kNetC; ++co)
-              acc = fmaf(wsm[(t * kNetC + lane) * WS + co], __shfl_sync(0xffffffffu, gv, co), acc);
+            bf16 gv[9] = {};
+            const bf16 *gq = gpad + sh.ps(b, sz, qy, qx, 0, 0, 0) * kNetC + lane;
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+              const int sx = qx + 1 - t % 3, sy = qy + 1 - t / 3;
+              if (sx >= 0 && sx < sh.nx && sy >= 0 && sy < sh.ny)
+                gv[t] = gq[((int64_t)(1 - t / 3) * sh.px() + (1 - t % 3)) * kNetC];
+            }
+            __syncwarp();
+#pragma unroll
+            for (int t = 0; t < 9; ++t) gs[t * kNetC + lane] = __bfloat162float(gv[t]);
+            __syncwarp();
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+              const int sx = qx + 1 - t % 3, sy = qy + 1 - t / 3;
+              if (sx < 0 || sx >= sh.nx || sy < 0 || sy >= sh.ny) continue;
+              const ulonglong2 *wr = reinterpret_cast<const ulonglong2 *>(wsm + ((tz + t) * kNetC + lane) * kNetC);
+              const ulonglong2 *gr = reinterpret_cast<const ulonglong2 *>(gs + t * kNetC);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                const ulonglong2 w = wr[k ^ (lane & 7)], v = gr[k];
+                acc = fma2(w.x, v.x, acc);
+                acc = fma2(w.y, v.y, acc);
+              }
+            }
           }
-          g += acc;
+          float even, odd;
+          unpack2(acc, even, odd);
+          g += even + odd;
         }
     const float zv = __bfloat162float(zprev[i * kNetC + lane]);
     gprevpad[sh.ps(b, z, y, x, 0, 0, 0) * kNetC + lane] = __float2bfloat16_rn(g * net_gelu_grad(zv));
@@ -643,7 +675,7 @@ static cudaError_t net_backward_t(const NetBuffers &nb, const NetShape &sh, cons
     e = net_conv_rows(1, nb.gz[l], nb.wd + (l - 1) * per, nullptr, sh, nullptr, nb.gz[l - 1], nb.raw,
                       nb.z[l - 1], nb.status, num_sms, s);
     if (e != cudaSuccess) return e;
-    net_dgrad_faces_k<NDIM><<<(int)std::min<int64_t>((n + 7) / 8, (int64_t)num_sms * (NDIM == 3 ? 2 : 4)), 256, faces_smem<NDIM>(), s>>>(
+    net_dgrad_faces_k<NDIM><<<(int)std::min<int64_t>((n + kFacesThreads / 32 - 1) / (kFacesThreads / 32), (int64_t)num_sms * (NDIM == 3 ? 1 : 2)), kFacesThreads, faces_smem<NDIM>(), s>>>(
         nb.raw, nb.gz[l], nb.params, L.w[l], sh, nb.z[l - 1], nb.gz[l - 1]);
   }
   net_first_wgrad_k<NDIM><<<(int)std::min<int64_t>(end_items, (int64_t)num_sms * occ_first), 256,
