@@ -32,25 +32,33 @@
 namespace ac {
 
 // ------------------------------------------------------------ first layer --
-// A thread per cell of a 32 x 8 block of one z (no index division), packed FP32
-// pairs of channels.
+// A thread per cell of a 32 x 8 tile of one z, packed FP32 pairs of channels;
+// a block takes one tile after another.  Bound by latency (the taps' loads, then
+// 16 chains of multiply-adds): three blocks to an SM in 80 registers, two where
+// that would spill.  1024^2 31 us (36 with 84 registers and two blocks), 32 x
+// 256^2 with the pre-activations 66 (81).  Weights in registers, a quarter of
+// the channels a lane, and cells marching along y: 41 and 87 us.
 template <int NDIM, bool TRAIN>
-__global__ void __launch_bounds__(256) net_first_fwd_k(const float *__restrict__ phi,
-                                                       const float *__restrict__ params,
-                                                       int64_t w_off, int64_t b_off, NetShape sh,
-                                                       bf16 *__restrict__ z1, bf16 *__restrict__ a1pad) {
+constexpr int first_blocks() { return NDIM == 3 && TRAIN ? 2 : 3; }
+
+template <int NDIM, bool TRAIN>
+__global__ void __launch_bounds__(256, first_blocks<NDIM, TRAIN>())
+    net_first_fwd_k(const float *__restrict__ phi, const float *__restrict__ params, int64_t w_off,
+                    int64_t b_off, NetShape sh, bf16 *__restrict__ z1, bf16 *__restrict__ a1pad) {
   constexpr int T = net_taps(NDIM);
   __shared__ __align__(16) float w[T * kNetC];
   __shared__ __align__(16) float bb[kNetC];
   for (int i = threadIdx.x; i < T * kNetC; i += blockDim.x) w[i] = params[w_off + i];
   if (threadIdx.x < kNetC) bb[threadIdx.x] = params[b_off + threadIdx.x];
   __syncthreads();
-  const int x = (int)blockIdx.x * 32 + (threadIdx.x & 31);
-  const int64_t planes = (int64_t)sh.batch * sh.nz;
-  if (x >= sh.nx) return;
-  for (int64_t bz = blockIdx.z; bz < planes; bz += gridDim.z)
-  for (int y = (int)blockIdx.y * 8 + (threadIdx.x >> 5); y < sh.ny; y += (int)gridDim.y * 8) {
-    const int b = (int)(bz / sh.nz), z = (int)(bz - (int64_t)b * sh.nz);
+  const uint32_t tiles_x = (uint32_t)(sh.nx + 31) / 32, tiles_y = (uint32_t)(sh.ny + 7) / 8;
+  const uint32_t tiles = tiles_x * tiles_y * (uint32_t)sh.batch * (uint32_t)sh.nz;
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const uint32_t r = tile / tiles_x, bz = r / tiles_y;
+    const int x = (int)(tile - r * tiles_x) * 32 + (threadIdx.x & 31);
+    const int y = (int)(r - bz * tiles_y) * 8 + (threadIdx.x >> 5);
+    if (x >= sh.nx || y >= sh.ny) continue;
+    const int b = NDIM == 2 ? (int)bz : (int)(bz / (uint32_t)sh.nz), z = NDIM == 2 ? 0 : (int)(bz - (uint32_t)b * sh.nz);
     uint64_t acc[kNetC / 2];
 #pragma unroll
     for (int c = 0; c < kNetC / 2; ++c) acc[c] = reinterpret_cast<const uint64_t *>(bb)[c];
@@ -620,14 +628,11 @@ static cudaError_t net_forward_t(const NetBuffers &nb, const NetShape &sh, const
   cudaError_t e = setup_attrs<NDIM>();
   if (e != cudaSuccess) return e;
   const NetLayout &L = nb.layout;
-  // first layer: about six blocks to an SM, each over several row tiles, as
-  // every block stages the weights first
-  const int fx = (sh.nx + 31) / 32, fy = (sh.ny + 7) / 8;
-  const int64_t planes = (int64_t)sh.batch * sh.nz;
-  const int64_t fz = std::min<int64_t>(planes, 65535);
-  const dim3 first_grid((unsigned)fx,
-                        (unsigned)std::min<int64_t>(fy, std::max<int64_t>(1, (int64_t)num_sms * 6 / (fx * fz) + 1)),
-                        (unsigned)fz);
+  // 32-bit tile and pixel indices, here as in the convolutions
+  if (sh.padded_cells() >= (int64_t)INT32_MAX) return cudaErrorInvalidValue;
+  const int64_t first_tiles = (int64_t)sh.batch * sh.nz * ((sh.nx + 31) / 32) * ((sh.ny + 7) / 8);
+  const int first_grid = (int)std::min<int64_t>(
+      first_tiles, (int64_t)num_sms * (train ? first_blocks<NDIM, true>() : first_blocks<NDIM, false>()));
   if (train)
     net_first_fwd_k<NDIM, true><<<first_grid, 256, 0, s>>>(phi, nb.params, L.w[0], L.b[0], sh, nb.z[0], nb.a[0]);
   else
