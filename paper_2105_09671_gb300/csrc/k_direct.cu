@@ -95,8 +95,9 @@ __device__ __forceinline__ void fx_store(double *row, int xl, int lane, int nx, 
 }
 
 // A warp owns kFx2W columns and marches over `chunk` rows.  Bound by integer
-// issue (some 140 instructions a cell, 14 of them wide multiply-adds): 4096^2
-// 253 -> 116 us a step, 2048^2 64 -> 32 against the FP64 operations.
+// issue (some 140 instructions a cell, 14 of them wide multiply-adds, which
+// take more than one slot: 63 % of the slots busy): 4096^2 253 -> 94 us a
+// step, 2048^2 64 -> 28 against the FP64 operations.
 __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__restrict__ src,
                                                            double *__restrict__ dst, GridParams g, int strips,
                                                            int chunk) {
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__re
 // A warp owns kFx3W columns of kFx3R rows and marches over `chunk` planes; it
 // takes apart kFx3R + 2 rows of each plane (against a barrier a plane to share
 // them; two rows in 124 registers rather than three or four in 160).  256^3
-// 317 -> 228 us a step, 200 x 100 x 100 45 -> 26.
+// 317 -> 159 us a step, 200 x 100 x 100 45 -> 23.
 __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restrict__ src,
                                                            double *__restrict__ dst, GridParams g, int strips,
                                                            int bands, int chunk) {
@@ -240,16 +241,48 @@ __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restr
   }
 }
 
+// Rows (planes) per item of a march.  An item converts two more rows than it
+// writes and starts with a wait for memory (together `pro` rows' time), and an
+// SM holds kFxOcc CTAs: with q CTAs to an SM a row of each takes one + add q us
+// up to one full round, with more of them `full` us a round.  So for every q
+// the most items that keep to it, and of these the cheapest (up to 24 CTAs to
+// an SM more than the fewest: there the starts of the items outweigh the rest).  Fitted to sweeps
+// over chunks for 64^3 .. 256^3 and 1152^2 .. 8192^2, where the choice is
+// within 4 % of the best.  One round of about 16 (2D: 24) warps an SM, rounded
+// to whole items, took 197 us against 159 at 256^3, whose CTAs it dealt 3.2 to
+// an SM, and 375 against 351 at 8192^2.
+struct FxMarch {
+  int occ;
+  double one, add, full, pro;
+};
+constexpr FxMarch kFxMarch2 = {6, 0.443, 0.314, 2.10, 0.91}, kFxMarch3 = {4, 0.705, 0.371, 2.07, 0.71};
+constexpr int kFxSms = 152;
+
+static int64_t fx_chunk(const FxMarch &m, int64_t columns, int64_t len) {
+  const int64_t q0 = (columns + kFxSms * kFxWarps - 1) / (kFxSms * kFxWarps);
+  double best[2] = {1e300, 1e300};  // one round; several
+  int64_t best_chunk[2] = {len, len};
+  for (int64_t qt = q0; qt < q0 + 24; ++qt) {
+    const int64_t chunk = (len + qt * kFxSms * kFxWarps / columns - 1) / (qt * kFxSms * kFxWarps / columns);
+    const int64_t warps = columns * ((len + chunk - 1) / chunk);
+    const int64_t q = (warps + kFxSms * kFxWarps - 1) / (kFxSms * kFxWarps);
+    const int64_t rounds = q / m.occ, rest = q % m.occ;
+    const double row = q <= m.occ ? m.one + m.add * (double)q
+                                  : m.full * (double)rounds + (rest ? m.one + m.add * (double)rest : 0.0);
+    const double cost = row * ((double)chunk + m.pro);
+    const int several = q > m.occ;
+    if (cost < best[several]) best[several] = cost, best_chunk[several] = chunk;
+    if (chunk == 1) break;
+  }
+  return best_chunk[best[1] < 0.97 * best[0]];  // the fit's own error
+}
+
 static cudaError_t direct_fx(int ndim, const GridParams &g, const double *src, double *dst, cudaStream_t s) {
-  // chunks of rows (planes) that give every SM about 16 warps (each chunk
-  // converts two more rows than it writes, so no shorter ones)
-  const int64_t kFxTarget = 152 * (ndim == 2 ? 24 : 16), kMin = 1;
   const int w = ndim == 2 ? kFx2W : kFx3W;
   const int64_t strips = (g.nx + w - 2 * kFxHalo - 1) / (w - 2 * kFxHalo);
   const int64_t bands = ndim == 2 ? 1 : (g.ny + kFx3R - 1) / kFx3R;
   const int64_t len = ndim == 2 ? g.ny : g.nz;
-  const int64_t chunks = std::max<int64_t>(1, std::min(kFxTarget / std::max<int64_t>(1, strips * bands), len / kMin));
-  const int64_t chunk = (len + chunks - 1) / chunks;
+  const int64_t chunk = fx_chunk(ndim == 2 ? kFxMarch2 : kFxMarch3, strips * bands, len);
   const int64_t warps = strips * bands * ((len + chunk - 1) / chunk);
   const unsigned blocks = (unsigned)((warps + kFxWarps - 1) / kFxWarps);
   if (ndim == 2) step2d_fx<<<blocks, kFxWarps * 32, 0, s>>>(src, dst, g, (int)strips, (int)chunk);
