@@ -10,8 +10,8 @@
 //            from 32 x 32 -> 64-bit multiply-adds on balanced halves,
 //   phi'     = phi + beta lap + alpha (phi - phi^3), rounded once to FP64.
 // Against 128-bit arithmetic its error is smaller than that of the FP64
-// operations (fused as in ac_update): 0.4 to 0.87 of their rms error and 0.16
-// to 0.75 of their largest one, for amplitudes 1e-6 .. 1.2, alpha 0.0004 ..
+// operations (fused as in ac_update): 0.40 to 0.80 of their rms error and 0.16
+// to 0.63 of their largest one, for amplitudes 1e-6 .. 1.2, alpha 0.0004 ..
 // 0.6, 2D and 3D, rough and smooth stencils.  +-1 and 0 stay exact fixed
 // points and mirrored fields stay mirrored bit for bit.  A cell whose stencil
 // holds a value of 1.25 or more in size (fields of the scheme have |phi| <= 1),

@@ -28,16 +28,17 @@ constexpr B2Variant kB2[] = {
     {4, 7, 64, 1.49, 1.81, 0.131, 0.0363},
     {4, 8, 112, 1.13, 2.15, 0.005, 0.0404},
     {4, 9, 64, 2.18, 1.41, 0.207, 0.0476},  // FP16 storage
-    // FP64 (block2d_fx.cuh): two rows a lane for the smallest grids (200^2 1.42
-    // us a step against 1.66 with four), four from 512^2 on (3.56 against 4.14)
-    {1, 2, 32, 1.30, 1.37, 0.0, 0.0632},
-    {1, 4, 56, 2.09, 0.97, 0.629, 0.1161},
+    // FP64 (block2d_fx.cuh): two rows a lane for the smallest grids (200^2 1.29
+    // us a step against 1.49 with four), four from 512^2 on (3.18 against 3.69)
+    {1, 2, 32, 0.84, 2.06, 0.0, 0.0514},
+    {1, 4, 56, 2.20, 1.16, 0.432, 0.0973},
 };
 constexpr int kB2Count = sizeof(kB2) / sizeof(kB2[0]);
 
-// A step of the marching FP64 kernel (k_direct.cu) on GB300: 11.7, 32 and 116
-// us at 1024^2, 2048^2 and 4096^2.
-double march_cost(int64_t nx, int64_t ny) { return 3.5 + 6.7e-6 * (double)nx * (double)ny; }
+// A step of the marching FP64 kernel (k_direct.cu) on GB300: 11.1, 13.4, 27.6
+// and 94.2 us at 1024^2, 1280^2, 2048^2 and 4096^2, where tiles take 9.7 and
+// 13.8 us at the first two.
+double march_cost(int64_t nx, int64_t ny) { return 5.0 + 5.45e-6 * (double)nx * (double)ny; }
 
 bool offered(const B2Variant &b, int dtype) {
   return dtype == AC_F64 ? b.E == 1 : b.E == 4 && (b.R != 9 || dtype == AC_F16S);

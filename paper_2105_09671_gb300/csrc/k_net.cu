@@ -374,9 +374,11 @@ __host__ __device__ constexpr int last_bwd_smem() {
 // grid): the cell at p - t, and per axis, where p is a face cell, the cell
 // at offset 0 once more for the tap that points out of the grid.
 // Second pass: dW6[t][c] += a5[p + t][c] g6[p] from the staged a5.
-// Bound by instruction issue (about 9 + 9 multiply-adds and a gelu' per cell
-// and channel).  One warp per cell with every operand read from global memory
-// took 2818 us for 32 x 256^2 cells.
+// Bound by instruction issue and latency (about 9 + 9 multiply-adds and a
+// gelu' per cell and channel, on two channels an instruction; 16 warps to an SM
+// in 128 registers).  32 x 256^2 cells: 155 us; with scalar arithmetic 196, the
+// copies not asynchronous 245, one warp per cell and every operand read from
+// global memory 2818.
 template <int NDIM>
 __global__ void __launch_bounds__(256, 2) net_last_bwd_k(const float *__restrict__ g6,
                                                          const float *__restrict__ params, int64_t w_off,

@@ -22,7 +22,7 @@
 // ~48 clocks) and the L2 reads (192 bytes a pixel, a rows twice).  The kernel
 // before this one built the operands with 2-byte shared-memory stores by all
 // threads, one chunk at a time, waiting for each MMA: 32 x 256^2 pixels took
-// 2809 us a layer.
+// 2809 us a layer, this one 72 (272 MB from DRAM: 40 us at the copy rate).
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs, warps 2 and 3 sum g for the
 // bias; all four add the accumulators to the global gradient at the end.

@@ -227,8 +227,9 @@ __device__ __forceinline__ uint64_t net_gelu_fast2(uint64_t x) {
 // and s = 1 / (1 + e), tanh u = 2 s - 1 and 1 - tanh^2 u = 4 s (e s), so
 //   gelu'(x) = (1 + t) / 2 + x/2 (1 - t^2) u' = s + 2 x u' s (e s),
 // in which nothing cancels: against FP64 over [-10, 10] its error is at most
-// 2.1e-7 (2.9e-8 rms), that of the form with tanhf 5.6e-7 (1.1e-7 rms).  e is 2^y with the factor
-// -2 log2(e) in u's coefficients; the exponent's bound keeps e s finite.
+// 2.1e-7 (2.9e-8 rms), that of the form with tanhf 5.6e-7 (1.1e-7 rms).  e is
+// 2^y with the factor -2 log2(e) in u's coefficients; the exponent's bound
+// keeps e s finite.
 __device__ __forceinline__ float net_exp2(float y) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fminf(y, 125.0f)));
@@ -246,7 +247,8 @@ __device__ __forceinline__ float net_gelu_grad(float x) {
   const float s = net_rcp(1.0f + e);
   return fmaf(x * fmaf(6.0f * k * c, x2, 2.0f * k), s * (e * s), s);
 }
-// The same on two values, packed.
+// The same on two values, packed: the data gradient's kernel takes 85 us with
+// it, 115 with the scalar form (32 x 256^2 pixels).
 __device__ __forceinline__ uint64_t net_gelu_grad2(uint64_t x) {
   const float k = 0.7978845608028654f, l2e = 1.4426950408889634f, c = 0.044715f;
   const float a1 = -2.0f * k * l2e * c, a0 = -2.0f * k * l2e, b1 = 6.0f * k * c, b0 = 2.0f * k;
