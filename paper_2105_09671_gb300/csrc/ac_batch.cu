@@ -45,7 +45,7 @@ struct ac_batch {
   std::vector<void *> phi, ws;
   int k = 0;            // plan depth (0 = default)
   int tile = 0;         // strip width (0: default strips, 1: 8-cell FP32 strips)
-  int chunk_rows = 64;  // rows per work item
+  int chunk_rows = 0;   // rows per work item (chosen with the items)
   bool items_valid = false;
   int items_k = -1, items_tile = -1;
   // host / device tables
@@ -85,6 +85,32 @@ static void release_graph(ac_batch *b) {
   b->graph = nullptr;
 }
 
+// Rows of a work item.  A step-block takes as long as the longer of two: an
+// item from end to end (an instance's next block waits for it), which grows
+// with its rows, or all items over the resident warps, which falls with them
+// (every item computes 2k halo rows more and fills its pipeline).  They meet
+// where there are about 1.25 items to a warp, so the fewest rows (a multiple of
+// 4, at least 8) that keep to it; on large batches, where no size does, 256.
+// FP32, 64 rows always -> this: 16 grids to 256^2 27 -> 11 us a block, 32 of
+// 256^2 to 512^2 36 -> 20, 64 to 1024^2 66 -> 65, 512 to 1024^2 449 -> 395;
+// FP16 storage alike.  FP64 is bound by arithmetic at any size and wants many
+// items to share out evenly: 64 rows at most (64 grids to 1024^2: 1.95 ms a
+// block against 2.15 with 1.25 items to a warp; 16 to 256^2 0.74 -> 0.13).
+static int rows_per_item(const ac_batch *b, int ow, int64_t warps) {
+  auto items = [&](int64_t rows) {
+    int64_t n = 0;
+    for (const ac_grid_desc &d : b->d) n += ((d.nx + ow - 1) / ow) * ((d.ny + rows - 1) / rows);
+    return n;
+  };
+  int lo = 2, hi = b->dtype == AC_F64 ? 16 : 64;  // in units of 4 rows
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (items(4 * mid) * 4 <= warps * 5) hi = mid;
+    else lo = mid + 1;
+  }
+  return 4 * lo;
+}
+
 // Work items for plan depth k: per instance, strips of the 2D streaming
 // kernel (halo HX(k)) times row chunks, each with its 3 x 3 neighbourhood.
 static int build_items(ac_batch *b, int k) {
@@ -93,6 +119,10 @@ static int build_items(ac_batch *b, int k) {
   release_graph(b);
   int sw, hx, ow, vec;
   batch_strip_geom(b->dtype, k, b->tile, &sw, &hx, &ow, &vec);
+  int ctas = 0;  // of the launch (no steps: only the grid's size)
+  BC_CUDA(batch2d_launch(b->dtype, b->tile, nullptr, nullptr, 0, nullptr, nullptr, nullptr, 0, nullptr, 0,
+                         b->num_sms, b->stream, &ctas));
+  b->chunk_rows = rows_per_item(b, ow, (int64_t)ctas * kBatchWarps);
   b->h_items.clear();
   for (int i = 0; i < b->count; ++i) {
     const ac_grid_desc &d = b->d[i];

@@ -26,6 +26,7 @@
 namespace ac {
 
 static_assert(kBatchBoxRows == kS2Rows, "batch tensor maps use the 2D kernel's box");
+static_assert(kBatchWarps == kS2Warps, "resident warps");
 
 __device__ __forceinline__ int ld_acquire(const int *p) {
   int v;
@@ -160,6 +161,7 @@ cudaError_t batch2d_launch_t(const BInst *insts, const BItem *items, int n_items
   // every CTA of the grid must be resident at once (the waits rely on it)
   const int blocks = std::max(1, num_sms) * occ;
   if (grid_out) *grid_out = blocks;
+  if (total == 0) return cudaSuccess;
   batch2d_k<T, VPL><<<blocks, kS2Warps * 32, BatchGeom<T, VPL>::SMEM, s>>>(
       insts, items, n_items, maps, progress, ticket, total, status, wait_limit);
   return cudaGetLastError();

@@ -27,6 +27,7 @@ struct BItem {
 constexpr int kBatchKMax = 4;      // depths of the default strips (tile 0)
 constexpr int kBatchKMaxWide = 6;  // depths of the 8-cell FP32 strips (tile 1)
 constexpr int kBatchBoxRows = 2;   // rows per TMA box (equals the 2D kernel's)
+constexpr int kBatchWarps = 8;     // warps per CTA (equals the 2D kernel's)
 
 // tile 0: the storage type's default strips; tile 1: FP32 strips of two
 // 16-byte vectors per lane (as tile 1 of the single-grid 2D stepper)
@@ -34,6 +35,7 @@ inline int batch_kmax(int dtype, int tile) {
   return tile == 0 ? kBatchKMax : (tile == 1 && dtype == AC_F32 ? kBatchKMaxWide : 0);
 }
 
+// total = 0: nothing is launched, only *grid_out is set.
 cudaError_t batch2d_launch(int dtype, int tile, const BInst *insts, const BItem *items, int n_items,
                            const CUtensorMap *maps, int *progress, unsigned long long *ticket,
                            long long total, int *status, uint32_t wait_limit, int num_sms,
