@@ -612,14 +612,14 @@ __global__ void net_pack_k(const float *__restrict__ params, int T, int64_t w0, 
 // default, once per device (thread-safe; the occupancy query is unused).
 template <int NDIM>
 static cudaError_t setup_attrs() {
-  static KernelSetup k_last_t, k_last_f, k_dfin;
+  static KernelSetup k_last_t, k_last_f, k_faces;
   int occ = 0;
   cudaError_t e;
   e = kernel_setup(k_last_t, (const void *)net_last_fwd_k<NDIM, true>, 32, last_smem_bytes<NDIM>(), &occ);
   if (e != cudaSuccess) return e;
   e = kernel_setup(k_last_f, (const void *)net_last_fwd_k<NDIM, false>, 32, last_smem_bytes<NDIM>(), &occ);
   if (e != cudaSuccess) return e;
-  return kernel_setup(k_dfin, (const void *)net_dgrad_faces_k<NDIM>, 32,
+  return kernel_setup(k_faces, (const void *)net_dgrad_faces_k<NDIM>, 32,
                       faces_smem<NDIM>(), &occ);
 }
 
