@@ -109,3 +109,22 @@ def test_a_step_is_no_less_exact_than_fp64_operations(shape, amp, smooth):
     native = (p + beta * (s - 2 * p.ndim * p)) + alpha * (p - p * p * p)
     rms = lambda a: float(np.sqrt(np.mean(((a - exact).astype(np.float64)) ** 2)))
     assert rms(out) <= rms(native), f"{rms(out):.3e} against {rms(native):.3e}"
+
+
+@pytest.mark.parametrize("shape", [(200, 197, 203), (3001, 3100), (7, 1030, 130), (2, 600, 1300)])
+def test_marches_of_several_rounds_give_the_same_bits(shape):
+    # items of a warp each, in several rounds of the resident CTAs (the first
+    # two) and in one; the last item is shorter than the others
+    h = 1.0 / max(shape)
+    a = oracle.init_random(shape, seed=11)
+    got = []
+    for variant in (ac.AC_VARIANT_DIRECT, ac.AC_VARIANT_STREAM):
+        sim = ac.Simulation(shape, h, 2.5 * h, 0.1 * h * h, dtype="f64")
+        try:
+            sim.load(a)
+            sim.set_schedule(variant, 1)
+            sim.step(3)
+            got.append(sim.to_numpy())
+        finally:
+            sim.close()
+    assert np.array_equal(*got)
