@@ -49,7 +49,7 @@ enum {
 /* ------------------------------------------------------ storage types ---- */
 typedef enum {
   AC_F64 = 0,  /* FP64 storage, FP64 arithmetic (or 64-bit integer
-                  arithmetic of smaller error, see fixed64.cuh)          */
+                  arithmetic of no larger error, see fixed64.cuh)        */
   AC_F32 = 1,  /* FP32 storage, FP32 arithmetic                        */
   AC_F16S = 2  /* FP16 storage (IEEE binary16), FP32 arithmetic; values
                   are rounded to nearest-even only when written to memory */

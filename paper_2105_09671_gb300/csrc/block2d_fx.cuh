@@ -56,19 +56,24 @@ __global__ void __launch_bounds__(kB2FxMaxWarps * 32)
     hi.m = sm[ia];
     hi.e = se[ia];
     double nv[R];
+    uint32_t fp64 = 0;  // rows whose cell takes the FP64 operations
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const FxV w = fx_shfl<-1>(f[r]), ea = fx_shfl<1>(f[r]);
       const FxV &b = r == 0 ? lo : f[r > 0 ? r - 1 : 0], &a = r == R - 1 ? hi : f[r + 1 < R ? r + 1 : 0];
       const int m = max(max(max(w.e, ea.e), max(b.e, a.e)), f[r].e);
-      const bool in = coef.fx && fx_in_range(m);
       const int64_t ns = (fx_align(w, m) + fx_align(ea, m)) + (fx_align(b, m) + fx_align(a, m));
-      nv[r] = fx_update<2>(f[r], ns, m, coef);
-      if (__any_sync(0xffffffffu, !in)) {  // some cell of the row takes the FP64 operations
+      if (!(fx_update<2>(f[r], ns, m, coef, &nv[r]) && coef.fx)) fp64 |= 1u << r;
+    }
+    const uint32_t any = __reduce_or_sync(0xffffffffu, fp64);
+    if (any) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if (!((any >> r) & 1u)) continue;
         const double vw = __shfl_up_sync(0xffffffffu, v[r], 1), ve = __shfl_down_sync(0xffffffffu, v[r], 1);
         const double vb = r == 0 ? sv[ib] : v[r > 0 ? r - 1 : 0], va = r == R - 1 ? sv[ia] : v[r + 1 < R ? r + 1 : 0];
         const double t = ac_update<double>(v[r], (vw + ve) + (vb + va), -4.0, coef.alpha, coef.beta);
-        nv[r] = in ? nv[r] : t;
+        if ((fp64 >> r) & 1u) nv[r] = t;
       }
     }
 #pragma unroll

@@ -130,22 +130,24 @@ __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__re
       fx_load<kFx2E>(src + (int64_t)reflect(y + 2, ny) * g.pitch, xl, xi, inside, v);
     const FxV left = fx_shfl<-1>(x[kFx2E - 1]), right = fx_shfl<1>(x[0]);
     double out[kFx2E];
+    bool ok[kFx2E], all = true;
 #pragma unroll
     for (int e = 0; e < kFx2E; ++e) {
       const FxV &w = e == 0 ? left : x[e - 1], &ea = e == kFx2E - 1 ? right : x[e + 1];
       const int m = max(max(max(w.e, ea.e), max(below[e].e, up[e].e)), x[e].e);
-      if (fx_in_range(m)) {
-        const int64_t ns =
-            (fx_align(w, m) + fx_align(ea, m)) + (fx_align(below[e], m) + fx_align(up[e], m));
-        out[e] = fx_update<2>(x[e], ns, m, coef);
-      } else {
-        // the FP64 operations, from memory
+      const int64_t ns = (fx_align(w, m) + fx_align(ea, m)) + (fx_align(below[e], m) + fx_align(up[e], m));
+      ok[e] = fx_update<2>(x[e], ns, m, coef, &out[e]);
+      all = all && ok[e];
+    }
+    if (!all) {  // some take the FP64 operations, from memory
+      const double *row = src + (int64_t)y * g.pitch;
+      const double *rs = src + (int64_t)max(y - 1, 0) * g.pitch, *rn = src + (int64_t)min(y + 1, ny - 1) * g.pitch;
+#pragma unroll
+      for (int e = 0; e < kFx2E; ++e) {
+        if (ok[e]) continue;
         const int im = xi[e] > 0 ? xi[e] - 1 : 0, ip = min(xi[e] + 1, nx - 1);
-        const double *row = src + (int64_t)y * g.pitch;
-        out[e] = ac_update<double>(row[xi[e]],
-                                   (row[im] + row[ip]) + (src[(int64_t)max(y - 1, 0) * g.pitch + xi[e]] +
-                                                          src[(int64_t)min(y + 1, ny - 1) * g.pitch + xi[e]]),
-                                   -4.0, coef.alpha, coef.beta);
+        out[e] = ac_update<double>(row[xi[e]], (row[im] + row[ip]) + (rs[xi[e]] + rn[xi[e]]), -4.0, coef.alpha,
+                                   coef.beta);
       }
     }
     fx_store<kFx2E>(dst + (int64_t)y * g.pitch, xl, lane, nx, out);
@@ -211,26 +213,31 @@ __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restr
     for (int r = 0; r < R; ++r) {
       const FxV left = fx_shfl<-1>(x[r + 1][E - 1]), right = fx_shfl<1>(x[r + 1][0]);
       double out[E];
+      bool ok[E], all = true;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const FxV &p = x[r + 1][e], &w = e == 0 ? left : x[r + 1][e - 1],
                   &ea = e == E - 1 ? right : x[r + 1][e + 1];
         const FxV &s = x[r][e], &n = x[r + 2][e], &lo = below[r][e], &hi = up[r + 1][e];
         const int m = max(max(max(max(w.e, ea.e), max(s.e, n.e)), max(lo.e, hi.e)), p.e);
-        if (fx_in_range(m)) {
-          const int64_t ns = ((fx_align(w, m) + fx_align(ea, m)) + (fx_align(s, m) + fx_align(n, m))) +
-                             (fx_align(lo, m) + fx_align(hi, m));
-          out[e] = fx_update<3>(p, ns, m, coef);
-        } else {
+        const int64_t ns = ((fx_align(w, m) + fx_align(ea, m)) + (fx_align(s, m) + fx_align(n, m))) +
+                           (fx_align(lo, m) + fx_align(hi, m));
+        ok[e] = fx_update<3>(p, ns, m, coef, &out[e]);
+        all = all && ok[e];
+        below[r][e] = p;
+      }
+      if (!all) {  // some take the FP64 operations, from memory
+        const double *pl = src + (int64_t)z * plane, *row = pl + ro[r + 1];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          if (ok[e]) continue;
           const int im = xi[e] > 0 ? xi[e] - 1 : 0, ip = min(xi[e] + 1, nx - 1);
-          const double *pl = src + (int64_t)z * plane, *row = pl + ro[r + 1];
           out[e] = ac_update<double>(
               row[xi[e]],
               ((row[im] + row[ip]) + (pl[ro[r] + xi[e]] + pl[ro[r + 2] + xi[e]])) +
                   (src[(int64_t)max(z - 1, 0) * plane + ro[r + 1] + xi[e]] + zp[ro[r + 1] + xi[e]]),
               -6.0, coef.alpha, coef.beta);
         }
-        below[r][e] = p;
       }
       if (y0 + r < ny) fx_store<E>(dst + (int64_t)z * plane + (int64_t)(y0 + r) * g.pitch, xl, lane, nx, out);
     }

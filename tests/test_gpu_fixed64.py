@@ -128,3 +128,92 @@ def test_marches_of_several_rounds_give_the_same_bits(shape):
         finally:
             sim.close()
     assert np.array_equal(*got)
+
+
+# fields whose small cells have large neighbours: fronts that cross zero close
+# to cell centres, planar and slightly tilted, and rough noise
+def _crossing_field(shape, seed):
+    rng = np.random.default_rng(seed)
+    x = np.arange(shape[-1], dtype=np.float64)
+    rows = int(np.prod(shape[:-1]))
+    off = 10.0 ** rng.uniform(-9, -0.3, rows) * rng.choice([-1.0, 1.0], rows)
+    if seed % 2 == 0:
+        off = off[0] + 1e-4 * np.sin(np.arange(rows) * 0.1)
+    mid = shape[-1] // 2
+    return np.tanh((x[None, :] - mid + off[:, None]) / 3.0).reshape(shape)
+
+
+def _axis_neighbours(p):
+    out = []
+    for ax in reversed(range(p.ndim)):  # x, y, z
+        n = p.shape[ax]
+        out.append(np.take(p, np.maximum(np.arange(n) - 1, 0), axis=ax))
+        out.append(np.take(p, np.minimum(np.arange(n) + 1, n - 1), axis=ax))
+    return out
+
+
+@pytest.mark.parametrize("shape", [(24, 40), (5, 6, 40)])
+@pytest.mark.parametrize("kind", [0, 1, "rough"])
+def test_cells_of_every_size_are_no_less_exact_than_fp64_operations(shape, kind):
+    # against exact rationals, cells binned by their result's size relative to
+    # the stencil's largest value; the baseline is ac_update with its fused
+    # operations, each rounded once
+    from fractions import Fraction as Q
+    h = 1.0 / 64
+    eps, dt = 2.5 * h, 0.1 * h * h
+    phi0 = 0.1 * wl.random_field(shape, seed=4) if kind == "rough" else _crossing_field(shape, kind)
+    out = gpu_run(phi0, h, eps, dt, 1, "f64", ac.AC_VARIANT_DIRECT, 1).reshape(-1)
+    alpha, beta = dt / (eps * eps), dt / (h * h)
+    nb = [a.reshape(-1) for a in _axis_neighbours(phi0)]
+    p = phi0.reshape(-1)
+    m2d = -2 * phi0.ndim
+    bins = {}
+    for i in range(p.size):
+        v = [float(a[i]) for a in nb]
+        c = float(p[i])
+        exact = Q(c) + Q(beta) * (sum(map(Q, v)) + m2d * Q(c)) + Q(alpha) * (Q(c) - Q(c) ** 3)
+        ns = (v[0] + v[1]) + (v[2] + v[3])
+        if phi0.ndim == 3:
+            ns += v[4] + v[5]
+        lap = float(Q(m2d) * Q(c) + Q(ns))
+        re = float(Q(-c * c) * Q(c) + Q(c))
+        fused = float(Q(alpha) * Q(re) + Q(float(Q(beta) * Q(lap) + Q(c))))
+        top = max(abs(c), max(map(abs, v)))
+        b = min(14, int(-np.log2(abs(float(exact)) / top))) if exact else 14
+        e = bins.setdefault(b // 2, [0, 0.0, 0.0])
+        e[0] += 1
+        e[1] += float(Q(float(out[i])) - exact) ** 2
+        e[2] += float(Q(fused) - exact) ** 2
+    assert len(bins) > 1
+    for b, (n, mine, base) in sorted(bins.items()):
+        if n >= 20:
+            assert mine <= base, f"2^-{2 * b}: {np.sqrt(mine / n):.3e} against {np.sqrt(base / n):.3e} ({n} cells)"
+
+
+@pytest.mark.parametrize("shape", [(24, 40), (130, 249), (515, 517), (5, 6, 40), (65, 64, 66)])
+@pytest.mark.parametrize("kind", [0, 1, "rough", "large"])
+def test_negated_fields_step_to_the_negated_result(shape, kind):
+    h = 1.0 / 64
+    eps, dt = 2.5 * h, 0.1 * h * h
+    if kind in (0, 1):
+        phi0 = _crossing_field(shape, kind)
+    else:
+        phi0 = (3.0 if kind == "large" else 0.1) * wl.random_field(shape, seed=4)
+        dt *= 0.2 if kind == "large" else 1.0
+    phi0.reshape(-1)[7:9] = [0.0, -0.0]
+    for v, k in ((None, None), (ac.AC_VARIANT_DIRECT, 1), (ac.AC_VARIANT_STREAM, 2)):
+        a = gpu_run(phi0, h, eps, dt, 6, "f64", v, k) if v is not None else gpu_run(phi0, h, eps, dt, 6, "f64")
+        b = gpu_run(-phi0, h, eps, dt, 6, "f64", v, k) if v is not None else gpu_run(-phi0, h, eps, dt, 6, "f64")
+        assert np.array_equal(a, -b), f"{shape} {kind} schedule {v} {k}"
+
+
+@pytest.mark.parametrize("shape,n", [((16, 16), 2000), ((40, 64), 600), ((520, 510), 100), ((4, 6, 64), 600)])
+def test_a_field_odd_about_its_middle_stays_so(shape, n):
+    h = 1.0 / 64
+    x = np.arange(shape[-1]) - (shape[-1] - 1) / 2
+    phi0 = np.broadcast_to(np.tanh(x / 3.0), shape).copy()
+    phi0 += np.broadcast_to(1e-3 * np.sin(x), shape)
+    phi0 = 0.5 * (phi0 - phi0[..., ::-1])
+    assert np.array_equal(phi0, -phi0[..., ::-1])
+    out = gpu_run(phi0, h, 2.5 * h, 0.1 * h * h, n, "f64")
+    assert np.array_equal(out, -out[..., ::-1])
