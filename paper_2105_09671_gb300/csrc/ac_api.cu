@@ -221,6 +221,7 @@ extern "C" int ac_create(const ac_grid_desc *desc, void *phi_dev, void *workspac
   c->gp.pitch = desc->pitch_x;
   c->gp.alpha = desc->dt / (desc->eps * desc->eps);
   c->gp.beta = desc->dt / (desc->h * desc->h);
+  if (desc->dtype == AC_F64) c->gp.fx = fx_coef(c->gp.alpha, c->gp.beta);
   cudaError_t e = cudaMalloc(&c->d_status, sizeof(int));
   if (e == cudaSuccess) e = observe_alloc(&c->d_partials, c->stream);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_out, sizeof(double) * 4);
@@ -407,7 +408,7 @@ bool ac_plan_depths(int64_t n, int k, std::vector<int> &depths) {
 static bool takes_stand_in(const ac_ctx *c, int variant, int k, int tile) {
   if (c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO) return false;
   if (c->d.ndim == 3 && !step3d_vec_serves(c->d.dtype, c->gp)) return false;
-  if (c->d.dtype == AC_F64 && !fx_coefficients(c->gp.alpha, c->gp.beta)) return false;
+  if (c->d.dtype == AC_F64 && !c->gp.fx.on) return false;
   int dv, dk;
   default_schedule(c, &dv, &dk);
   return variant == dv && k == dk && tile == default_tile(c, dk);

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "batch_types.h"
+#include "fixed64.cuh"
 
 using namespace ac;
 
@@ -214,6 +215,7 @@ extern "C" int ac_batch_create(const ac_grid_desc *descs, void *const *phi_devs,
     in.pitch = descs[i].pitch_x;
     in.alpha = descs[i].dt / (descs[i].eps * descs[i].eps);
     in.beta = descs[i].dt / (descs[i].h * descs[i].h);
+    if (b->dtype == AC_F64) in.fx = fx_coef(in.alpha, in.beta);
   }
   // per-instance tensor maps of phi and workspace (box SW x rows, zero fill)
   // for each strip width the storage type offers; over-aligned type: a

@@ -54,8 +54,8 @@ __device__ __forceinline__ bool batch_item(const S2Ring<T> &ring, uint32_t &u, c
                                            T *dst, const S2Item &si, const BInst &in, int *status) {
   using C = typename Traits<T>::C;
   if (in.fastx)
-    return s2_item<T, D, true, VPL>(ring.smem, ring.bars, u, map, dst, si, Coef<C>(in.alpha, in.beta), status);
-  return s2_item<T, D, false, VPL>(ring.smem, ring.bars, u, map, dst, si, Coef<C>(in.alpha, in.beta), status);
+    return s2_item<T, D, true, VPL>(ring.smem, ring.bars, u, map, dst, si, Coef<C>(in), status);
+  return s2_item<T, D, false, VPL>(ring.smem, ring.bars, u, map, dst, si, Coef<C>(in), status);
 }
 
 // VPL: 16-byte vectors per lane of every strip (the storage type's default,

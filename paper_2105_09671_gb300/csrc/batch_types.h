@@ -11,6 +11,7 @@ struct BInst {
   int nx, ny;
   int64_t pitch;
   double alpha, beta;
+  FxCoef fx;             // of FP64 instances
   int S;                 // step-blocks of the current plan
   int k;                 // depth of step-blocks before tail_start
   int tail_start;        // first step-block whose depth comes from tail[]

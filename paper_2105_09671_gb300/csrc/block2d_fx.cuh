@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kB2FxMaxWarps * 32)
   const int nx = (int)g.nx, ny = (int)g.ny;
   const int x0 = (int)blockIdx.x * (32 - 2 * k) - k, y0 = (int)blockIdx.y * (nw * R - 2 * k) - k;
   const int x = x0 + lane, yr = y0 + warp * R;
-  const Coef<double> coef(g.alpha, g.beta);
+  const Coef<double> coef(g);
   // The previous launch on the stream writes what this one reads.
   pdl_wait();
   double v[R];
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kB2FxMaxWarps * 32)
       const FxV &b = r == 0 ? lo : f[r > 0 ? r - 1 : 0], &a = r == R - 1 ? hi : f[r + 1 < R ? r + 1 : 0];
       const int m = max(max(max(w.e, ea.e), max(b.e, a.e)), f[r].e);
       const int64_t ns = (fx_align(w, m) + fx_align(ea, m)) + (fx_align(b, m) + fx_align(a, m));
-      if (!(fx_update<2>(f[r], ns, m, coef, &nv[r]) && coef.fx)) fp64 |= 1u << r;
+      if (!fx_update<2>(f[r], ns, m, coef, &nv[r])) fp64 |= 1u << r;
     }
     const uint32_t any = __reduce_or_sync(0xffffffffu, fp64);
     if (any) {

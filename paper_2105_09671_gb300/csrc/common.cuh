@@ -126,10 +126,18 @@ __device__ __forceinline__ C ac_update(C p, C nsum, C minus_2d, C alpha, C beta)
 }
 
 // ----------------------------------------------------------- parameters ---
+// alpha 2^63 and beta 2^65 as hi 2^32 + lo, lo signed (fixed64.cuh); on is 0
+// where they don't fit (alpha near 1, beta at the 2D stability limit), which
+// leaves every cell to the FP64 operations.
+struct FxCoef {
+  int ah, al, bh, bl, on;
+};
+
 struct GridParams {
   int64_t nx, ny, nz;
   int64_t pitch;  // elements between rows; plane stride = pitch * ny
   double alpha, beta;
+  FxCoef fx;      // of FP64 grids
   int *status;    // device error word (AC_ERR_TIMEOUT on an expired wait)
 };
 

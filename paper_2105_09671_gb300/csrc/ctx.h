@@ -14,7 +14,7 @@ struct ac_ctx {
   void *phi = nullptr, *ws = nullptr;
   cudaStream_t stream = nullptr;
   int device = 0, num_sms = 1;
-  ac::GridParams gp;
+  ac::GridParams gp{};
   int *d_status = nullptr;
   double *d_partials = nullptr, *d_out = nullptr, *h_out = nullptr;
   int variant = AC_VARIANT_AUTO, k = 0;  // user request

@@ -27,6 +27,8 @@
 // same bits.
 #pragma once
 
+#include <cmath>
+
 #include "common.cuh"
 
 namespace ac {
@@ -34,7 +36,7 @@ namespace ac {
 struct Fx {  // x = hi 2^32 + lo with lo signed
   int hi, lo;
 };
-__device__ __forceinline__ Fx fx_split(int64_t x) {
+__host__ __device__ __forceinline__ Fx fx_split(int64_t x) {
   Fx r;
   r.lo = (int)(uint32_t)x;
   r.hi = (int)(x >> 32) + (int)((uint32_t)x >> 31);
@@ -104,28 +106,36 @@ __device__ __forceinline__ FxV fx_shfl(const FxV &v) {  // of the lane D above
   return r;
 }
 
-// Whether alpha 2^63 and beta 2^65 fit (not for alpha near 1 or beta at the 2D
-// stability limit, where every cell takes the FP64 operations).
-__host__ __device__ constexpr bool fx_coefficients(double alpha, double beta) {
-  return alpha < 0.99 && beta < 0.2499;
+// The fixed-point coefficients of a grid (formed on the host: the conversions
+// take longer than an update).
+inline FxCoef fx_coef(double alpha, double beta) {
+  FxCoef c{};
+  if (!(alpha < 0.99 && beta < 0.2499)) return c;
+  const Fx a = fx_split((int64_t)std::llrint(alpha * 0x1p63)), b = fx_split((int64_t)std::llrint(beta * 0x1p65));
+  c.ah = a.hi;
+  c.al = a.lo;
+  c.bh = b.hi;
+  c.bl = b.lo;
+  c.on = 1;
+  return c;
 }
 
-// Coefficients of the update for one grid; FP64: also in fixed point.
+// Coefficients of the update for one grid, from its GridParams or BInst; FP64:
+// also in fixed point.
 template <typename C>
 struct Coef {
   C alpha, beta;
-  __device__ __forceinline__ Coef(double a, double b) : alpha((C)a), beta((C)b) {}
+  template <typename P>
+  __device__ __forceinline__ explicit Coef(const P &g) : alpha((C)g.alpha), beta((C)g.beta) {}
 };
 template <>
 struct Coef<double> {
   double alpha, beta;
   Fx A, B;
-  bool fx;
-  __device__ __forceinline__ Coef(double a, double b) : alpha(a), beta(b) {
-    fx = fx_coefficients(a, b);
-    A = fx_split(__double2ll_rn((fx ? a : 0.0) * 0x1p63));
-    B = fx_split(__double2ll_rn((fx ? b : 0.0) * 0x1p65));
-  }
+  int on;
+  template <typename P>
+  __device__ __forceinline__ explicit Coef(const P &g)
+      : alpha(g.alpha), beta(g.beta), A{g.fx.ah, g.fx.al}, B{g.fx.bh, g.fx.bl}, on(g.fx.on) {}
 };
 
 // The updated cell from p, the sum of its neighbours' fx_align and the
@@ -151,43 +161,84 @@ __device__ __forceinline__ bool fx_update(const FxV &p, int64_t nsum, int e, con
   return (big & ~(2u * kKeep - 1u)) != 0 && p.e > 0 && fx_in_range(e);
 }
 
-// The FP64 step of one cell from its neighbours, whose sum in FP64 is nsum.
-// (Calls, not inlined: the streaming kernels would hold a copy per level.)
-__device__ __noinline__ inline double fx_cell2(double p, double w, double e, double s, double n, double nsum,
-                                               const Coef<double> &c) {
-  if (c.fx) {
-    const FxV x = fx_in(p), xw = fx_in(w), xe = fx_in(e), xs = fx_in(s), xn = fx_in(n);
-    const int m = max(max(max(x.e, xw.e), max(xe.e, xs.e)), xn.e);
+// One explicit Euler step of a cell (see ac_update) from its neighbours w, e, s,
+// n [, b, f].
+template <int NDIM>
+__device__ __forceinline__ double fx_cell(double p, const double (&v)[2 * NDIM], const Coef<double> &c) {
+  if (c.on) {
+    const FxV x = fx_in(p);
+    FxV f[2 * NDIM];
+    int m = x.e;
+#pragma unroll
+    for (int d = 0; d < 2 * NDIM; ++d) {
+      f[d] = fx_in(v[d]);
+      m = max(m, f[d].e);
+    }
+    int64_t ns = 0;
+#pragma unroll
+    for (int d = 0; d < 2 * NDIM; ++d) ns += fx_align(f[d], m);
     double out;
-    if (fx_update<2>(x, (fx_align(xw, m) + fx_align(xe, m)) + (fx_align(xs, m) + fx_align(xn, m)), m, c, &out)) return out;
+    if (fx_update<NDIM>(x, ns, m, c, &out)) return out;
   }
-  return ac_update<double>(p, nsum, -4.0, c.alpha, c.beta);
-}
-__device__ __noinline__ inline double fx_cell3(double p, double w, double e, double s, double n, double b,
-                                               double f, double nsum, const Coef<double> &c) {
-  if (c.fx) {
-    const FxV x = fx_in(p), xw = fx_in(w), xe = fx_in(e), xs = fx_in(s), xn = fx_in(n), xb = fx_in(b),
-              xf = fx_in(f);
-    const int m = max(max(max(x.e, xw.e), max(xe.e, xs.e)), max(xn.e, max(xb.e, xf.e)));
-    double out;
-    if (fx_update<3>(x, ((fx_align(xw, m) + fx_align(xe, m)) + (fx_align(xs, m) + fx_align(xn, m))) +
-                             (fx_align(xb, m) + fx_align(xf, m)), m, c, &out)) return out;
-  }
-  return ac_update<double>(p, nsum, -6.0, c.alpha, c.beta);
+  double nsum = (v[0] + v[1]) + (v[2] + v[3]);
+  if constexpr (NDIM == 3) nsum = nsum + (v[4] + v[5]);
+  return ac_update<double>(p, nsum, -2.0 * NDIM, c.alpha, c.beta);
 }
 
-// One explicit Euler step of a cell from its neighbours (see ac_update).
-template <typename C>
-__device__ __forceinline__ C cell_update2(C p, C w, C e, C s, C n, const Coef<C> &c) {
-  const C nsum = (w + e) + (s + n);
-  if constexpr (sizeof(C) == 8) return fx_cell2(p, w, e, s, n, nsum, c);
-  else return ac_update<C>(p, nsum, C(-4), c.alpha, c.beta);
+// The same of a lane's E adjacent cells: row[0] and row[E + 1] are the cells
+// beside them, y[d] the other neighbours s, n [, b, f].  Only cells x0 + e in
+// [0, nx) are read by anyone: the zeros that lie outside the grid don't send the
+// warp through the FP64 operations.
+template <int NDIM, int E>
+struct FxCells {
+  double row[E + 2], y[2 * NDIM - 2][E];
+};
+template <int E>
+struct FxResult {
+  double v[E];
+};
+template <int NDIM, int E>
+__device__ __forceinline__ FxResult<E> fx_cells(const FxCells<NDIM, E> &in, const Coef<double> &c, int x0, int nx) {
+  FxResult<E> out;
+  bool ok[E], all = false;
+  if (c.on) {
+    all = true;
+    FxV x[E + 2];
+#pragma unroll
+    for (int e = 0; e < E + 2; ++e) x[e] = fx_in(in.row[e]);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      FxV f[2 * NDIM - 2];
+      int m = max(max(x[e].e, x[e + 1].e), x[e + 2].e);
+#pragma unroll
+      for (int d = 0; d < 2 * NDIM - 2; ++d) {
+        f[d] = fx_in(in.y[d][e]);
+        m = max(m, f[d].e);
+      }
+      int64_t ns = fx_align(x[e], m) + fx_align(x[e + 2], m);
+#pragma unroll
+      for (int d = 0; d < 2 * NDIM - 2; ++d) ns += fx_align(f[d], m);
+      ok[e] = fx_update<NDIM>(x[e + 1], ns, m, c, &out.v[e]);
+      all = all && ok[e];
+    }
+  }
+  if (!all) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      if ((c.on && ok[e]) || (unsigned)(x0 + e) >= (unsigned)nx) continue;
+      double nsum = (in.row[e] + in.row[e + 2]) + (in.y[0][e] + in.y[1][e]);
+      if constexpr (NDIM == 3) nsum = nsum + (in.y[2][e] + in.y[3][e]);
+      out.v[e] = ac_update<double>(in.row[e + 1], nsum, -2.0 * NDIM, c.alpha, c.beta);
+    }
+  }
+  return out;
 }
-template <typename C>
-__device__ __forceinline__ C cell_update3(C p, C w, C e, C s, C n, C b, C f, const Coef<C> &c) {
-  const C nsum = ((w + e) + (s + n)) + (b + f);
-  if constexpr (sizeof(C) == 8) return fx_cell3(p, w, e, s, n, b, f, nsum, c);
-  else return ac_update<C>(p, nsum, C(-6), c.alpha, c.beta);
+
+// As a call: the 2D streaming kernels would hold a copy per level and unrolled
+// row, and run out of instruction cache.
+template <int NDIM, int E>
+__device__ __noinline__ FxResult<E> fx_cells_call(FxCells<NDIM, E> in, Coef<double> c, int x0, int nx) {
+  return fx_cells<NDIM, E>(in, c, x0, nx);
 }
 
 }  // namespace ac

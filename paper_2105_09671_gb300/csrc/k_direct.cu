@@ -22,7 +22,9 @@ __device__ __forceinline__ void step2d_cell(const T *__restrict__ src, T *__rest
   C p = to_c(row[i]);
   C w = to_c(row[im]), e = to_c(row[ip]);
   C s = to_c(src[jm * g.pitch + i]), n = to_c(src[jp * g.pitch + i]);
-  dst[j * g.pitch + i] = from_c<T>(cell_update2<C>(p, w, e, s, n, Coef<C>(g.alpha, g.beta)));
+  const Coef<C> c(g);
+  if constexpr (sizeof(T) == 8) dst[j * g.pitch + i] = fx_cell<2>(p, {w, e, s, n}, c);
+  else dst[j * g.pitch + i] = from_c<T>(ac_update<C>(p, (w + e) + (s + n), C(-4), c.alpha, c.beta));
 }
 
 template <typename T>
@@ -38,7 +40,10 @@ __device__ __forceinline__ void step3d_cell(const T *__restrict__ src, T *__rest
   C w = to_c(row[im]), e = to_c(row[ip]);
   C s = to_c(src[k * plane + jm * g.pitch + i]), n = to_c(src[k * plane + jp * g.pitch + i]);
   C b = to_c(src[km * plane + j * g.pitch + i]), f = to_c(src[kp * plane + j * g.pitch + i]);
-  dst[k * plane + j * g.pitch + i] = from_c<T>(cell_update3<C>(p, w, e, s, n, b, f, Coef<C>(g.alpha, g.beta)));
+  const Coef<C> c(g);
+  if constexpr (sizeof(T) == 8) dst[k * plane + j * g.pitch + i] = fx_cell<3>(p, {w, e, s, n, b, f}, c);
+  else dst[k * plane + j * g.pitch + i] =
+      from_c<T>(ac_update<C>(p, ((w + e) + (s + n)) + (b + f), C(-6), c.alpha, c.beta));
 }
 
 // one thread per x; y and z as for_cell_yz (see cell_grid)
@@ -112,7 +117,7 @@ __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__re
   int xi[kFx2E];
 #pragma unroll
   for (int e = 0; e < kFx2E; ++e) xi[e] = reflect(xl + e, nx);
-  const Coef<double> coef(g.alpha, g.beta);
+  const Coef<double> coef(g);
   double v[kFx2E];
   FxV below[kFx2E], x[kFx2E];  // the row below, the row
   fx_load<kFx2E>(src + (int64_t)reflect(ya - 1, ny) * g.pitch, xl, xi, inside, v);
@@ -183,7 +188,7 @@ __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restr
   int64_t ro[R + 2];
 #pragma unroll
   for (int r = 0; r < R + 2; ++r) ro[r] = (int64_t)reflect(y0 - 1 + r, ny) * g.pitch;
-  const Coef<double> coef(g.alpha, g.beta);
+  const Coef<double> coef(g);
   FxV below[R][E], x[R + 2][E];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -398,7 +403,7 @@ cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *
     case AC_F64:
       // below that many cells a march's few warps wait for one row after
       // another: one thread a cell (64^2 1.9 us a step against 3.5)
-      if (fx_coefficients(g.alpha, g.beta) && g.nx * g.ny * g.nz >= kFxMarchCells)
+      if (g.fx.on && g.nx * g.ny * g.nz >= kFxMarchCells)
         return direct_fx(ndim, g, (const double *)src, (double *)dst, s);
       return direct_t<double>(ndim, g, src, dst, s);
     case AC_F32: return direct_t<float>(ndim, g, src, dst, s);

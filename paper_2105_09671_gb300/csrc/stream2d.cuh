@@ -168,21 +168,46 @@ __device__ __forceinline__ bool s2_item(T *ring_smem, uint64_t *bars, uint32_t &
       const C left = __shfl_up_sync(0xffffffffu, mid[E - 1], 1);
       const C right = __shfl_down_sync(0xffffffffu, mid[0], 1);
       C out[E];
+      if constexpr (sizeof(T) == 8) {
+        if (R < lo0) continue;  // before the first row
+        // beside a face the row continues with the face cell (what lies there
+        // is outside the grid)
+        FxCells<2, E> in;
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const C p = mid[e];
-        C w = (e == 0) ? left : mid[e - 1];
-        C ea = (e == E - 1) ? right : mid[e + 1];
-        if constexpr (FASTX) {
-          if (e % V == 0) w = lfix[e / V] ? p : w;
-          if (e % V == V - 1) ea = rfix[e / V] ? p : ea;
-        } else {
-          if (edge) {
-            if (e == eL) w = p;
-            if (e == eR) ea = p;
+        for (int e = 0; e < E; ++e) {
+          in.row[e + 1] = mid[e];
+          in.y[0][e] = ring[l][SA][e];
+          in.y[1][e] = ring[l][SN][e];
+        }
+        in.row[0] = left;
+        in.row[E + 1] = right;
+        if (edge) {
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            if (e == eL) in.row[e] = mid[e];
+            if (e == eR) in.row[e + 2] = mid[e];
           }
         }
-        out[e] = cell_update2<C>(p, w, ea, ring[l][SA][e], ring[l][SN][e], coef);
+        const FxResult<E> r = fx_cells_call<2, E>(in, coef, xl, nx);
+#pragma unroll
+        for (int e = 0; e < E; ++e) out[e] = r.v[e];
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const C p = mid[e];
+          C w = (e == 0) ? left : mid[e - 1];
+          C ea = (e == E - 1) ? right : mid[e + 1];
+          if constexpr (FASTX) {
+            if (e % V == 0) w = lfix[e / V] ? p : w;
+            if (e % V == V - 1) ea = rfix[e / V] ? p : ea;
+          } else {
+            if (edge) {
+              if (e == eL) w = p;
+              if (e == eR) ea = p;
+            }
+          }
+          out[e] = ac_update<C>(p, (w + ea) + (ring[l][SA][e] + ring[l][SN][e]), C(-4), coef.alpha, coef.beta);
+        }
       }
       if (l + 1 < K) {
 #pragma unroll
@@ -289,7 +314,7 @@ __global__ void __launch_bounds__(kS2Warps * 32, 1)
   }
   __syncwarp();
   uint32_t u = 0;
-  s2_item<T, K, FASTX, VPL_>(ring.smem, ring.bars, u, &src_map, dst, it, Coef<C>(g.alpha, g.beta),
+  s2_item<T, K, FASTX, VPL_>(ring.smem, ring.bars, u, &src_map, dst, it, Coef<C>(g),
                              g.status);
 }
 

@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(S3Geom<T, K, TILE>::NT, S3Geom<T, K, TILE>::MI
   const int r0 = R * qg;
   const int nx = (int)g.nx, ny = (int)g.ny, nz = (int)g.nz;
   const int64_t plane_stride = g.pitch * g.ny;
-  const Coef<C> coef(g.alpha, g.beta);
+  const Coef<C> coef(g);
   const bool esm = lsm || rsm;
 
   // Level l keeps its last three planes in a ring of register slots: at
@@ -434,24 +434,54 @@ __global__ void __launch_bounds__(S3Geom<T, K, TILE>::NT, S3Geom<T, K, TILE>::MI
             er = rfix ? mid[V - 1] : er;
           }
           C out[V];
+          if constexpr (sizeof(T) == 8) {
+            if (Z < lo0) continue;  // before the first plane
+            FxCells<3, V> in;
 #pragma unroll
-          for (int e = 0; e < V; ++e) {
-            const C p = mid[e];
-            C w = (e == 0) ? wl : mid[e - 1];
-            C ea = (e == V - 1) ? er : mid[e + 1];
+            for (int e = 0; e < V; ++e) {
+              const C p = mid[e];
+              in.row[e + 1] = p;
+              in.y[0][e] = BND && sself ? p : sp[e];
+              in.y[1][e] = BND && nself ? p : np[e];
+              in.y[2][e] = ring[l][SA][i][e];
+              in.y[3][e] = ring[l][SN][i][e];
+            }
+            in.row[0] = wl;
+            in.row[V + 1] = er;
             if constexpr (!FASTX) {
-              if (xedge) {
-                const int gx = gx0 + e;
-                if (gx == 0) w = p;
-                if (gx == nx - 1) ea = p;
+              if (xedge) {  // the row continues with the face cell
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                  if (gx0 + e == 0) in.row[e] = mid[e];
+                  if (gx0 + e == nx - 1) in.row[e + 2] = mid[e];
+                }
               }
             }
-            C sv = sp[e], nv = np[e];
-            if constexpr (BND) {
-              sv = sself ? p : sv;
-              nv = nself ? p : nv;
+            const int y = by + r0 + i;
+            const FxResult<V> r = fx_cells<3, V>(in, coef, gx0, (unsigned)y < (unsigned)ny ? nx : 0);
+#pragma unroll
+            for (int e = 0; e < V; ++e) out[e] = r.v[e];
+          } else {
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+              const C p = mid[e];
+              C w = (e == 0) ? wl : mid[e - 1];
+              C ea = (e == V - 1) ? er : mid[e + 1];
+              if constexpr (!FASTX) {
+                if (xedge) {
+                  const int gx = gx0 + e;
+                  if (gx == 0) w = p;
+                  if (gx == nx - 1) ea = p;
+                }
+              }
+              C sv = sp[e], nv = np[e];
+              if constexpr (BND) {
+                sv = sself ? p : sv;
+                nv = nself ? p : nv;
+              }
+              const C nsum = ((w + ea) + (sv + nv)) + (ring[l][SA][i][e] + ring[l][SN][i][e]);
+              out[e] = ac_update<C>(p, nsum, C(-6), coef.alpha, coef.beta);
             }
-            out[e] = cell_update3<C>(p, w, ea, sv, nv, ring[l][SA][i][e], ring[l][SN][i][e], coef);
           }
           if (l + 1 < K) {
 #pragma unroll
