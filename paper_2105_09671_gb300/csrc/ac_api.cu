@@ -472,7 +472,7 @@ static int issue_steps(ac_ctx *c, int64_t n, int variant, int k, int tile) {
     void *dst = src_is_phi ? c->ws : c->phi;
     cudaError_t e;
     if (variant == AC_VARIANT_DIRECT) {
-      e = launch_direct(c->d.ndim, c->d.dtype, c->gp, src, dst, c->stream);
+      e = launch_direct(c->d.ndim, c->d.dtype, c->gp, src, dst, c->num_sms, c->stream);
     } else if (vec3d && dep == 1) {
       e = launch_step3d_vec(c->gp, src, dst, c->stream);
     } else {

@@ -28,17 +28,24 @@ constexpr B2Variant kB2[] = {
     {4, 7, 64, 1.49, 1.81, 0.131, 0.0363},
     {4, 8, 112, 1.13, 2.15, 0.005, 0.0404},
     {4, 9, 64, 2.18, 1.41, 0.207, 0.0476},  // FP16 storage
-    // FP64 (block2d_fx.cuh): two rows a lane for the smallest grids (200^2 1.29
-    // us a step against 1.49 with four), four from 512^2 on (3.18 against 3.69)
-    {1, 2, 32, 0.84, 2.06, 0.0, 0.0514},
-    {1, 4, 56, 2.20, 1.16, 0.432, 0.0973},
+    // FP64 (block2d_fx.cuh), fitted to 64^2 .. 1024^2: two rows a lane for the
+    // smallest grids (200^2 1.61 us a step against 1.79 with four), four from 512^2
+    // on (700^2 4.89 against 5.44)
+    {1, 2, 40, 2.67, 0.0, 0.036, 0.0627},
+    {1, 4, 64, 2.84, 0.0, 1.16, 0.120},
 };
 constexpr int kB2Count = sizeof(kB2) / sizeof(kB2[0]);
 
-// A step of the marching FP64 kernel (k_direct.cu) on GB300: 11.1, 13.4, 27.6
-// and 94.2 us at 1024^2, 1280^2, 2048^2 and 4096^2, where tiles take 9.7 and
-// 13.8 us at the first two.
-double march_cost(int64_t nx, int64_t ny) { return 5.0 + 5.45e-6 * (double)nx * (double)ny; }
+// A step of the FP64 kernels that take one step a launch (k_direct.cu) on
+// GB300: 1.5, 1.8, 2.8, 3.6, 5.6, 10.0 and 13.7 us at 64^2, 256^2, 400^2, 512^2,
+// 700^2, 1024^2 and 1280^2, where the best tiles take 1.1, 1.7, 2.6, 3.5, 4.9, 9.9
+// and 14.3.  The fit of the tiles is up to a third short where they fill the
+// SMs' last round exactly (400^2), so a tenth is asked of them: the choice is then
+// within 15 % of the best at 64^2 .. 1024^2.
+double single_cost(int64_t nx, int64_t ny) {
+  const double cells = (double)nx * (double)ny;
+  return (cells < (double)kFxMarch2Cells ? 1.3 + 8.9e-6 * cells : 5.0 + 5.5e-6 * cells) / 1.1;
+}
 
 bool offered(const B2Variant &b, int dtype) {
   return dtype == AC_F64 ? b.E == 1 : b.E == 4 && (b.R != 9 || dtype == AC_F16S);
@@ -108,7 +115,7 @@ cudaError_t launch_fx_t(const GridParams &g, const void *src, void *dst, int war
 bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, int num_sms, Block2DPlan *out) {
   if (passes < 1) return false;
   // FP64: against one step a launch
-  double best = dtype == AC_F64 ? (double)passes * march_cost(nx, ny) : 1e300;
+  double best = dtype == AC_F64 ? (double)passes * single_cost(nx, ny) : 1e300;
   bool found = false;
   for (int v = 0; v < kB2Count; ++v) {
     if (!offered(kB2[v], dtype)) continue;

@@ -7,6 +7,8 @@
 // Larger FP64 grids march: a value is taken apart for the integer form of the
 // update (fixed64.cuh) once per lane and shared by warp shuffles (x) and
 // registers (y, z) while a warp walks a chunk of rows or planes.
+#include <algorithm>
+
 #include "fixed64.cuh"
 #include "kernels.h"
 
@@ -51,6 +53,8 @@ template <typename T, bool TALL>
 __global__ void __launch_bounds__(256) step2d_direct(const T *__restrict__ src,
                                                      T *__restrict__ dst, GridParams g) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();  // (see direct_t)
+  pdl_launch_dependents();
   if (i >= g.nx) return;
   for_cell_yz<TALL>(g, [&](int64_t j, int64_t) { step2d_cell(src, dst, g, i, j); });
 }
@@ -59,12 +63,18 @@ template <typename T, bool TALL>
 __global__ void __launch_bounds__(256) step3d_direct(const T *__restrict__ src,
                                                      T *__restrict__ dst, GridParams g) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();  // (see direct_t)
+  pdl_launch_dependents();
   if (i >= g.nx) return;
   for_cell_yz<TALL>(g, [&](int64_t j, int64_t k) { step3d_cell(src, dst, g, i, j, k); });
 }
 
 // -------------------------------------------------- FP64, integer form --
-constexpr int64_t kFxMarchCells = 512 * 512;
+// Grids that march.  Below, a march's few warps wait for one row (plane) after
+// another: one thread a cell takes 3.8 us a step against 4.9 at 512^2, 4.5
+// against 7.9 at 64^3 and 9.5 against 10.3 at 80^3; 10.5 against 10.3 at 1024^2,
+// 16.2 against 15.1 at 100^3 (128^3, whose rows fill its blocks: 25.8 against 29.4).
+constexpr int64_t kFxMarch3Cells = 700000;
 constexpr int kFxWarps = 4;                      // per CTA, independent of one another
 constexpr int kFx2E = 4, kFx2W = 32 * kFx2E;      // 2D: cells a lane, columns a warp
 constexpr int kFx3E = 2, kFx3W = 32 * kFx3E;      // 3D
@@ -268,16 +278,16 @@ struct FxMarch {
   double one, add, full, pro;
 };
 constexpr FxMarch kFxMarch2 = {6, 0.443, 0.314, 2.10, 0.91}, kFxMarch3 = {4, 0.705, 0.371, 2.07, 0.71};
-constexpr int kFxSms = 152;
 
-static int64_t fx_chunk(const FxMarch &m, int64_t columns, int64_t len) {
-  const int64_t q0 = (columns + kFxSms * kFxWarps - 1) / (kFxSms * kFxWarps);
+static int64_t fx_chunk(const FxMarch &m, int64_t columns, int64_t len, int num_sms) {
+  const int64_t round = (int64_t)std::max(1, num_sms) * kFxWarps;  // warps of one CTA an SM
+  const int64_t q0 = (columns + round - 1) / round;
   double best[2] = {1e300, 1e300};  // one round; several
   int64_t best_chunk[2] = {len, len};
   for (int64_t qt = q0; qt < q0 + 24; ++qt) {
-    const int64_t chunk = (len + qt * kFxSms * kFxWarps / columns - 1) / (qt * kFxSms * kFxWarps / columns);
+    const int64_t chunk = (len + qt * round / columns - 1) / (qt * round / columns);
     const int64_t warps = columns * ((len + chunk - 1) / chunk);
-    const int64_t q = (warps + kFxSms * kFxWarps - 1) / (kFxSms * kFxWarps);
+    const int64_t q = (warps + round - 1) / round;
     const int64_t rounds = q / m.occ, rest = q % m.occ;
     const double row = q <= m.occ ? m.one + m.add * (double)q
                                   : m.full * (double)rounds + (rest ? m.one + m.add * (double)rest : 0.0);
@@ -289,12 +299,13 @@ static int64_t fx_chunk(const FxMarch &m, int64_t columns, int64_t len) {
   return best_chunk[best[1] < 0.97 * best[0]];  // the fit's own error
 }
 
-static cudaError_t direct_fx(int ndim, const GridParams &g, const double *src, double *dst, cudaStream_t s) {
+static cudaError_t direct_fx(int ndim, const GridParams &g, const double *src, double *dst, int num_sms,
+                             cudaStream_t s) {
   const int w = ndim == 2 ? kFx2W : kFx3W;
   const int64_t strips = (g.nx + w - 2 * kFxHalo - 1) / (w - 2 * kFxHalo);
   const int64_t bands = ndim == 2 ? 1 : (g.ny + kFx3R - 1) / kFx3R;
   const int64_t len = ndim == 2 ? g.ny : g.nz;
-  const int64_t chunk = fx_chunk(ndim == 2 ? kFxMarch2 : kFxMarch3, strips * bands, len);
+  const int64_t chunk = fx_chunk(ndim == 2 ? kFxMarch2 : kFxMarch3, strips * bands, len, num_sms);
   const int64_t warps = strips * bands * ((len + chunk - 1) / chunk);
   const unsigned blocks = (unsigned)((warps + kFxWarps - 1) / kFxWarps);
   if (ndim == 2) step2d_fx<<<blocks, kFxWarps * 32, 0, s>>>(src, dst, g, (int)strips, (int)chunk);
@@ -382,32 +393,38 @@ cudaError_t launch_step3d_vec(const GridParams &g, const void *src, void *dst, c
   }
 }
 
+// FP64 grids of at most two blocks an SM are launched to overlap the previous
+// launch's tail (programmatic stream serialization): 16^3 1.78 -> 1.56 us a step,
+// 32^3 1.92 -> 1.76, 256^2 1.98 -> 1.85.  With more blocks the next launch's take the SMs of this one's
+// (48^3 3.15 -> 3.42).
 template <typename T>
-static cudaError_t direct_t(int ndim, const GridParams &g, const void *src, void *dst,
+static cudaError_t direct_t(int ndim, const GridParams &g, const void *src, void *dst, int num_sms,
                             cudaStream_t s) {
-  const dim3 block(kCellBlockX, kCellBlockY), grid = cell_grid(g);
   const bool tall = cell_grid_tall(g);
-  if (ndim == 2) {
-    if (tall) step2d_direct<T, true><<<grid, block, 0, s>>>((const T *)src, (T *)dst, g);
-    else step2d_direct<T, false><<<grid, block, 0, s>>>((const T *)src, (T *)dst, g);
-  } else {
-    if (tall) step3d_direct<T, true><<<grid, block, 0, s>>>((const T *)src, (T *)dst, g);
-    else step3d_direct<T, false><<<grid, block, 0, s>>>((const T *)src, (T *)dst, g);
-  }
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = cell_grid(g);
+  cfg.blockDim = dim3(kCellBlockX, kCellBlockY);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = sizeof(T) == 8 && (int64_t)cfg.gridDim.x * cfg.gridDim.y * cfg.gridDim.z <= 2 * num_sms ? 1 : 0;
+  void (*k)(const T *, T *, GridParams);
+  if (ndim == 2) k = tall ? step2d_direct<T, true> : step2d_direct<T, false>;
+  else k = tall ? step3d_direct<T, true> : step3d_direct<T, false>;
+  return cudaLaunchKernelEx(&cfg, k, (const T *)src, (T *)dst, g);
 }
 
-cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *src, void *dst,
+cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *src, void *dst, int num_sms,
                           cudaStream_t s) {
   switch (dtype) {
     case AC_F64:
-      // below that many cells a march's few warps wait for one row after
-      // another: one thread a cell (64^2 1.9 us a step against 3.5)
-      if (g.fx.on && g.nx * g.ny * g.nz >= kFxMarchCells)
-        return direct_fx(ndim, g, (const double *)src, (double *)dst, s);
-      return direct_t<double>(ndim, g, src, dst, s);
-    case AC_F32: return direct_t<float>(ndim, g, src, dst, s);
-    case AC_F16S: return direct_t<__half>(ndim, g, src, dst, s);
+      if (g.fx.on && g.nx * g.ny * g.nz >= (ndim == 2 ? kFxMarch2Cells : kFxMarch3Cells))
+        return direct_fx(ndim, g, (const double *)src, (double *)dst, num_sms, s);
+      return direct_t<double>(ndim, g, src, dst, num_sms, s);
+    case AC_F32: return direct_t<float>(ndim, g, src, dst, num_sms, s);
+    case AC_F16S: return direct_t<__half>(ndim, g, src, dst, num_sms, s);
   }
   return cudaErrorInvalidValue;
 }

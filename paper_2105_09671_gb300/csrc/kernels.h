@@ -58,7 +58,8 @@ inline dim3 cell_grid(const GridParams &g) {
               (unsigned)std::min<int64_t>(g.nz, 65535));
 }
 
-cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *src, void *dst,
+constexpr int64_t kFxMarch2Cells = 1000000;  // 2D FP64 grids that march (see k_direct.cu)
+cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *src, void *dst, int num_sms,
                           cudaStream_t s);
 // One step of a small 3D FP32 grid (see k_direct.cu).
 bool step3d_vec_serves(int dtype, const GridParams &g);

@@ -190,7 +190,7 @@ def test_cells_of_every_size_are_no_less_exact_than_fp64_operations(shape, kind)
             assert mine <= base, f"2^-{2 * b}: {np.sqrt(mine / n):.3e} against {np.sqrt(base / n):.3e} ({n} cells)"
 
 
-@pytest.mark.parametrize("shape", [(24, 40), (130, 249), (515, 517), (5, 6, 40), (65, 64, 66)])
+@pytest.mark.parametrize("shape", [(24, 40), (130, 249), (515, 517), (1003, 1001), (5, 6, 40), (65, 64, 66), (99, 101, 103)])
 @pytest.mark.parametrize("kind", [0, 1, "rough", "large"])
 def test_negated_fields_step_to_the_negated_result(shape, kind):
     h = 1.0 / 64
