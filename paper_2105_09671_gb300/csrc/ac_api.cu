@@ -408,7 +408,7 @@ bool ac_plan_depths(int64_t n, int k, std::vector<int> &depths) {
 static bool takes_stand_in(const ac_ctx *c, int variant, int k, int tile) {
   if (c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO) return false;
   if (c->d.ndim == 3 && !step3d_vec_serves(c->d.dtype, c->gp)) return false;
-  if (c->d.dtype == AC_F64 && !c->gp.fx.on) return false;
+  if (c->d.dtype == AC_F64 && !c->gp.fx.limit) return false;
   int dv, dk;
   default_schedule(c, &dv, &dk);
   return variant == dv && k == dk && tile == default_tile(c, dk);

@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(kB2FxMaxWarps * 32)
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     v[r] = src[(int64_t)reflect(yr + r, ny) * g.pitch + xi];
-    f[r] = fx_in(v[r]);
+    f[r] = fx_in(v[r], coef.limit);
   }
   for (int s = 0; s < k; ++s) {
     const int first = (s & 1) * 2 * nw * 32 + lane, last = first + nw * 32;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kB2FxMaxWarps * 32)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       v[r] = nv[r];
-      f[r] = fx_in(nv[r]);
+      f[r] = fx_in(nv[r], coef.limit);
     }
   }
   pdl_launch_dependents();

@@ -126,11 +126,14 @@ __device__ __forceinline__ C ac_update(C p, C nsum, C minus_2d, C alpha, C beta)
 }
 
 // ----------------------------------------------------------- parameters ---
-// alpha 2^63 and beta 2^65 as hi 2^32 + lo, lo signed (fixed64.cuh); on is 0
-// where they don't fit (alpha near 1, beta at the 2D stability limit), which
-// leaves every cell to the FP64 operations.
+// alpha 2^63 and beta 2^65 as hi 2^32 + lo, lo signed, and the values that the
+// integer form takes (fixed64.cuh): those whose top word without the sign, times
+// two, is below limit.  0 where the coefficients don't fit (alpha near 1, beta at
+// the 2D stability limit), which leaves every cell to the FP64 operations.  keep:
+// the size of the high half from which a result is taken.
 struct FxCoef {
-  int ah, al, bh, bl, on;
+  int ah, al, bh, bl;
+  uint32_t limit, keep;
 };
 
 struct GridParams {

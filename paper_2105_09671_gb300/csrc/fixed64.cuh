@@ -14,17 +14,20 @@
 // operations (fused as in ac_update) beat where a cell much smaller than its
 // neighbours stays so because theirs cancel: at a zero crossing their sums are
 // exact.  There the cell takes them: when the result and its Laplacian part
-// both are below 2^-5 2^E.  Otherwise the rms error, by the size of the result
-// against the stencil (down to 2^-10) and for rough, smooth and planar
-// stencils, is 0.03 to 0.98 of the FP64 operations', its largest value at most
-// 0.95 of theirs (128-bit arithmetic, amplitudes 1e-6 .. 1.7, alpha 0.0004 ..
-// 0.6, 2D and 3D).  +-1 and 0 stay exact fixed points, and mirrored or negated
-// fields give the mirrored or negated result bit for bit.
+// both are below 2^-5 2^E (alpha = 0: 2^-4).  Otherwise the rms error, by the size
+// of the result against the stencil (down to 2^-10) and for rough, smooth and
+// planar stencils, is 0.03 to 0.98 of the FP64 operations', its largest value at
+// most 0.98 of theirs (128-bit arithmetic, amplitudes 1e-6 .. 1.7, alpha 0 and
+// 1e-9 .. 0.6, 2D and 3D).  +-1 and 0 stay exact fixed points, and mirrored or
+// negated fields give the mirrored or negated result bit for bit.
 // Likewise a cell whose stencil holds a value of 1.75 or more in size (fields
-// of the scheme have |phi| <= 1), NaN or infinity, or none above 2^-959, and one
-// that is 0, takes the FP64 operations.  The form a cell takes and its result
-// depend on its stencil's values alone, so every kernel and schedule gives the
-// same bits.
+// of the scheme have |phi| <= 1; in the heat equation, alpha = 0: 2^340), NaN or
+// infinity, or none above 2^-959, and one that is 0, takes the FP64 operations.
+// (A field that is all beyond 1.75 is formed twice: 4096^2 348 us a step against
+// 253 by the FP64 operations alone.  A test that spares it the first form cost
+// every field 2.5 %.)
+// The form a cell takes and its result depend on its stencil's values alone, so
+// every kernel and schedule gives the same bits.
 #pragma once
 
 #include <cmath>
@@ -68,17 +71,17 @@ struct FxV {
 constexpr int kFxOut = 2047;
 // (Integer instructions only: the conversions from and to 64-bit integers
 // are slower than the FP64 operations they would replace.)
-__device__ __forceinline__ FxV fx_in(double v) {
+__device__ __forceinline__ FxV fx_in(double v, uint32_t limit) {
   const int hi = __double2hiint(v);
   const uint32_t twice = 2u * (uint32_t)hi;  // without the sign
   const uint64_t a = ((uint64_t)(uint32_t)((hi & 0xfffff) | 0x100000) << 32 | (uint32_t)__double2loint(v)) << 9;
   FxV r;
   r.m = (int64_t)a ^ (int64_t)(hi >> 31);
-  r.e = twice < 2u * 0x3ffc0000u ? (int)(twice >> 21) : kFxOut;
+  r.e = twice < limit ? (int)(twice >> 21) : kFxOut;
   return r;
 }
 // Whether a stencil with largest exponent e takes the integer form.
-__device__ __forceinline__ bool fx_in_range(int e) { return (unsigned)(e - 64) < 1024u - 64u; }
+__device__ __forceinline__ bool fx_in_range(int e) { return (unsigned)(e - 64) < (unsigned)(kFxOut - 64); }
 // m / 2^d, d >= 0, rounded down (the instruction clamps d).
 __device__ __forceinline__ int64_t fx_shift(int64_t m, int d) {
   int64_t r;
@@ -116,7 +119,10 @@ inline FxCoef fx_coef(double alpha, double beta) {
   c.al = a.lo;
   c.bh = b.hi;
   c.bl = b.lo;
-  c.on = 1;
+  // 2^55 units, 2^-5 2^E; twice that where the FP64 operations round once less
+  c.keep = alpha > 0.0 ? 1u << 23 : 1u << 24;
+  // 1.75: phi (1 - phi^2) stays below 4; 2^340: phi^3 stays finite
+  c.limit = 2u * (alpha > 0.0 ? 0x3ffc0000u : 1363u << 20);
   return c;
 }
 
@@ -132,10 +138,10 @@ template <>
 struct Coef<double> {
   double alpha, beta;
   Fx A, B;
-  int on;
+  uint32_t limit, keep;
   template <typename P>
   __device__ __forceinline__ explicit Coef(const P &g)
-      : alpha(g.alpha), beta(g.beta), A{g.fx.ah, g.fx.al}, B{g.fx.bh, g.fx.bl}, on(g.fx.on) {}
+      : alpha(g.alpha), beta(g.beta), A{g.fx.ah, g.fx.al}, B{g.fx.bh, g.fx.bl}, limit(g.fx.limit), keep(g.fx.keep) {}
 };
 
 // The updated cell from p, the sum of its neighbours' fx_align and the
@@ -155,23 +161,22 @@ __device__ __forceinline__ bool fx_update(const FxV &p, int64_t nsum, int e, con
   const int64_t b = fx_mulhi(fx_split(lap), c.B);     // units 2^(e - 1082)
   const int64_t r = (x << 2) + (b << 1) + fx_shift(a, e - p.e);
   *out = fx_out(r, e, neg);
-  // r or 2 b of 2^55 = 2^-5 2^E units or more (high halves of 2^23)
-  constexpr uint32_t kKeep = 1u << 23;
-  const uint32_t big = ((uint32_t)(r >> 32) + kKeep) | (2u * (uint32_t)(b >> 32) + kKeep);
-  return (big & ~(2u * kKeep - 1u)) != 0 && p.e > 0 && fx_in_range(e);
+  // r or 2 b large enough, their high halves c.keep (a power of two) or more
+  const uint32_t big = ((uint32_t)(r >> 32) + c.keep) | (2u * (uint32_t)(b >> 32) + c.keep);
+  return big >= 2u * c.keep && p.e > 0 && fx_in_range(e);
 }
 
 // One explicit Euler step of a cell (see ac_update) from its neighbours w, e, s,
 // n [, b, f].
 template <int NDIM>
 __device__ __forceinline__ double fx_cell(double p, const double (&v)[2 * NDIM], const Coef<double> &c) {
-  if (c.on) {
-    const FxV x = fx_in(p);
+  if (c.limit) {
+    const FxV x = fx_in(p, c.limit);
     FxV f[2 * NDIM];
     int m = x.e;
 #pragma unroll
     for (int d = 0; d < 2 * NDIM; ++d) {
-      f[d] = fx_in(v[d]);
+      f[d] = fx_in(v[d], c.limit);
       m = max(m, f[d].e);
     }
     int64_t ns = 0;
@@ -201,18 +206,18 @@ template <int NDIM, int E>
 __device__ __forceinline__ FxResult<E> fx_cells(const FxCells<NDIM, E> &in, const Coef<double> &c, int x0, int nx) {
   FxResult<E> out;
   bool ok[E], all = false;
-  if (c.on) {
+  if (c.limit) {
     all = true;
     FxV x[E + 2];
 #pragma unroll
-    for (int e = 0; e < E + 2; ++e) x[e] = fx_in(in.row[e]);
+    for (int e = 0; e < E + 2; ++e) x[e] = fx_in(in.row[e], c.limit);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       FxV f[2 * NDIM - 2];
       int m = max(max(x[e].e, x[e + 1].e), x[e + 2].e);
 #pragma unroll
       for (int d = 0; d < 2 * NDIM - 2; ++d) {
-        f[d] = fx_in(in.y[d][e]);
+        f[d] = fx_in(in.y[d][e], c.limit);
         m = max(m, f[d].e);
       }
       int64_t ns = fx_align(x[e], m) + fx_align(x[e + 2], m);
@@ -225,7 +230,7 @@ __device__ __forceinline__ FxResult<E> fx_cells(const FxCells<NDIM, E> &in, cons
   if (!all) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      if ((c.on && ok[e]) || (unsigned)(x0 + e) >= (unsigned)nx) continue;
+      if ((c.limit && ok[e]) || (unsigned)(x0 + e) >= (unsigned)nx) continue;
       double nsum = (in.row[e] + in.row[e + 2]) + (in.y[0][e] + in.y[1][e]);
       if constexpr (NDIM == 3) nsum = nsum + (in.y[2][e] + in.y[3][e]);
       out.v[e] = ac_update<double>(in.row[e + 1], nsum, -2.0 * NDIM, c.alpha, c.beta);

@@ -40,11 +40,11 @@ constexpr int kB2Count = sizeof(kB2) / sizeof(kB2[0]);
 // GB300: 1.5, 1.8, 2.8, 3.6, 5.6, 10.0 and 13.7 us at 64^2, 256^2, 400^2, 512^2,
 // 700^2, 1024^2 and 1280^2, where the best tiles take 1.1, 1.7, 2.6, 3.5, 4.9, 9.9
 // and 14.3.  The fit of the tiles is up to a third short where they fill the
-// SMs' last round exactly (400^2), so a tenth is asked of them: the choice is then
-// within 15 % of the best at 64^2 .. 1024^2.
+// SMs' last round exactly (400^2), and rough fields cost them more (256^2 2.7
+// against 2.2 for the heat equation from noise), so a quarter is asked of them.
 double single_cost(int64_t nx, int64_t ny) {
   const double cells = (double)nx * (double)ny;
-  return (cells < (double)kFxMarch2Cells ? 1.3 + 8.9e-6 * cells : 5.0 + 5.5e-6 * cells) / 1.1;
+  return (cells < (double)kFxMarch2Cells ? 1.3 + 8.9e-6 * cells : 5.0 + 5.5e-6 * cells) / 1.25;
 }
 
 bool offered(const B2Variant &b, int dtype) {

@@ -73,8 +73,14 @@ __global__ void __launch_bounds__(256) step3d_direct(const T *__restrict__ src,
 // Grids that march.  Below, a march's few warps wait for one row (plane) after
 // another: one thread a cell takes 3.8 us a step against 4.9 at 512^2, 4.5
 // against 7.9 at 64^3 and 9.5 against 10.3 at 80^3; 10.5 against 10.3 at 1024^2,
-// 16.2 against 15.1 at 100^3 (128^3, whose rows fill its blocks: 25.8 against 29.4).
-constexpr int64_t kFxMarch3Cells = 700000;
+// 16.2 against 15.1 at 100^3.  In 3D rows that fill its blocks move the line up
+// (128^3 25.8 against 29.4; 256^3 197 against 164).
+static bool fx_marches(int ndim, const GridParams &g) {
+  const int64_t cells = g.nx * g.ny * g.nz;
+  if (ndim == 2) return cells >= kFxMarch2Cells;
+  const int64_t full = (g.nx + kCellBlockX - 1) / kCellBlockX * kCellBlockX * g.ny * g.nz;
+  return cells >= (10 * full <= 11 * cells ? 3000000 : 700000);
+}
 constexpr int kFxWarps = 4;                      // per CTA, independent of one another
 constexpr int kFx2E = 4, kFx2W = 32 * kFx2E;      // 2D: cells a lane, columns a warp
 constexpr int kFx3E = 2, kFx3W = 32 * kFx3E;      // 3D
@@ -132,15 +138,15 @@ __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__re
   FxV below[kFx2E], x[kFx2E];  // the row below, the row
   fx_load<kFx2E>(src + (int64_t)reflect(ya - 1, ny) * g.pitch, xl, xi, inside, v);
 #pragma unroll
-  for (int e = 0; e < kFx2E; ++e) below[e] = fx_in(v[e]);
+  for (int e = 0; e < kFx2E; ++e) below[e] = fx_in(v[e], coef.limit);
   fx_load<kFx2E>(src + (int64_t)ya * g.pitch, xl, xi, inside, v);
 #pragma unroll
-  for (int e = 0; e < kFx2E; ++e) x[e] = fx_in(v[e]);
+  for (int e = 0; e < kFx2E; ++e) x[e] = fx_in(v[e], coef.limit);
   fx_load<kFx2E>(src + (int64_t)reflect(ya + 1, ny) * g.pitch, xl, xi, inside, v);
   for (int y = ya; y < ye; ++y) {
     FxV up[kFx2E];
 #pragma unroll
-    for (int e = 0; e < kFx2E; ++e) up[e] = fx_in(v[e]);
+    for (int e = 0; e < kFx2E; ++e) up[e] = fx_in(v[e], coef.limit);
     if (y + 1 < ye)  // the row after next, ahead of its use
       fx_load<kFx2E>(src + (int64_t)reflect(y + 2, ny) * g.pitch, xl, xi, inside, v);
     const FxV left = fx_shfl<-1>(x[kFx2E - 1]), right = fx_shfl<1>(x[0]);
@@ -205,14 +211,14 @@ __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restr
     double v[E];
     fx_load<E>(src + (int64_t)reflect(za - 1, nz) * plane + ro[r + 1], xl, xi, inside, v);
 #pragma unroll
-    for (int e = 0; e < E; ++e) below[r][e] = fx_in(v[e]);
+    for (int e = 0; e < E; ++e) below[r][e] = fx_in(v[e], coef.limit);
   }
 #pragma unroll
   for (int r = 0; r < R + 2; ++r) {
     double v[E];
     fx_load<E>(src + (int64_t)za * plane + ro[r], xl, xi, inside, v);
 #pragma unroll
-    for (int e = 0; e < E; ++e) x[r][e] = fx_in(v[e]);
+    for (int e = 0; e < E; ++e) x[r][e] = fx_in(v[e], coef.limit);
   }
   for (int z = za; z < ze; ++z) {
     FxV up[R + 2][E];
@@ -222,7 +228,7 @@ __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restr
       double v[E];
       fx_load<E>(zp + ro[r], xl, xi, inside, v);
 #pragma unroll
-      for (int e = 0; e < E; ++e) up[r][e] = fx_in(v[e]);
+      for (int e = 0; e < E; ++e) up[r][e] = fx_in(v[e], coef.limit);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -393,7 +399,7 @@ cudaError_t launch_step3d_vec(const GridParams &g, const void *src, void *dst, c
   }
 }
 
-// FP64 grids of at most two blocks an SM are launched to overlap the previous
+// FP64 grids (integer form) of at most two blocks an SM are launched to overlap the previous
 // launch's tail (programmatic stream serialization): 16^3 1.78 -> 1.56 us a step,
 // 32^3 1.92 -> 1.76, 256^2 1.98 -> 1.85.  With more blocks the next launch's take the SMs of this one's
 // (48^3 3.15 -> 3.42).
@@ -409,7 +415,7 @@ static cudaError_t direct_t(int ndim, const GridParams &g, const void *src, void
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = sizeof(T) == 8 && (int64_t)cfg.gridDim.x * cfg.gridDim.y * cfg.gridDim.z <= 2 * num_sms ? 1 : 0;
+  cfg.numAttrs = g.fx.limit && (int64_t)cfg.gridDim.x * cfg.gridDim.y * cfg.gridDim.z <= 2 * num_sms ? 1 : 0;
   void (*k)(const T *, T *, GridParams);
   if (ndim == 2) k = tall ? step2d_direct<T, true> : step2d_direct<T, false>;
   else k = tall ? step3d_direct<T, true> : step3d_direct<T, false>;
@@ -420,7 +426,7 @@ cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *
                           cudaStream_t s) {
   switch (dtype) {
     case AC_F64:
-      if (g.fx.on && g.nx * g.ny * g.nz >= (ndim == 2 ? kFxMarch2Cells : kFxMarch3Cells))
+      if (g.fx.limit && fx_marches(ndim, g))
         return direct_fx(ndim, g, (const double *)src, (double *)dst, num_sms, s);
       return direct_t<double>(ndim, g, src, dst, num_sms, s);
     case AC_F32: return direct_t<float>(ndim, g, src, dst, num_sms, s);

@@ -154,14 +154,16 @@ def _axis_neighbours(p):
 
 @pytest.mark.parametrize("shape", [(24, 40), (5, 6, 40)])
 @pytest.mark.parametrize("kind", [0, 1, "rough"])
-def test_cells_of_every_size_are_no_less_exact_than_fp64_operations(shape, kind):
+@pytest.mark.parametrize("heat", [False, True])
+def test_cells_of_every_size_are_no_less_exact_than_fp64_operations(shape, kind, heat):
     # against exact rationals, cells binned by their result's size relative to
     # the stencil's largest value; the baseline is ac_update with its fused
     # operations, each rounded once
     from fractions import Fraction as Q
     h = 1.0 / 64
-    eps, dt = 2.5 * h, 0.1 * h * h
+    eps, dt = np.inf if heat else 2.5 * h, 0.1 * h * h
     phi0 = 0.1 * wl.random_field(shape, seed=4) if kind == "rough" else _crossing_field(shape, kind)
+    phi0 = (300.0 if heat else 1.0) * phi0
     out = gpu_run(phi0, h, eps, dt, 1, "f64", ac.AC_VARIANT_DIRECT, 1).reshape(-1)
     alpha, beta = dt / (eps * eps), dt / (h * h)
     nb = [a.reshape(-1) for a in _axis_neighbours(phi0)]
@@ -205,6 +207,25 @@ def test_negated_fields_step_to_the_negated_result(shape, kind):
         a = gpu_run(phi0, h, eps, dt, 6, "f64", v, k) if v is not None else gpu_run(phi0, h, eps, dt, 6, "f64")
         b = gpu_run(-phi0, h, eps, dt, 6, "f64", v, k) if v is not None else gpu_run(-phi0, h, eps, dt, 6, "f64")
         assert np.array_equal(a, -b), f"{shape} {kind} schedule {v} {k}"
+
+
+@pytest.mark.parametrize("shape", [(40, 64), (300, 310), (1003, 1001), (9, 13, 61), (64, 65, 66), (99, 101, 103)])
+def test_temperatures_of_any_size_give_the_same_bits_on_every_kernel(shape):
+    # the heat equation: no bound on the field; from 2^340 = 2.2e102 on the FP64
+    # operations
+    h = 1.0 / 64
+    phi0 = wl.random_field(shape, seed=4) * np.linspace(1.0, 400.0, shape[-1])
+    spikes = phi0.copy()
+    spikes.reshape(-1)[11:14] = [1e101, 3e102, -5e102]
+    for f in (phi0, spikes):
+        outs = [gpu_run(f, h, np.inf, 0.1 * h * h, 3, "f64", *s)
+                for s in ((), (ac.AC_VARIANT_DIRECT, 1), (ac.AC_VARIANT_STREAM, 1), (ac.AC_VARIANT_STREAM, 2))]
+        assert np.isfinite(outs[0]).all()
+        for o in outs[1:]:
+            assert np.array_equal(outs[0], o)
+        if f is phi0:
+            ref = oracle.step(f, h, np.inf, 0.1 * h * h, 3)
+            assert np.max(np.abs(outs[0] - ref)) <= 1e-14 * 400
 
 
 @pytest.mark.parametrize("shape,n", [((16, 16), 2000), ((40, 64), 600), ((520, 510), 100), ((4, 6, 64), 600)])
