@@ -374,13 +374,18 @@ __global__ void __launch_bounds__(64) step3d_vec(const float *__restrict__ src, 
   }
 }
 
+// (A streaming pass over a few large planes has short chains: 700 x 700 x 2 and
+// 600 x 600 x 3 3.1 and 3.6 us a step against 3.7 and 4.4, 400 x 400 x 2 3.1 against
+// 2.1.)
 bool step3d_vec_serves(int dtype, const GridParams &g) {
-  return dtype == AC_F32 && g.nx * g.ny * g.nz <= 1500000 && g.nz <= 65535;
+  return dtype == AC_F32 && g.nx * g.ny * g.nz <= (g.nz < 6 ? 400000 : 1500000) && g.nz <= 65535;
 }
 
 cudaError_t launch_step3d_vec(const GridParams &g, const void *src, void *dst, cudaStream_t s) {
   const int nvx = (int)((g.nx + 3) / 4);
-  const int rz = g.nx * g.ny * g.nz < 64000 ? 1 : g.nx * g.ny * g.nz < 500000 ? 2 : 4;
+  // planes a thread: no more than there are
+  const int64_t cells = g.nx * g.ny * g.nz;
+  const int rz = cells < 64000 || g.nz < 2 ? 1 : cells < 500000 || g.nz < 4 ? 2 : 4;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((g.ny * nvx + 63) / 64), (unsigned)((g.nz + rz - 1) / rz));
   cfg.blockDim = dim3(64);

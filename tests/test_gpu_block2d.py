@@ -45,7 +45,8 @@ def test_default_equals_the_streaming_schedule_bitwise(shape, dtype):
         b.close()
 
 
-@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 5), (7, 1, 64), (33, 35, 31), (40, 60, 70), (81, 90, 101)])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 5), (7, 1, 64), (33, 35, 31), (40, 60, 70), (81, 90, 101),
+                                   (1, 300, 301), (3, 200, 301), (5, 280, 283), (6, 300, 301)])
 def test_small_3d_default_equals_the_streaming_schedule_bitwise(shape):
     # one step to a launch, in each of its plane counts a thread; odd step
     # counts start with a pass of two
