@@ -414,15 +414,25 @@ static bool takes_stand_in(const ac_ctx *c, int variant, int k, int tile) {
   return variant == dv && k == dk && tile == default_tile(c, dk);
 }
 
-// n steps on the register-tile kernels; *done is false if none serves the
-// grid (nothing was launched).
-static int issue_block2d(ac_ctx *c, int64_t n, int k, bool *done) {
+// n steps on the register-tile kernels; *done is false if the default schedule's
+// kernel is faster or none serves the grid (nothing was launched).
+static int issue_block2d(ac_ctx *c, int64_t n, int k, int tile, bool *done) {
+  std::vector<int> depths;
+  int64_t count[AC_MAX_K + 1] = {0};  // the default schedule's passes by depth
+  if (c->d.dtype == AC_F64) {
+    count[1] = n;
+  } else {
+    ac_plan_depths(n, k, depths);
+    for (int dep : depths) ++count[dep];
+  }
   // FP16 storage: the passes whose ends round the field; else single steps
   std::vector<int> passes;
-  if (c->d.dtype == AC_F16S) ac_plan_depths(n, k, passes);
+  if (c->d.dtype == AC_F16S) passes.swap(depths);
   const int64_t np = c->d.dtype == AC_F16S ? (int64_t)passes.size() : n;
   Block2DPlan plan;
-  *done = block2d_plan(c->d.dtype, c->d.nx, c->d.ny, np, c->d.dtype == AC_F16S ? k : 1, c->num_sms, &plan);
+  const double other = block2d_other(c->d.dtype, tile, c->d.nx, c->d.ny, count, AC_MAX_K, c->num_sms);
+  *done = block2d_plan(c->d.dtype, c->d.nx, c->d.ny, np, passes.empty() ? 1 : k,
+                       passes.empty() ? nullptr : passes.data(), other, c->num_sms, &plan);
   if (!*done) return AC_OK;
   void *src = c->phi, *dst = c->ws;
   for (int64_t i = 0; i < plan.launches; ++i) {
@@ -453,7 +463,7 @@ static int issue_steps(ac_ctx *c, int64_t n, int variant, int k, int tile) {
   const bool stand_in = takes_stand_in(c, variant, k, tile);
   if (stand_in && c->d.ndim == 2) {
     bool done = false;
-    const int rc = issue_block2d(c, n, k, &done);
+    const int rc = issue_block2d(c, n, k, tile, &done);
     if (rc || done) return rc;
   }
   const bool vec3d = stand_in && c->d.ndim == 3;

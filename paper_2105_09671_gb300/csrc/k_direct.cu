@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256) step3d_direct(const T *__restrict__ src,
 // (128^3 25.8 against 29.4; 256^3 197 against 164).
 static bool fx_marches(int ndim, const GridParams &g) {
   const int64_t cells = g.nx * g.ny * g.nz;
-  if (ndim == 2) return cells >= kFxMarch2Cells;
+  if (ndim == 2) return cells >= 1000000;
   const int64_t full = (g.nx + kCellBlockX - 1) / kCellBlockX * kCellBlockX * g.ny * g.nz;
   return cells >= (10 * full <= 11 * cells ? 3000000 : 700000);
 }

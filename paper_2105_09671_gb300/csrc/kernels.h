@@ -58,7 +58,6 @@ inline dim3 cell_grid(const GridParams &g) {
               (unsigned)std::min<int64_t>(g.nz, 65535));
 }
 
-constexpr int64_t kFxMarch2Cells = 1000000;  // 2D FP64 grids that march (see k_direct.cu)
 cudaError_t launch_direct(int ndim, int dtype, const GridParams &g, const void *src, void *dst, int num_sms,
                           cudaStream_t s);
 // One step of a small 3D FP32 grid (see k_direct.cu).
@@ -71,17 +70,20 @@ cudaError_t launch_stream2d(int dtype, int k, int tile, const GridParams &g, con
 cudaError_t launch_stream3d(int dtype, int k, int tile, const GridParams &g,
                             const CUtensorMap *src_map, void *dst, int num_sms, cudaStream_t s);
 
-// Register-tile 2D stencils: launches of up to
-// kB2MaxDepth steps.  A plan covers `passes` passes of at most `depth` steps
-// each, spread evenly over plan.launches launches (an even count unless there
-// is a single pass); false if no variant serves the grid (FP64: if one step a
-// launch is faster).
+// Register-tile 2D stencils: launches of up to kB2MaxDepth steps.  A plan covers
+// `passes` passes of at most `depth` steps each (depths, or all of one step), spread
+// evenly over plan.launches launches (an even count unless there is a single pass);
+// false if the kernels that the tiles stand in for are faster, or none serves the
+// grid.  other: their time, from passes[k], the number of passes of depth k <=
+// kmax, on the streaming kernel (FP64: one step a launch).
 constexpr int kB2MaxDepth = 16;
 struct Block2DPlan {
   int variant, warps;
   int64_t launches;
 };
-bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, int num_sms, Block2DPlan *out);
+double block2d_other(int dtype, int tile, int64_t nx, int64_t ny, const int64_t *passes, int kmax, int num_sms);
+bool block2d_plan(int dtype, int64_t nx, int64_t ny, int64_t passes, int depth, const int *depths, double other,
+                  int num_sms, Block2DPlan *out);
 // One launch: k steps; bit s of round_mask rounds to the storage type after
 // step s + 1 (a pass end inside the launch).
 cudaError_t launch_block2d(int dtype, const Block2DPlan &p, const GridParams &g, const void *src, void *dst,

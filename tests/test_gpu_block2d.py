@@ -1,7 +1,8 @@
 """The kernels that stand in for the default schedule (2D register tiles, small
 3D grids) against the streaming kernel at the schedule they stand for: the
-same bits, for every variant that the rules can pick, with ragged tiles, grids smaller than a tile (the halo reflected
-several times), and step counts that split unevenly over the launches."""
+same bits, for every variant that the rules can pick (on 152 SMs), with ragged
+tiles, grids smaller than a tile (the halo reflected several times), and step
+counts that split unevenly over the launches."""
 import numpy as np
 import pytest
 
@@ -13,7 +14,11 @@ from gpu_util import assert_parity, oracle_run
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(1, 1), (1, 37), (29, 1), (3, 5), (17, 130), (200, 400), (513, 509), (1023, 1030), (2049, 2100)]
+# (16 and more steps: 4 rows a lane up to 513 x 509, 8 at 1023 x 1030, 7 for FP32
+# from 2049 x 2100 on and FP16 storage at 1500 x 1500, 9 beyond; 4100 x 4200: passes of
+# six steps; wide grids of few rows and large ones with few steps: streamed)
+SHAPES = [(1, 1), (1, 37), (29, 1), (3, 5), (17, 130), (200, 400), (513, 509), (1023, 1030), (1500, 1500),
+          (2049, 2100), (4100, 4200), (1, 200000), (3, 140000), (12, 130000)]
 
 
 @pytest.mark.parametrize("dtype", ["f32", "f16s"])
