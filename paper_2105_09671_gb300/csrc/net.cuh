@@ -228,11 +228,12 @@ __device__ __forceinline__ uint64_t net_gelu_fast2(uint64_t x) {
 //   gelu'(x) = (1 + t) / 2 + x/2 (1 - t^2) u' = s + 2 x u' s (e s),
 // in which nothing cancels: against FP64 over [-10, 10] its error is at most
 // 2.1e-7 (2.9e-8 rms), that of the form with tanhf 5.6e-7 (1.1e-7 rms).  e is
-// 2^y with the factor -2 log2(e) in u's coefficients; the exponent's bound
-// keeps e s finite.
+// 2^y with the factor -2 log2(e) in u's coefficients.  Beyond, it is 0 and 1: the
+// exponent's bound keeps e s finite while s, 2^-127, is flushed to 0, and x^2's
+// (from |x| = 20 on) the factor 2 x u' up to 1e36.
 __device__ __forceinline__ float net_exp2(float y) {
   float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fminf(y, 125.0f)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fminf(y, 127.0f)));
   return r;
 }
 __device__ __forceinline__ float net_rcp(float y) {
@@ -242,7 +243,7 @@ __device__ __forceinline__ float net_rcp(float y) {
 }
 __device__ __forceinline__ float net_gelu_grad(float x) {
   const float k = 0.7978845608028654f, l2e = 1.4426950408889634f, c = 0.044715f;
-  const float x2 = x * x;
+  const float x2 = fminf(x * x, 400.0f);
   const float e = net_exp2(x * fmaf(-2.0f * k * l2e * c, x2, -2.0f * k * l2e));
   const float s = net_rcp(1.0f + e);
   return fmaf(x * fmaf(6.0f * k * c, x2, 2.0f * k), s * (e * s), s);
@@ -252,7 +253,9 @@ __device__ __forceinline__ float net_gelu_grad(float x) {
 __device__ __forceinline__ uint64_t net_gelu_grad2(uint64_t x) {
   const float k = 0.7978845608028654f, l2e = 1.4426950408889634f, c = 0.044715f;
   const float a1 = -2.0f * k * l2e * c, a0 = -2.0f * k * l2e, b1 = 6.0f * k * c, b0 = 2.0f * k;
-  const uint64_t x2 = mul2(x, x);
+  float qa, qb;
+  unpack2(mul2(x, x), qa, qb);
+  const uint64_t x2 = pack2(fminf(qa, 400.0f), fminf(qb, 400.0f));
   float ya, yb;
   unpack2(mul2(x, fma2(pack2(a1, a1), x2, pack2(a0, a0))), ya, yb);
   const uint64_t e = pack2(net_exp2(ya), net_exp2(yb));

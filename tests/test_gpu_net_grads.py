@@ -48,3 +48,34 @@ def test_gradients_at_tile_edges(ndim, shape):
         for got, ref in ((gw, rw), (gb, rb)):
             assert _rel(got, ref) <= TOL_GRAD, f"layer {li}"
             assert _elementwise_ratio(got, ref) <= C_GRAD, f"layer {li}"
+
+
+@pytest.mark.parametrize("ndim,shape", [(2, (2, 9, 40)), (3, (1, 5, 6, 33))])
+@pytest.mark.parametrize("bias", [-30.0, -1e10, -1e13, -1e18, 1e10, 1e13, 1e18])
+@pytest.mark.parametrize("layer", [0, 2, 4])
+def test_saturated_units_pass_no_gradient_or_all_of_it(ndim, shape, bias, layer):
+    # pre-activations at which gelu' is 0 or 1 exactly (FP32): with negative ones the
+    # layers before get gradient 0; with positive ones and the next layer's weights 0
+    # (and the loss finite) it is 0 as well, and every gradient is finite
+    import torch
+    params = [(w.copy(), b.copy()) for w, b in _params(ndim, seed=11)]
+    params[layer][1][:] = bias
+    if bias > 0:
+        params[layer + 1][0][:] = 0.0
+    rng = np.random.default_rng(13)
+    phi = rng.uniform(-1, 1, size=shape)
+    h = L.ac_net_create(ndim, torch.cuda.current_stream().cuda_stream)
+    try:
+        L.ac_net_set_params(h, _flat(params))
+        d_phi = torch.tensor(phi, dtype=torch.float32, device="cuda")
+        d_tgt = d_phi + 0.1
+        b, nx, ny, nz = _shape_args(ndim, shape)
+        loss, g = L.ac_net_loss_grads(h, d_phi.data_ptr(), d_tgt.data_ptr(), b, nx, ny, nz, 0.1, want_grads=True)
+    finally:
+        L.ac_net_destroy(h)
+    assert np.isfinite(loss)
+    for li, (gw, gb) in enumerate(_unflat(g.astype(np.float64), params)):
+        if li <= layer:
+            assert np.max(np.abs(gw)) == 0.0 and np.max(np.abs(gb)) == 0.0, f"layer {li}"
+        elif bias < 0:
+            assert np.isfinite(gw).all() and np.isfinite(gb).all(), f"layer {li}"
