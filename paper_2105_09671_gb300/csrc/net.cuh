@@ -177,17 +177,7 @@ __device__ __forceinline__ void store_replicated(bf16 *outpad, const NetShape &s
       }
 }
 
-// The forward passes' GELU (tanh form) with the hardware tanh
-// approximation (tanh.approx.f32, relative error about 2^-11, below the BF16
-// rounding of the stored activation).
-__device__ __forceinline__ float net_gelu_fast(float x) {
-  const float k = 0.7978845608028654f;
-  const float u = k * fmaf(0.044715f * x, x * x, x);
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
-  return 0.5f * x * (1.0f + t);
-}
-// The same on two values with packed FP32 arithmetic (fma/mul.rn.f32x2: half
+// Two FP32 values as an operand of packed arithmetic (fma/mul/add.rn.f32x2: half
 // the issue slots).
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
   uint64_t r;
@@ -212,6 +202,9 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+// The forward passes' GELU (tanh form) of two values, with the hardware tanh
+// approximation (tanh.approx.f32, relative error about 2^-11, below the BF16
+// rounding of the stored activation).
 __device__ __forceinline__ uint64_t net_gelu_fast2(uint64_t x) {
   const float k = 0.7978845608028654f;
   const uint64_t u = mul2(x, fma2(pack2(k * 0.044715f, k * 0.044715f), mul2(x, x), pack2(k, k)));
