@@ -193,6 +193,8 @@ enum {
  * ac_step.  variant = AC_VARIANT_AUTO with k = 0 restores the default. */
 #define AC_MAX_K 8
 int ac_set_schedule(ac_ctx *ctx, int32_t variant, int32_t k);
+/* The schedule in effect (with ac_get_tile): what runs if it was forced, else the
+ * one whose results the steps have (see AC_VARIANT_AUTO). */
 int ac_get_schedule(ac_ctx *ctx, int32_t *variant, int32_t *k);
 
 /* Tile shape of the streaming kernel.  3D: the xy block each CTA streams
@@ -224,14 +226,16 @@ int ac_get_tile(ac_ctx *ctx, int32_t *tile);
  * phi is saved to a temporary device buffer that this call allocates and
  * frees, and restored after every trial, so the field is unchanged.  The
  * choice is cached per (ndim, dtype, log2 of the cell count, device model,
- * graph replay on or off) for the process lifetime (and in a file, see ac_set_tune_cache); later
- * contexts of the same class reuse it without timing.  Synchronises the
- * stream. */
+ * graph replay on or off, kernels that may stand in or not) for the process
+ * lifetime (and in a file, see ac_set_tune_cache); later contexts of the same
+ * class reuse it without timing.  A schedule or tile forced on the context is
+ * set aside meanwhile.  Synchronises the stream. */
 int ac_autotune(ac_ctx *ctx, int64_t steps_per_trial);
 
 /* Keep autotuning results in a text file as well (one line per choice:
  * "ac-tune-v2 ndim dtype size_class device graph variant k tile", device =
- * the model name and SM count, graph = 1 for choices timed as graph
+ * the model name and SM count, with "+s" where other kernels may stand in for
+ * the default schedule (choices timed without them don't apply), graph = 1 for choices timed as graph
  * replays; lines of the earlier v1 form, without the graph field, are read
  * as graph = 0), so that later processes skip the timing:
  * ac_autotune first looks in the process cache, then in the file, and

@@ -399,16 +399,19 @@ bool ac_plan_depths(int64_t n, int k, std::vector<int> &depths) {
   return false;
 }
 
-// Whether a schedule may run on the kernels that stand in for the default
-// one's (in 2D the register-tile kernels of block2d.cuh and block2d_fx.cuh, on
-// small 3D FP32 grids step3d_vec): the default schedule, unless the caller
-// forced a schedule or a tile (those run as asked).  The results are bit for
-// bit those of the default schedule's passes: FP32 and FP64 do not depend on
-// the depth, and FP16 storage is rounded where they end.
+// Whether the default schedule of a grid may run on the kernels that stand in for
+// its own (in 2D the register-tile kernels of block2d.cuh and block2d_fx.cuh, on
+// small 3D FP32 grids step3d_vec).  The results are bit for bit those of its
+// passes: FP32 and FP64 do not depend on the depth, and FP16 storage is rounded
+// where they end.
+static bool stand_in_offered(const ac_ctx *c) {
+  if (c->d.ndim == 3) return step3d_vec_serves(c->d.dtype, c->gp);
+  return c->d.dtype != AC_F64 || c->gp.fx.limit != 0;
+}
+// Whether a schedule takes them: the default one, unless the caller forced a
+// schedule or a tile (those run as asked).
 static bool takes_stand_in(const ac_ctx *c, int variant, int k, int tile) {
-  if (c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO) return false;
-  if (c->d.ndim == 3 && !step3d_vec_serves(c->d.dtype, c->gp)) return false;
-  if (c->d.dtype == AC_F64 && !c->gp.fx.limit) return false;
+  if (c->variant != AC_VARIANT_AUTO || c->tile != AC_TILE_AUTO || !stand_in_offered(c)) return false;
   int dv, dk;
   default_schedule(c, &dv, &dk);
   return variant == dv && k == dk && tile == default_tile(c, dk);
@@ -640,7 +643,9 @@ extern "C" int ac_init_random(ac_ctx *c, uint64_t seed, double amplitude) {
 namespace {
 // Tuning results are keyed by grid kind, storage type, size class (log2 of
 // the cell count) and the device model (name and SM count, so that a cache
-// file carries over between processes and between GPUs of the same model).
+// file carries over between processes and between GPUs of the same model; "+s"
+// where other kernels may stand in for the default schedule, whose time then is
+// theirs: choices timed without them don't apply).
 struct TuneKey {
   int ndim, dtype, cls;
   std::string device;
@@ -656,13 +661,13 @@ struct TuneChoice {
 std::map<TuneKey, TuneChoice> g_tune_cache;
 std::string g_tune_file;  // optional on-disk cache (empty: none)
 
-std::string device_key(int device) {
+std::string device_key(int device, bool stand_in) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return "unknown";
   std::string name(prop.name);
   for (char &ch : name)
     if (ch == ' ' || ch == '\t') ch = '_';
-  return name + "_sm" + std::to_string(prop.multiProcessorCount);
+  return name + "_sm" + std::to_string(prop.multiProcessorCount) + (stand_in ? "+s" : "");
 }
 
 // File format, one entry per line:
@@ -715,7 +720,8 @@ static int size_class(const ac_grid_desc &d) {
 extern "C" int ac_autotune(ac_ctx *c, int64_t steps_per_trial) {
   if (!c) return fail(AC_ERR_INVALID, "ctx is NULL");
   if (steps_per_trial < 1) return fail(AC_ERR_INVALID, "steps_per_trial must be >= 1");
-  const TuneKey key{c->d.ndim, c->d.dtype, size_class(c->d), device_key(c->device),
+  const TuneKey key{c->d.ndim, c->d.dtype, size_class(c->d),
+                    device_key(c->device, stand_in_offered(c)),
                     (c->use_graph && c->stream != nullptr) ? 1 : 0};
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -746,6 +752,10 @@ extern "C" int ac_autotune(ac_ctx *c, int64_t steps_per_trial) {
   float best = 1e30f;
   TuneChoice best_c = cand.front();
   cudaMemcpyAsync(backup, c->phi, bytes, cudaMemcpyDeviceToDevice, c->stream);
+  // A forced schedule or tile is for the caller's steps, not for the trials.
+  const int forced_variant = c->variant, forced_tile = c->tile;
+  c->variant = AC_VARIANT_AUTO;
+  c->tile = AC_TILE_AUTO;
   // A context that replays its steps through a CUDA graph has them timed the
   // same way (small grids are bound by launch overhead, which graphs remove).
   const bool graphed = c->use_graph && c->stream != nullptr;
@@ -792,6 +802,8 @@ extern "C" int ac_autotune(ac_ctx *c, int64_t steps_per_trial) {
     if (per_step < best) { best = per_step; best_c = cd; }
     cudaMemcpyAsync(c->phi, backup, bytes, cudaMemcpyDeviceToDevice, c->stream);
   }
+  c->variant = forced_variant;
+  c->tile = forced_tile;
   cudaStreamSynchronize(c->stream);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

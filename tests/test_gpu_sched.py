@@ -155,3 +155,48 @@ def test_autotune_with_graph_replay_times_graphs():
     finally:
         sim.close()
     assert_parity(out, oracle_run(phi0, h, eps, dt, 40, "f64"), "f64", f"graph-tuned v{v} k{k}")
+
+
+def test_a_forced_schedule_does_not_enter_the_trials():
+    # choices are kept for every context of the class: while a schedule is
+    # forced the trials still time the default one on the kernels that stand in
+    # for it (here many times faster than any streaming schedule)
+    shape = (300, 310)
+    h = 1.0 / 310
+    ac.ac_set_tune_cache(None)  # (empties the process's choices)
+    sim = ac.Simulation(shape, h, 2.5 * h, 0.1 * h * h, dtype="f32")
+    try:
+        default = sim.schedule(), sim.tile()
+        sim.load(wl.smooth_field(shape, seed=5))
+        sim.set_schedule(ac.AC_VARIANT_DIRECT, 1)
+        sim.set_tile(1)
+        sim.autotune(240)
+        assert sim.schedule() == (ac.AC_VARIANT_DIRECT, 1)
+        sim.set_schedule(ac.AC_VARIANT_AUTO, 0)
+        sim.set_tile(-1)
+        assert (sim.schedule(), sim.tile()) == default
+    finally:
+        sim.close()
+        ac.ac_set_tune_cache(None)
+
+
+def test_choices_timed_without_the_stand_in_kernels_do_not_apply(tmp_path):
+    # lines of earlier builds name the device without the mark of grids whose
+    # default schedule runs on other kernels
+    import torch
+    p = torch.cuda.get_device_properties(0)
+    dev = p.name.replace(" ", "_") + f"_sm{p.multi_processor_count}"
+    path = tmp_path / "tune.txt"
+    cls = int(np.floor(np.log2(300 * 310)))
+    path.write_text(f"ac-tune-v2 2 {ac.AC_F32} {cls} {dev} 0 {ac.AC_VARIANT_DIRECT} 1 0\n")
+    h = 1.0 / 310
+    ac.ac_set_tune_cache(str(path))
+    sim = ac.Simulation((300, 310), h, 2.5 * h, 0.1 * h * h, dtype="f32")
+    try:
+        n0 = sim.launch_count()
+        sim.autotune(48)
+        assert sim.launch_count() > n0, "adopted without timing"
+        assert path.read_text().splitlines()[-1].split()[4] == dev + "+s"
+    finally:
+        sim.close()
+        ac.ac_set_tune_cache(None)
