@@ -406,7 +406,11 @@ bool ac_plan_depths(int64_t n, int k, std::vector<int> &depths) {
 // where they end.
 static bool stand_in_offered(const ac_ctx *c) {
   if (c->d.ndim == 3) return step3d_vec_serves(c->d.dtype, c->gp);
-  return c->d.dtype != AC_F64 || c->gp.fx.limit != 0;
+  if (c->d.dtype != AC_F64) return true;
+  // (Temperatures of the heat equation send more cells through the FP64
+  // operations, for which a tile waits: a hot square in a cold 200^2 3.0 us a step
+  // in tiles, 1.9 with one step a launch; 64^2 1.3 against 1.5.)
+  return c->gp.fx.limit != 0 && (c->gp.alpha > 0.0 || c->d.nx * c->d.ny <= 10000);
 }
 // Whether a schedule takes them: the default one, unless the caller forced a
 // schedule or a tile (those run as asked).

@@ -72,8 +72,7 @@ __global__ void __launch_bounds__(kB2FxMaxWarps * 32)
         if (!((any >> r) & 1u)) continue;
         const double vw = __shfl_up_sync(0xffffffffu, v[r], 1), ve = __shfl_down_sync(0xffffffffu, v[r], 1);
         const double vb = r == 0 ? sv[ib] : v[r > 0 ? r - 1 : 0], va = r == R - 1 ? sv[ia] : v[r + 1 < R ? r + 1 : 0];
-        const double t = ac_update<double>(v[r], (vw + ve) + (vb + va), -4.0, coef.alpha, coef.beta);
-        if ((fp64 >> r) & 1u) nv[r] = t;
+        if ((fp64 >> r) & 1u) nv[r] = fx_plain<2>(v[r], {vw, ve, vb, va}, coef);
       }
     }
 #pragma unroll

@@ -167,8 +167,7 @@ __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__re
       for (int e = 0; e < kFx2E; ++e) {
         if (ok[e]) continue;
         const int im = xi[e] > 0 ? xi[e] - 1 : 0, ip = min(xi[e] + 1, nx - 1);
-        out[e] = ac_update<double>(row[xi[e]], (row[im] + row[ip]) + (rs[xi[e]] + rn[xi[e]]), -4.0, coef.alpha,
-                                   coef.beta);
+        out[e] = fx_plain<2>(row[xi[e]], {row[im], row[ip], rs[xi[e]], rn[xi[e]]}, coef);
       }
     }
     fx_store<kFx2E>(dst + (int64_t)y * g.pitch, xl, lane, nx, out);
@@ -253,11 +252,10 @@ __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restr
         for (int e = 0; e < E; ++e) {
           if (ok[e]) continue;
           const int im = xi[e] > 0 ? xi[e] - 1 : 0, ip = min(xi[e] + 1, nx - 1);
-          out[e] = ac_update<double>(
-              row[xi[e]],
-              ((row[im] + row[ip]) + (pl[ro[r] + xi[e]] + pl[ro[r + 2] + xi[e]])) +
-                  (src[(int64_t)max(z - 1, 0) * plane + ro[r + 1] + xi[e]] + zp[ro[r + 1] + xi[e]]),
-              -6.0, coef.alpha, coef.beta);
+          out[e] = fx_plain<3>(row[xi[e]],
+                               {row[im], row[ip], pl[ro[r] + xi[e]], pl[ro[r + 2] + xi[e]],
+                                src[(int64_t)max(z - 1, 0) * plane + ro[r + 1] + xi[e]], zp[ro[r + 1] + xi[e]]},
+                               coef);
         }
       }
       if (y0 + r < ny) fx_store<E>(dst + (int64_t)z * plane + (int64_t)(y0 + r) * g.pitch, xl, lane, nx, out);

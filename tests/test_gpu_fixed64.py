@@ -228,6 +228,26 @@ def test_temperatures_of_any_size_give_the_same_bits_on_every_kernel(shape):
             assert np.max(np.abs(outs[0] - ref)) <= 1e-14 * 400
 
 
+@pytest.mark.parametrize("shape", [(40, 64), (200, 210), (1003, 1001), (9, 13, 61), (99, 101, 103)])
+@pytest.mark.parametrize("eps", [np.inf, 2.5 / 64])
+def test_fields_at_rest_stay_so_beside_others(shape, eps):
+    # zeros of either sign, a square of other values among them and subnormal ones
+    # in its neighbourhood; the same bits on every kernel
+    h = 1.0 / 64
+    phi0 = np.zeros(shape)
+    phi0[..., ::3] = -0.0
+    mid = tuple(slice(n // 3, n // 3 + max(1, n // 8)) for n in shape)
+    phi0[mid] = 0.9 * wl.random_field(phi0[mid].shape, seed=4)
+    phi0.reshape(-1)[3:6] = [5e-324, -3e-310, 1e-300]
+    outs = [gpu_run(phi0, h, eps, 0.1 * h * h, 4, "f64", *s)
+            for s in ((), (ac.AC_VARIANT_DIRECT, 1), (ac.AC_VARIANT_STREAM, 1), (ac.AC_VARIANT_STREAM, 2))]
+    for o in outs[1:]:
+        assert np.array_equal(outs[0], o)
+    ref = oracle.step(phi0, h, eps, 0.1 * h * h, 4)
+    assert np.max(np.abs(outs[0] - ref)) <= 1e-14
+    assert np.array_equal(outs[0] == 0.0, ref == 0.0)
+
+
 @pytest.mark.parametrize("shape,n", [((16, 16), 2000), ((40, 64), 600), ((520, 510), 100), ((4, 6, 64), 600)])
 def test_a_field_odd_about_its_middle_stays_so(shape, n):
     h = 1.0 / 64
