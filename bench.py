@@ -337,8 +337,11 @@ def measure_grid(w, dtype, jobs, warmup, local):
         peak, _ = hbm_peak()
         launch_s = ms / 1e3 / max(1, launches)
         return {"workload": w.name, "grid": list(w.shape), "dtype": dtype, "euler_steps": w.steps,
+                # the default schedule; where launches take other numbers of steps than its k,
+                # the kernels that stand in for it ran (AC_VARIANT_AUTO in ac.h)
                 "jobs": jobs, "schedule": {"variant": "stream" if v == 2 else "direct", "k": k,
-                                           "tile": sim.tile()},
+                                           "tile": sim.tile(),
+                                           "steps_per_launch": w.steps * jobs / max(1, launches)},
                 "value": w.cells * w.steps * jobs / (ms / 1e3) / 1e9, "unit": UNIT,
                 "avg_launch_ms": launch_s * 1e3,
                 "hbm_frac_per_launch": 2 * es * w.cells / launch_s / 1e9 / peak}

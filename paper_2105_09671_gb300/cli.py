@@ -62,19 +62,24 @@ def main(argv=None):
     tile = sim.tile()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     times = []
+    n0 = sim.launch_count()
     for _ in range(args.repeat):
         e0.record(stream)
         sim.step(args.steps)
         e1.record(stream)
         stream.synchronize()
         times.append(e0.elapsed_time(e1))
+    launches = (sim.launch_count() - n0) / args.repeat
     energy = sim.energy()
     cells = 1
     for s in shape:
         cells *= s
     best = min(times)
     print(json.dumps({"shape": list(shape), "dtype": args.dtype, "variant": v, "k": k, "tile": tile,
-                      "graph": bool(args.graph), "steps": args.steps, "ms": best,
+                      "graph": bool(args.graph), "steps": args.steps,
+                      # unless a schedule is forced, kernels of other depths may run
+                      # for it (AC_VARIANT_AUTO in ac.h)
+                      "launches": launches, "ms": best,
                       "gcell_updates_per_s": cells * args.steps / (best / 1e3) / 1e9,
                       "energy": energy, "status": sim.status()}))
     sim.close()
