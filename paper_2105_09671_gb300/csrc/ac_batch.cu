@@ -92,12 +92,17 @@ static void release_graph(ac_batch *b) {
 // (every item computes 2k halo rows more and fills its pipeline).  They meet
 // where there are about 1.25 items to a warp, so the fewest rows (a multiple of
 // 4, at least 8) that keep to it; on large batches, where no size does, 256.
+// Grids whose width is no multiple of the vector's take more instructions a row
+// and are shared out better in items of 64 rows, while these are two to a warp at
+// most (64 such grids to 1024^2, 100 steps: FP32 2.51 ms with 76 rows, 2.42, FP16
+// storage 5.0 with 84, 4.0; 64 grids of multiples of 32, FP32: 1.51 and 1.55).
+// From 16 rows on, but for FP64, up to the next even number that leaves the row
+// loop, unrolled by three, no remainder (FP16 storage 4.6 ms with 88).
 // FP32, 64 rows always -> this: 16 grids to 256^2 27 -> 11 us a block, 32 of
-// 256^2 to 512^2 36 -> 20, 64 to 1024^2 66 -> 65, 512 to 1024^2 449 -> 395;
-// FP16 storage alike.  FP64 is bound by arithmetic at any size and wants many
-// items to share out evenly: 64 rows at most (64 grids to 1024^2: 1.95 ms a
-// block against 2.15 with 1.25 items to a warp; 16 to 256^2 0.74 -> 0.13).
-static int rows_per_item(const ac_batch *b, int ow, int64_t warps) {
+// 256^2 to 512^2 36 -> 20, 64 to 1024^2 66 -> 65, 512 to 1024^2 449 -> 395.  FP64 is
+// bound by arithmetic at any size and wants many items to share out evenly: 64
+// rows at most.
+static int rows_per_item(const ac_batch *b, int ow, int vec, int k, int64_t warps) {
   auto items = [&](int64_t rows) {
     int64_t n = 0;
     for (const ac_grid_desc &d : b->d) n += ((d.nx + ow - 1) / ow) * ((d.ny + rows - 1) / rows);
@@ -109,7 +114,13 @@ static int rows_per_item(const ac_batch *b, int ow, int64_t warps) {
     if (items(4 * mid) * 4 <= warps * 5) hi = mid;
     else lo = mid + 1;
   }
-  return 4 * lo;
+  int rows = 4 * lo;
+  int whole = 0;
+  for (const ac_grid_desc &d : b->d) whole += d.nx % vec == 0;
+  if (2 * whole < b->count && rows > 64 && items(64) <= 2 * warps) rows = 64;
+  if (b->dtype != AC_F64 && rows > 16)
+    while ((rows + 2 * k) % 3) rows += 2;
+  return rows;
 }
 
 // Work items for plan depth k: per instance, strips of the 2D streaming
@@ -123,7 +134,7 @@ static int build_items(ac_batch *b, int k) {
   int ctas = 0;  // of the launch (no steps: only the grid's size)
   BC_CUDA(batch2d_launch(b->dtype, b->tile, nullptr, nullptr, 0, nullptr, nullptr, nullptr, 0, nullptr, 0,
                          b->num_sms, b->stream, &ctas));
-  b->chunk_rows = rows_per_item(b, ow, (int64_t)ctas * kBatchWarps);
+  b->chunk_rows = rows_per_item(b, ow, vec, k, (int64_t)ctas * kBatchWarps);
   b->h_items.clear();
   for (int i = 0; i < b->count; ++i) {
     const ac_grid_desc &d = b->d[i];

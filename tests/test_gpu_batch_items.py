@@ -11,9 +11,12 @@ pytestmark = pytest.mark.gpu
 
 
 # (513, 500) is 5 strips: 2 grids take 8 rows (FP32: 1.25 items to each of 2432
-# resident warps), 60 grids 52, 300 grids 256 (even these leave 4500 items).
-@pytest.mark.parametrize("dtype,k,copies", [("f32", 4, 2), ("f32", 4, 60), ("f32", 4, 300),
-                                            ("f16s", 3, 300), ("f64", 1, 60), ("f64", 3, 2)])
+# resident warps), 60 grids 52, 300 grids 256 (even these leave 4500 items); FP16
+# storage, 3 strips, 80 grids 64 rows.  Depths 4 and 3 round the rows up to 4 and 0
+# modulo 6.
+@pytest.mark.parametrize("dtype,k,copies", [("f32", 4, 2), ("f32", 4, 60), ("f32", 4, 300), ("f32", 2, 60),
+                                            ("f16s", 3, 300), ("f16s", 4, 80), ("f16s", 3, 80), ("f64", 1, 60),
+                                            ("f64", 3, 2)])
 def test_item_heights_equal_single_grid_stepper(dtype, k, copies):
     shapes = [(513, 500), (9, 130), (257, 33)]
     inits = [oracle.init_random(s, seed=7 + i) for i, s in enumerate(shapes)]
