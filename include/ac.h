@@ -591,7 +591,7 @@ int ac_slab_destroy(ac_slab *slab);
  *
  * Asynchronous: nothing is copied to the host and the stream is not
  * synchronised.  Grids with ny * nz above 1048576 rows (the fixed scratch
- * holds 16384 blocks of 64 rows) are rejected with AC_ERR_INVALID and a
+ * holds 16384 blocks of at most 64 rows) are rejected with AC_ERR_INVALID and a
  * message naming the limit.  The first call on each device looks up the
  * array's device address with that device current; make that first call
  * before any stream capture on the device.  All calls on a device share the

@@ -183,11 +183,15 @@ __global__ void __launch_bounds__(256) observe_k(const T *__restrict__ phi, Grid
 // One warp to a segment of 512 cells (16 a lane, a float-float group).  With one
 // warp to a row, two kernels and 20 FP64 additions a lane to reduce a warp,
 // 1024^2 FP32 took 27 + 8 us.
+static int observe_blocks(const GridParams &g) {
+  const int64_t units = g.ny * g.nz * ((g.nx + 32 * kFFGroup - 1) / (32 * kFFGroup));
+  return (int)std::min<int64_t>((units + 7) / 8, kReduceBlocks);
+}
+
 template <typename T>
 static cudaError_t observe_t(const GridParams &g, const void *phi, double *partials, double *out,
                              cudaStream_t s) {
-  const int64_t units = g.ny * g.nz * ((g.nx + 32 * kFFGroup - 1) / (32 * kFFGroup));
-  const int blocks = (int)std::min<int64_t>((units + 7) / 8, kReduceBlocks);
+  const int blocks = observe_blocks(g);
   observe_k<T><<<blocks, 256, 0, s>>>((const T *)phi, g, partials,
                                       reinterpret_cast<unsigned int *>(partials + 4 * kReduceBlocks), out);
   return cudaGetLastError();
@@ -210,10 +214,10 @@ cudaError_t observe_alloc(double **partials, cudaStream_t s) {
 }
 
 // ------------------------------------------------- allocation-free variant --
-// ac_observe_noalloc (see include/ac.h) forms the same per-block partial sums,
-// but over a grid of one block per kNoAllocRowsPerBlock rows, with
-// its partial sums in the fixed array below instead of a buffer from
-// ac_create.  The array is a module global: every GPU that loads the library
+// ac_observe_noalloc (see include/ac.h) forms the same per-block partial sums, over
+// as many blocks (more for grids of many rows: one to kNoAllocRowsPerBlock), in the
+// fixed array below instead of a buffer from ac_create.  (64 blocks for 4096^2
+// took 356 us with a warp to 512 cells, 309 with a warp to a row.)  The array is a module global: every GPU that loads the library
 // holds its 512 KiB until the process exits, and all calls on a device share
 // it.  Each call writes every partial slot it later reads, so nothing in it
 // has to start at zero; two calls that overlap on the GPU (e.g. on different
@@ -288,7 +292,7 @@ cudaError_t launch_observe_noalloc(int dtype, const GridParams &g, const void *p
   if (e != cudaSuccess) return e;
   double *scratch = noalloc_scratch(device, &e);
   if (!scratch) return e;
-  const int nb = (int)std::max<int64_t>(1, (rows + kNoAllocRowsPerBlock - 1) / kNoAllocRowsPerBlock);
+  const int nb = (int)std::max<int64_t>(observe_blocks(g), (rows + kNoAllocRowsPerBlock - 1) / kNoAllocRowsPerBlock);
   switch (dtype) {
     case AC_F64: observe_partial<double><<<nb, 256, 0, s>>>((const double *)phi, g, scratch); break;
     case AC_F32: observe_partial<float><<<nb, 256, 0, s>>>((const float *)phi, g, scratch); break;
