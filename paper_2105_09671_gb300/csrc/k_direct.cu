@@ -116,9 +116,10 @@ __device__ __forceinline__ void fx_store(double *row, int xl, int lane, int nx, 
 }
 
 // A warp owns kFx2W columns and marches over `chunk` rows.  Bound by integer
-// issue (some 140 instructions a cell, 14 of them wide multiply-adds, which
-// take more than one slot: 63 % of the slots busy): 4096^2 253 -> 94 us a
-// step, 2048^2 64 -> 28 against the FP64 operations.
+// issue (some 164 instructions a cell, 14 of them wide multiply-adds, which
+// take more than one slot: 64 % of the slots busy): 4096^2 253 -> 104 us a
+// step (from noise 113: more cells take the FP64 operations), 2048^2 64 -> 30
+// against the FP64 operations alone.
 __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__restrict__ src,
                                                            double *__restrict__ dst, GridParams g, int strips,
                                                            int chunk) {
@@ -181,8 +182,8 @@ __global__ void __launch_bounds__(kFxWarps * 32, 6) step2d_fx(const double *__re
 
 // A warp owns kFx3W columns of kFx3R rows and marches over `chunk` planes; it
 // takes apart kFx3R + 2 rows of each plane (against a barrier a plane to share
-// them; two rows in 124 registers rather than three or four in 160).  256^3
-// 317 -> 159 us a step, 200 x 100 x 100 45 -> 23.
+// them; two rows in 128 registers rather than three or four in 160).  256^3
+// 317 -> 165 us a step, 200 x 100 x 100 45 -> 27.
 __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restrict__ src,
                                                            double *__restrict__ dst, GridParams g, int strips,
                                                            int bands, int chunk) {
@@ -269,14 +270,14 @@ __global__ void __launch_bounds__(kFxWarps * 32) step3d_fx(const double *__restr
 
 // Rows (planes) per item of a march.  An item converts two more rows than it
 // writes and starts with a wait for memory (together `pro` rows' time), and an
-// SM holds kFxOcc CTAs: with q CTAs to an SM a row of each takes one + add q us
+// SM holds `occ` CTAs: with q CTAs to an SM a row of each takes one + add q us
 // up to one full round, with more of them `full` us a round.  So for every q
 // the most items that keep to it, and of these the cheapest (up to 24 CTAs to
-// an SM more than the fewest: there the starts of the items outweigh the rest).  Fitted to sweeps
-// over chunks for 64^3 .. 256^3 and 1152^2 .. 8192^2, where the choice is
+// an SM more than the fewest: there the starts of the items outweigh the rest).
+// Fitted to sweeps over chunks for 64^3 .. 256^3 and 1152^2 .. 8192^2, where the choice is
 // within 4 % of the best.  One round of about 16 (2D: 24) warps an SM, rounded
-// to whole items, took 197 us against 159 at 256^3, whose CTAs it dealt 3.2 to
-// an SM, and 375 against 351 at 8192^2.
+// to whole items, took 24 % longer at 256^3, whose CTAs it dealt 3.2 to an SM, and
+// 7 % at 8192^2.
 struct FxMarch {
   int occ;
   double one, add, full, pro;

@@ -376,7 +376,7 @@ __host__ __device__ constexpr int last_bwd_smem() {
 // Second pass: dW6[t][c] += a5[p + t][c] g6[p] from the staged a5.
 // Bound by instruction issue and latency (about 9 + 9 multiply-adds and a
 // gelu' per cell and channel, on two channels an instruction; 16 warps to an SM
-// in 128 registers).  32 x 256^2 cells: 155 us; with scalar arithmetic 196, the
+// in 128 registers).  32 x 256^2 cells: 160 us; with scalar arithmetic 196, the
 // copies not asynchronous 245, one warp per cell and every operand read from
 // global memory 2818.
 template <int NDIM>

@@ -35,7 +35,7 @@
 // A rows were read 18 times (2D) instead of 6 to 8 times: 720 clocks of
 // 128-byte reads per 128-pixel row.  In training the activations come next:
 // 32 x 256^2 pixels move 400 MB a layer (59 us at the copy rate) and take 80 us
-// forward, 85 us for the data gradient; 1024^2 without pre-activations 33 us
+// forward, 87 us for the data gradient; 1024^2 without pre-activations 33 us
 // (47 before the three rows shared an MMA).  A third epilogue group: 86 us.
 // Every wait is bounded; a timeout sets the status word and the roles wind
 // down without leaving copies or MMAs in flight.

@@ -241,7 +241,7 @@ __device__ __forceinline__ float net_gelu_grad(float x) {
   const float s = net_rcp(1.0f + e);
   return fmaf(x * fmaf(6.0f * k * c, x2, 2.0f * k), s * (e * s), s);
 }
-// The same on two values, packed: the data gradient's kernel takes 85 us with
+// The same on two values, packed: the data gradient's kernel takes 87 us with
 // it, 115 with the scalar form (32 x 256^2 pixels).
 __device__ __forceinline__ uint64_t net_gelu_grad2(uint64_t x) {
   const float k = 0.7978845608028654f, l2e = 1.4426950408889634f, c = 0.044715f;
