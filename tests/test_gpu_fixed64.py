@@ -13,9 +13,9 @@ from gpu_util import gpu_run, schedules
 
 pytestmark = pytest.mark.gpu
 
-# marching kernels from 512^2 cells on: strips of 124 (2D) and 60 (3D) columns, bands of 2 rows
+# marching kernels from 1 M cells on (3D 0.7 M): strips of 124 (2D) and 60 (3D) columns, bands of 2 rows
 SHAPES = [(1, 1), (3, 5), (9, 123), (33, 125), (130, 249), (1, 1, 1), (2, 3, 5), (5, 9, 59), (9, 13, 61), (4, 4, 121), (600, 700),
-          (65, 64, 66)]
+          (65, 64, 66), (1003, 1001), (99, 101, 103)]
 
 
 def _step_long(phi, h, eps, dt):
@@ -32,11 +32,13 @@ def _step_long(phi, h, eps, dt):
     return p + alpha * (p - p * p * p) + beta * (s - 2 * p.ndim * p)
 
 
-@pytest.mark.parametrize("shape", [(1, 1), (3, 5), (29, 31), (64, 64), (97, 200), (515, 517), (700, 900)])
+@pytest.mark.parametrize("shape", [(1, 1), (3, 5), (29, 31), (64, 64), (97, 200), (515, 517), (700, 900),
+                                   (1003, 1009)])
 @pytest.mark.parametrize("amp", [1.0, 0.1, 3.0])
 def test_default_equals_one_step_a_launch_bitwise(shape, amp):
-    # the register-tile kernel (several steps a launch; tiles with a value out
-    # of range mix both forms) and, from 512^2 cells on, the marching kernel
+    # the register-tile kernel up to 50000 cells (several steps a launch; tiles
+    # with a value out of range mix both forms), one thread a cell and, from 1 M
+    # cells on, the marching kernel
     h = 1.0 / max(shape)
     eps, dt = 2.5 * h, (0.1 if amp < 2 else 0.02) * h * h
     phi0 = amp * wl.random_field(shape, seed=sum(shape))
