@@ -105,8 +105,9 @@ static bool same_shape(const NetShape &a, const NetShape &b) {
 
 // Per-shape buffers: inference keeps two padded activations; training keeps
 // all five, the pre-activations, the padded gradients (zero ghost ring, set
-// once here) and the FP32 scratch.
-static int ensure_shape(ShapeBufs &s, const NetShape &sh, bool train) {
+// once here, on the network's stream: nothing orders the legacy stream before a
+// non-blocking one) and the FP32 scratch.
+static int ensure_shape(ShapeBufs &s, const NetShape &sh, bool train, cudaStream_t stream) {
   if (s.valid && same_shape(s.sh, sh) && s.train == train) return AC_OK;
   free_shape(s);
   const size_t act = (size_t)sh.padded_cells() * kNetC * sizeof(bf16);
@@ -117,7 +118,7 @@ static int ensure_shape(ShapeBufs &s, const NetShape &sh, bool train) {
     for (int i = 0; i < 5; ++i) {
       NC_CUDA(cudaMalloc(&s.nb.z[i], zb));
       NC_CUDA(cudaMalloc(&s.nb.gz[i], act));
-      NC_CUDA(cudaMemset(s.nb.gz[i], 0, act));
+      NC_CUDA(cudaMemsetAsync(s.nb.gz[i], 0, act, stream));
     }
     NC_CUDA(cudaMalloc(&s.nb.raw, (size_t)sh.cells() * kNetC * sizeof(float)));
     NC_CUDA(cudaMalloc(&s.nb.g6, (size_t)sh.cells() * sizeof(float)));
@@ -212,9 +213,9 @@ extern "C" int ac_net_create(int32_t ndim, void *cuda_stream, ac_net **out) {
   std::vector<float> init;
   he_init(b.layout, 0, init);
   if (e == cudaSuccess) e = cudaMemcpy(b.params, init.data(), pbytes, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(b.m, 0, pbytes);
-  if (e == cudaSuccess) e = cudaMemset(b.v, 0, pbytes);
-  if (e == cudaSuccess) e = cudaMemset(b.status, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.m, 0, pbytes, net->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.v, 0, pbytes, net->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.status, 0, sizeof(int), net->stream);
   if (e == cudaSuccess) e = net_pack(b, net->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
   if (e != cudaSuccess) {
@@ -251,8 +252,8 @@ extern "C" int ac_net_set_params(ac_net *net, const float *host_params, int64_t 
   NC_CUDA(cudaStreamSynchronize(net->stream));
   NC_CUDA(cudaMemcpy(net->base.params, host_params, count * sizeof(float), cudaMemcpyHostToDevice));
   const size_t pbytes = (size_t)count * sizeof(float);
-  NC_CUDA(cudaMemset(net->base.m, 0, pbytes));
-  NC_CUDA(cudaMemset(net->base.v, 0, pbytes));
+  NC_CUDA(cudaMemsetAsync(net->base.m, 0, pbytes, net->stream));
+  NC_CUDA(cudaMemsetAsync(net->base.v, 0, pbytes, net->stream));
   net->adam_step = 0;
   net->grads_valid = false;
   NC_CUDA(net_pack(net->base, net->stream));
@@ -282,7 +283,7 @@ extern "C" int ac_net_forward(ac_net *net, const float *phi_dev, float *out_dev,
   NetShape sh;
   int rc = check_shape(net->ndim, batch, nx, ny, nz, &sh);
   if (rc) return rc;
-  rc = ensure_shape(net->infer, sh, false);
+  rc = ensure_shape(net->infer, sh, false, net->stream);
   if (rc) return rc;
   cudaError_t e = net_forward(merged(net, net->infer), sh, phi_dev, (float)scale, out_dev, nullptr,
                               false, net->num_sms, net->stream);
@@ -299,7 +300,7 @@ extern "C" int ac_net_loss_grads(ac_net *net, const float *phi_dev, const float 
   NetShape sh;
   int rc = check_shape(net->ndim, batch, nx, ny, nz, &sh);
   if (rc) return rc;
-  rc = ensure_shape(net->train, sh, true);
+  rc = ensure_shape(net->train, sh, true, net->stream);
   if (rc) return rc;
   const NetBuffers nb = merged(net, net->train);
   NC_CUDA(cudaMemsetAsync(nb.loss, 0, sizeof(double), net->stream));
@@ -316,7 +317,7 @@ extern "C" int ac_net_loss_grads(ac_net *net, const float *phi_dev, const float 
   int st = 0;
   NC_CUDA(cudaMemcpy(&st, nb.status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st) {
-    NC_CUDA(cudaMemset(nb.status, 0, sizeof(int)));
+    NC_CUDA(cudaMemsetAsync(nb.status, 0, sizeof(int), net->stream));
     return nfail(AC_ERR_TIMEOUT, "a bounded tensor-core wait expired");
   }
   if (grads_host)

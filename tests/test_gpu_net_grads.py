@@ -79,3 +79,30 @@ def test_saturated_units_pass_no_gradient_or_all_of_it(ndim, shape, bias, layer)
             assert np.max(np.abs(gw)) == 0.0 and np.max(np.abs(gb)) == 0.0, f"layer {li}"
         elif bias < 0:
             assert np.isfinite(gw).all() and np.isfinite(gb).all(), f"layer {li}"
+
+
+def test_buffers_are_cleared_in_the_order_of_the_networks_stream():
+    # a network on a non-blocking stream, the legacy stream busy: the zero ghost
+    # ring of its gradients must not wait for that stream
+    import torch
+    params = _params(2, seed=11)
+    rng = np.random.default_rng(13)
+    phi = rng.uniform(-1, 1, size=(4, 70, 150)).astype(np.float32)
+    d_phi = torch.tensor(phi, device="cuda")
+    d_tgt = d_phi + 0.1
+    big = torch.rand((8192, 8192), device="cuda")
+    grads = []
+    for busy in (False, True):
+        stream = torch.cuda.Stream()
+        h = L.ac_net_create(2, stream.cuda_stream)
+        try:
+            L.ac_net_set_params(h, _flat(params))
+            torch.cuda.synchronize()
+            if busy:
+                for _ in range(20):
+                    big @ big
+            _, g = L.ac_net_loss_grads(h, d_phi.data_ptr(), d_tgt.data_ptr(), 4, 150, 70, 1, 0.1, want_grads=True)
+            grads.append(g.astype(np.float64))
+        finally:
+            L.ac_net_destroy(h)
+    assert _rel(grads[1], grads[0]) <= 1e-5  # (FP32 sums in another order)
